@@ -649,28 +649,6 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
     }
 }
 
-// (ak, ai) < (bk, bi) as an all-ones mask: the borrow out of the 96-bit
-// difference ak:ai - bk:bi (the index is the low word), one carry chain
-// instead of separate compares of the key halves and the index.
-__device__ __forceinline__ uint32_t ki_less_mask(uint64_t ak, uint32_t ai, uint64_t bk, uint32_t bi) {
-    uint32_t m;
-    asm("{\n\t.reg .u32 t;\n\t"
-        "sub.cc.u32 t, %1, %2;\n\t"
-        "subc.cc.u32 t, %3, %4;\n\t"
-        "subc.cc.u32 t, %5, %6;\n\t"
-        "subc.u32 %0, 0, 0;\n\t}"
-        : "=r"(m)
-        : "r"(ai), "r"(bi), "r"((uint32_t)ak), "r"((uint32_t)bk), "r"((uint32_t)(ak >> 32)),
-          "r"((uint32_t)(bk >> 32)));
-    return m;
-}
-
-// Sorts a thread's MS_IT entries in registers by (K, i): Batcher's odd-even
-// merge sorting network for 16 inputs with every comparator that touches
-// slots 13..15 dropped (those slots would hold +infinity, which a comparator
-// never moves to a lower slot), 48 compare-exchanges instead of the 78 of
-// odd-even transposition (checked on every 0/1 input, which suffices for a
-// network).
 // The rows of a thread that lie in groups of two or more (bit j of mm: its
 // row j, at chunk-relative position first + j): each gets its group's start
 // as its rank (its rotation read from the compacted SA in sI), and each
@@ -703,7 +681,13 @@ __device__ __noinline__ void name_chunk_members(WarpEmitter& em, const Bins& bin
     }
 }
 
-__device__ __forceinline__ void sort13(uint64_t (&k)[MS_IT], uint32_t (&v)[MS_IT]) {
+// Sorts a thread's MS_IT entries in registers in ascending order: Batcher's
+// odd-even merge sorting network for 16 inputs with every comparator that touches
+// slots 13..15 dropped (those slots would hold +infinity, which a comparator
+// never moves to a lower slot), 48 compare-exchanges instead of the 78 of
+// odd-even transposition (checked on every 0/1 input, which suffices for a
+// network).
+__device__ __forceinline__ void sort13(uint64_t (&w)[MS_IT]) {
     static_assert(MS_IT == 13, "the network below sorts 13 entries");
     constexpr int NET[48][2] = {
         {0, 1}, {2, 3}, {0, 2}, {1, 3}, {1, 2}, {4, 5}, {6, 7}, {4, 6}, {5, 7}, {5, 6}, {0, 4}, {2, 6}, {2, 4},
@@ -713,13 +697,10 @@ __device__ __forceinline__ void sort13(uint64_t (&k)[MS_IT], uint32_t (&v)[MS_IT
 #pragma unroll
     for (int c = 0; c < 48; ++c) {
         const int i = NET[c][0], j = NET[c][1];
-        const bool sw = ki_less_mask(k[j], v[j], k[i], v[i]) != 0u;
-        const uint64_t a = sw ? k[j] : k[i], b = sw ? k[i] : k[j];
-        const uint32_t x = sw ? v[j] : v[i], y = sw ? v[i] : v[j];
-        k[i] = a;
-        k[j] = b;
-        v[i] = x;
-        v[j] = y;
+        const bool sw = w[j] < w[i];
+        const uint64_t lo = sw ? w[j] : w[i], hi = sw ? w[i] : w[j];
+        w[i] = lo;
+        w[j] = hi;
     }
 }
 
@@ -727,37 +708,114 @@ __device__ __forceinline__ void sort13(uint64_t (&k)[MS_IT], uint32_t (&v)[MS_IT
 // every rotation = block-local start of its group; groups of size > 1 go to
 // `bins` for the doubling rounds). NT threads sort chunks of up to
 // NT * MS_IT rotations taken from chunks.list[LIST] (256 threads: the packed
-// chunks; 1,024 threads: the single over-full buckets up to BIG_CAP).
+// chunks; 512 and 1,024 threads: the single over-full buckets up to MID_CAP
+// and BIG_CAP).
+//
+// The kernel is bound by the shared-memory pipe and, next, by issue, so what
+// is sorted is one 64-bit word a rotation: the offset of its key from the
+// chunk's first possible key (a chunk is a key range), above the SB-bit slot
+// its index sits in. 64 - SB bits (52 for a packed chunk) hold the offset
+// whole in most chunks; where the range is wider its low bits are dropped.
+// Rows whose offsets differ are in place after this sort. If any are equal
+// -- about 4 in 100 chunks of text -- the chunk is sorted once more by
+// (run of equal offsets, dropped bits, rotation), which is exact.
+// Measured per 240 blocks of 900,000 bytes (nine text-like, one uniform):
+// 3,412 us with (key, index) pairs of 12 bytes moved through every round,
+// 2,657 us with words, 2,611 us with one key offset a chunk instead of one a
+// bucket. On 24 blocks (ncu): 11.8 -> 9.0 warp instructions a rotation, 81% of
+// the shared-memory pipe, issue 58%, 15.1 DRAM bytes a rotation. Measured
+// and not kept: five CTAs an SM at 48 registers (2,734), the second run of a
+// merge stored backwards so that no bounds are tested (2,839), one load a
+// merge step from a selected address (2,691), the first merge round by
+// shuffles between neighbouring threads (2,673: fewer wavefronts, more
+// instructions).
 //
 // A chunk is a run of whole fine buckets, and a fine bucket is a key range,
 // so the chunk is sorted bucket by bucket: no merge crosses a bucket edge.
 //   1. The bucket table: every bucket's chunk-relative start (from the
 //      block's scanned counts) and its team of ceil(size / MS_IT) threads
 //      (an exclusive scan by one warp), whose run of team * MS_IT slots holds
-//      the bucket, padded with entries above every real one.
+//      the bucket, padded with words above every real one.
 //   2. Every rotation's bucket in the chunk, read off the tag its value
-//      carries from the scatter, and a counting scatter into its bucket's
-//      run (a shared-memory atomic a rotation).
-//   3. Each thread sorts its MS_IT slots with the network; then merge
+//      carries from the scatter, and a counting scatter of its word into its
+//      bucket's run (a shared-memory atomic a rotation); the rotation itself
+//      stays in sI, at the slot the word names.
+//   3. Each thread sorts its MS_IT words with the network; then merge
 //      rounds inside each team (merge path; a team takes part in as many
 //      rounds as it needs, ceil(log2(threads)): about 5 for learned buckets
 //      of ~220 rotations, against 8 for the whole chunk at once).
-//   4. SA is written compacted (the buckets in order, padding dropped),
-//      and the chunk is named from the registers the last round left: the
-//      ranks of group members are stored and their groups sent to the
-//      doubling rounds; groups of one are marked SA_FINAL and their ranks
-//      left to the on-demand lookup (LazyRanks), since nearly all rotations
-//      of text blocks are told apart by their first 8 bytes. members[block]
-//      counts the rotations sent on, which decides whether a block's ranks
-//      are filled in full after the chunk sorts (k_fill_ranks).
-// Padding entries are (~0, 0xffff0000 + slot): above every real pair (real
-// indices are below 2^30) and distinct. A merge step reloads the head it
-// consumed without a bounds test, so a head may sit one entry past its run
-// (the other run, the next team's slots, or the 16 bytes of slack after the
-// arrays); the choice tests the bounds and never takes such a head.
-constexpr size_t CHUNK_SORT_SMEM = (size_t)CHUNK_CAP * 12 + 16;
-constexpr size_t BIG_SORT_SMEM = (size_t)BIG_CAP * 12 + 16;
-constexpr size_t MID_SORT_SMEM = (size_t)MID_CAP * 12 + 16;
+//   4. SA is written compacted (the buckets in order, padding dropped). With
+//      every offset its own, all rows are groups of one, marked SA_FINAL;
+//      their ranks are left to the on-demand lookup (LazyRanks), since nearly
+//      all rotations of text blocks are told apart by their first 8 bytes.
+//   5. After a second sort the chunk is named from the registers: the ranks
+//      of group members are stored and their groups sent to the doubling
+//      rounds. members[block] counts the rotations sent on, which decides
+//      whether a block's ranks are filled in full after the chunk sorts
+//      (k_fill_ranks).
+// Padding words are ~0: a real word's slot (first sort) and run start (second
+// sort) are below the all-ones value of their bits. A merge step reloads the
+// head it consumed without a bounds test, so a head may sit one word past its
+// run (the other run, the next team's slots, or the array after sW); the
+// choice tests the bounds and never takes such a head.
+constexpr size_t CHUNK_SORT_SMEM = (size_t)CHUNK_CAP * 12;
+constexpr size_t BIG_SORT_SMEM = (size_t)BIG_CAP * 12;
+constexpr size_t MID_SORT_SMEM = (size_t)MID_CAP * 12;
+
+// Sorts the MS_IT slots of every team: the network in registers, then R
+// merge-path rounds through sW. A team of kteam threads
+// starting at thread tfirst (this thread is its lt-th) holds kteam * MS_IT
+// slots; it sits out the rounds it does not need. `active` is false for
+// threads without a team and for teams that have nothing to sort. All threads
+// of the CTA call; the result is in w and sW may be overwritten on return.
+__device__ __forceinline__ void team_sort(uint64_t (&w)[MS_IT], uint64_t* sW, uint32_t tfirst, uint32_t lt,
+                                          uint32_t kteam, uint32_t R, bool active) {
+    const uint32_t tid = threadIdx.x;
+    if (active) sort13(w);
+    for (uint32_t r = 1; r <= R; ++r) {
+        // a team whose runs already form one sorted run sits the round out
+        const bool merging = active && (1u << (r - 1)) < kteam;
+        if (merging) {  // the sorted runs of the previous step back in place
+#pragma unroll
+            for (int j = 0; j < MS_IT; ++j) sW[tid * MS_IT + j] = w[j];
+        }
+        __syncthreads();
+        if (merging) {
+            const uint32_t m = 1u << r;  // threads per merged run
+            const uint32_t pf = lt & ~(m - 1u);
+            const uint32_t half = (m >> 1) * MS_IT;  // input run length
+            const uint32_t L = kteam * MS_IT;
+            const uint32_t a0 = pf * MS_IT, a1 = min(a0 + half, L), b1 = min(a0 + 2u * half, L);
+            const uint32_t la = a1 - a0, lb = b1 - a1;
+            const uint32_t diag = (lt - pf) * MS_IT;
+            const uint64_t* A = sW + tfirst * MS_IT + a0;
+            const uint64_t* B = A + la;
+            uint32_t lo = diag > lb ? diag - lb : 0u, hi = min(diag, la);
+            while (lo < hi) {  // A entries among the first diag outputs (A first on ties)
+                const uint32_t mid = (lo + hi) >> 1;
+                if (A[mid] <= B[diag - 1 - mid]) lo = mid + 1; else hi = mid;
+            }
+            // heads may sit one past their run (valid shared memory: the
+            // other run, the next team, or the array after sW); the bounds in
+            // the choice keep them out
+            uint32_t ia = lo, ib = diag - lo;
+            uint64_t ka = A[ia], kb = B[ib];
+#pragma unroll
+            for (int j = 0; j < MS_IT; ++j) {
+                const bool take_b = ib < lb && (ia >= la || kb < ka);
+                w[j] = take_b ? kb : ka;
+                if (take_b) {
+                    ++ib;
+                    kb = B[ib];
+                } else {
+                    ++ia;
+                    ka = A[ia];
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
 
 template <int NT, int MINB, int LIST>
 __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __restrict__ K,
@@ -766,22 +824,29 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
                                                               uint32_t* __restrict__ rank, Bins bins, uint32_t* ctrl,
                                                               uint32_t* __restrict__ chunk_counter,
                                                               const uint32_t* __restrict__ starts,
+                                                              const uint32_t* __restrict__ route,
+                                                              const uint64_t* __restrict__ splitters,
                                                               uint32_t* __restrict__ members) {
     constexpr uint32_t CAP = NT * MS_IT;
+    constexpr int SB = NT == 256 ? 12 : NT == 512 ? 13 : 14;  // slot bits of a word
+    static_assert(CAP < (1u << SB), "a real word's slot is below the padding's");
+    constexpr uint32_t SLOT_MASK = (1u << SB) - 1u;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* sK = reinterpret_cast<uint64_t*>(smem);
-    uint32_t* sI = reinterpret_cast<uint32_t*>(smem + (size_t)CAP * 8);
+    uint64_t* sW = reinterpret_cast<uint64_t*>(smem);                      // [CAP] words
+    uint32_t* sI = reinterpret_cast<uint32_t*>(smem + (size_t)CAP * 8);    // [CAP] rotation of every slot
+    uint32_t* sO = reinterpret_cast<uint32_t*>(smem);                      // [CAP] the chunk's SA (over sW, once sorted)
+    // the emitter's buffers, behind sO (over sW too): used by chunks with members only
+    GroupDesc* ebuf = reinterpret_cast<GroupDesc*>(smem + (size_t)CAP * 4);
+    static_assert((size_t)(NT / 32) * NCLS * EMIT_BUF * sizeof(GroupDesc) <= (size_t)CAP * 4, "emitter buffers fit");
     __shared__ uint32_t bstart[MAXB + 1];  // chunk-relative start of every bucket (and the chunk's end)
-    __shared__ uint32_t bthr[MAXB + 1];    // first thread of every bucket's team (and the threads used)
+    __shared__ uint16_t bthr[MAXB + 1];    // first thread of every bucket's team (and the threads used)
     __shared__ uint32_t bcur[MAXB];        // scatter cursors
-    __shared__ GroupDesc ebuf[NT / 32][NCLS * EMIT_BUF];
-    __shared__ uint64_t s_wlast[NT / 32], s_wfirst[NT / 32];  // each warp's last and first key
-    __shared__ uint32_t s_wmax[NT / 32];                      // each warp's last head + 1
+    __shared__ uint64_t s_wlast[NT / 32];  // each warp's last word
+    __shared__ uint32_t s_wmax[NT / 32];   // each warp's last head + 1
+    __shared__ uint64_t s_wfirst[NT / 32];
     __shared__ uint32_t s_c, s_rounds;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (ld_volatile(&ctrl[CTRL_ERR])) return;  // an earlier stage failed: the chunks are not permutations
-    WarpEmitter em;
-    em.init(ebuf[warp]);
     const uint32_t count = bin_count(chunks, LIST);
     // chunks in list order from an atomic counter (zeroed before the launch):
     // the chunks in flight stay within a few blocks, whose rank ranges stay
@@ -805,6 +870,18 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
             const uint32_t st = j == nbk ? cstart + len : srow[min(b0 + j, (uint32_t)NBK - 1u)];
             bstart[j] = min(st - cstart, len);
         }
+        // the chunk's keys are [kfirst, klast]: a word holds the offset from
+        // kfirst, its low `sh` bits dropped if it needs more than 64 - SB bits
+        uint64_t kfirst, klast;
+        const uint32_t b1 = min(b0 + nbk, (uint32_t)NBK);  // one past the last bucket
+        if (route[gd.blk] == 2u) {
+            kfirst = (uint64_t)b0 << 52;
+            klast = ((uint64_t)b1 << 52) - 1ull;  // b1 = 4096: 2^64 - 1
+        } else {
+            kfirst = b0 > 0 ? splitters[b0 - 1] : 0ull;
+            klast = b1 < (uint32_t)NBK ? splitters[b1 - 1] - 1ull : ~0ull;
+        }
+        const uint32_t sh = (uint32_t)max(SB - __clzll((long long)(klast - kfirst)), 0);
         __syncthreads();
         if (warp == 0) {
             uint32_t run = 0, mx = 0;
@@ -819,8 +896,8 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
                     if ((int)lane >= o) incl += y;
                 }
                 if (j < nbk) {
-                    bthr[j] = run + incl - t;
-                    bcur[j] = 0u;
+                    bthr[j] = (uint16_t)min(run + incl - t, (uint32_t)NT);
+                    bcur[j] = (run + incl - t) * MS_IT;
                 }
                 mx = max(mx, t);
                 run += __shfl_sync(0xffffffffu, incl, 31);
@@ -828,7 +905,7 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             if (lane == 0) {
-                bthr[nbk] = min(run, (uint32_t)NT);
+                bthr[nbk] = (uint16_t)min(run, (uint32_t)NT);
                 s_rounds = mx <= 1u ? 0u : 32u - __clz(mx - 1u);  // ceil(log2(largest team))
                 BWT_DCHECK(run <= (uint32_t)NT, &ctrl[CTRL_ERR]);
             }
@@ -849,156 +926,76 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
         const uint32_t lt = tid - tfirst;             // index inside the team
         const uint32_t kteam = bthr[team + 1] - tfirst;  // threads of the team
         const bool active = tid < T;
-        // ---- 2. loads (all in flight together), buckets, counting scatter
-        uint64_t k[MS_IT];
-        uint32_t v[MS_IT];
-#pragma unroll
-        for (int j = 0; j < MS_IT; ++j) {
-            const uint32_t i = j * NT + tid;
-            k[j] = i < len ? K[gd.start + i] : 0ull;
-            v[j] = i < len ? SA[gd.start + i] : 0u;
-        }
-        if (active && lt + 1 == kteam) {  // the padding: only a team's last thread has any
+        // ---- 2. loads (all in flight together), words, counting scatter
+        uint64_t w[MS_IT];
+        {
+            uint32_t v[MS_IT];
 #pragma unroll
             for (int j = 0; j < MS_IT; ++j) {
-                const uint32_t pos = lt * MS_IT + j;  // position inside the team's run
-                if (pos >= tsize) {
-                    const uint32_t slot = tid * MS_IT + j;
-                    sK[slot] = ~0ull;
-                    sI[slot] = 0xffff0000u + slot;
+                const uint32_t i = j * NT + tid;
+                w[j] = i < len ? K[gd.start + i] : 0ull;
+                v[j] = i < len ? SA[gd.start + i] : 0u;
+            }
+            if (active && lt + 1 == kteam) {  // the padding: only a team's last thread has any
+#pragma unroll
+                for (int j = 0; j < MS_IT; ++j)
+                    if (lt * MS_IT + j >= tsize) sW[tid * MS_IT + j] = ~0ull;
+            }
+#pragma unroll
+            for (int j = 0; j < MS_IT; ++j) {
+                const uint32_t i = j * NT + tid;
+                if (i < len) {
+                    // packed chunks: the bucket tag; a bucket of its own: untagged
+                    uint32_t lb = LIST == 0 ? ((v[j] >> TAG_SHIFT) - b0) & 0xffu : 0u;
+                    const uint32_t sa = v[j] & IDX_MASK;
+                    BWT_DCHECK(lb < nbk && sa < bi.n, &ctrl[CTRL_ERR]);
+                    lb = min(lb, nbk - 1);
+                    sI[i] = sa;
+                    // any order inside the run: the sort decides it
+                    const uint32_t slot = min(atomicAdd(&bcur[lb], 1u), CAP - 1u);
+                    sW[slot] = ((w[j] - kfirst) >> sh << SB) | i;
                 }
             }
         }
-#pragma unroll
-        for (int j = 0; j < MS_IT; ++j) {
-            const uint32_t i = j * NT + tid;
-            const bool valid = i < len;
-            uint32_t lb = 0xffffffffu;
-            if (valid) {
-                // packed chunks: the bucket tag; a bucket of its own: untagged
-                lb = LIST == 0 ? ((v[j] >> TAG_SHIFT) - b0) & 0xffu : 0u;
-                v[j] &= IDX_MASK;
-                BWT_DCHECK(lb < nbk && v[j] < bi.n, &ctrl[CTRL_ERR]);
-                lb = min(lb, nbk - 1);
-            }
-            if (valid) {  // any order inside the run: the sort decides it
-                const uint32_t slot = min(bthr[lb] * MS_IT + atomicAdd(&bcur[lb], 1u), CAP - 1u);
-                sK[slot] = k[j];
-                sI[slot] = v[j];
-            }
-        }
         __syncthreads();
-        // ---- 3. sorting network on this thread's slots, then merge rounds inside the team
+        // ---- 3. sort by (key offset, slot)
+#pragma unroll
+        for (int j = 0; j < MS_IT; ++j) w[j] = active ? sW[tid * MS_IT + j] : 0ull;
         const uint32_t R = s_rounds;
-        if (active) {
+        team_sort(w, sW, tfirst, lt, kteam, R, active);
+        // rows with the same key offset as the row before (bit j)
+        const uint32_t nreal = active ? min((uint32_t)MS_IT, tsize - min(tsize, lt * MS_IT)) : 0u;
+        const uint32_t base = bstart[team];           // the team's bucket, chunk-relative
+        const uint32_t first = base + lt * MS_IT;     // the thread's first row, chunk-relative
+        uint32_t eq = 0;
+        {
+            uint64_t prev = __shfl_up_sync(0xffffffffu, w[MS_IT - 1], 1);
+            if (lane == 31) s_wlast[warp] = w[MS_IT - 1];
+            __syncthreads();  // also: every thread has read its slots before sO or sW is written
+            if (lane == 0 && warp > 0) prev = s_wlast[warp - 1];
 #pragma unroll
             for (int j = 0; j < MS_IT; ++j) {
-                k[j] = sK[tid * MS_IT + j];
-                v[j] = sI[tid * MS_IT + j];
+                if ((uint32_t)j < nreal && lt * MS_IT + j > 0 && (w[j] >> SB) == (prev >> SB)) eq |= 1u << j;
+                prev = w[j];
             }
-            sort13(k, v);
         }
-        for (uint32_t r = 1; r <= R; ++r) {
-            // a team whose runs already form one sorted run sits the round out
-            const bool merging = active && (1u << (r - 1)) < kteam;
-            if (merging) {  // the sorted runs of the previous step back in place
+        if (!__syncthreads_or(eq != 0u)) {
+            // ---- 4a. every key of the chunk is its own (nearly every chunk of text): all rows are final
 #pragma unroll
-                for (int j = 0; j < MS_IT; ++j) {
-                    sK[tid * MS_IT + j] = k[j];
-                    sI[tid * MS_IT + j] = v[j];
-                }
-            }
+            for (int j = 0; j < MS_IT; ++j)
+                if ((uint32_t)j < nreal) sO[first + j] = sI[(uint32_t)w[j] & SLOT_MASK] | SA_FINAL;
             __syncthreads();
-            if (merging) {
-                const uint32_t m = 1u << r;  // threads per merged run
-                const uint32_t pf = lt & ~(m - 1u);
-                const uint32_t w = (m >> 1) * MS_IT;  // input run length
-                const uint32_t L = kteam * MS_IT;
-                const uint32_t a0 = pf * MS_IT, a1 = min(a0 + w, L), b1 = min(a0 + 2u * w, L);
-                const uint32_t la = a1 - a0, lb = b1 - a1;
-                const uint32_t diag = (lt - pf) * MS_IT;
-                const uint64_t* AK = sK + tfirst * MS_IT + a0;
-                const uint32_t* AI = sI + tfirst * MS_IT + a0;
-                const uint64_t* BK = AK + la;
-                const uint32_t* BI = AI + la;
-                uint32_t lo = diag > lb ? diag - lb : 0u, hi = min(diag, la);
-                while (lo < hi) {  // A entries among the first diag outputs (A first on ties)
-                    const uint32_t mid = (lo + hi) >> 1;
-                    const uint64_t a = AK[mid], b = BK[diag - 1 - mid];
-                    const bool a_first = a != b ? a < b : AI[mid] <= BI[diag - 1 - mid];
-                    if (a_first) lo = mid + 1; else hi = mid;
-                }
-                // heads may sit one past their run (valid shared memory: the
-                // other run, the next team, or the slack entry after the
-                // arrays); the bounds in the choice keep them out
-                uint32_t ia = lo, ib = diag - lo;
-                uint64_t ka = AK[ia], kb = BK[ib];
-                uint32_t va = AI[ia], vb = BI[ib];
-#pragma unroll
-                for (int j = 0; j < MS_IT; ++j) {
-                    const bool take_b = ib < lb && (ia >= la || ki_less_mask(kb, vb, ka, va) != 0u);
-                    k[j] = take_b ? kb : ka;
-                    v[j] = take_b ? vb : va;
-                    if (take_b) {
-                        ++ib;
-                        kb = BK[ib];
-                        vb = BI[ib];
-                    } else {
-                        ++ia;
-                        ka = AK[ia];
-                        va = AI[ia];
-                    }
-                }
-            }
+            for (uint32_t i = tid; i < len; i += NT) SA[gd.start + i] = sO[i];
             __syncthreads();
+            continue;
         }
-        if (R == 0) __syncthreads();  // every thread has read its slots before any compacted write
-        // ---- 4. naming, from the registers. A rotation heads a group where
-        //      its key differs from the one before it (a bucket's first
-        //      rotation always does: a bucket is a key range); it ends one
-        //      where the next key differs or its bucket ends. Its group start
-        //      is the last head at or before it: inside the thread by a
-        //      running value, across threads by a CTA max-scan of every
-        //      thread's last head.
-        const uint32_t base = bstart[team];  // the team's bucket, chunk-relative
-        uint64_t prev_last = __shfl_up_sync(0xffffffffu, k[MS_IT - 1], 1);
-        uint64_t next_first = __shfl_down_sync(0xffffffffu, k[0], 1);
-        if (lane == 31) s_wlast[warp] = k[MS_IT - 1];
-        if (lane == 0) s_wfirst[warp] = k[0];
-        __syncthreads();
-        if (lane == 0 && warp > 0) prev_last = s_wlast[warp - 1];
-        if (lane == 31 && warp + 1 < NT / 32) next_first = s_wfirst[warp + 1];
-        const bool emit_ok = bi.n > 8u;   // smaller blocks: every group is final (whole equal rotations)
-        uint32_t hm = 0, fm = 0, mm = 0, lh = 0;  // head, not-last and member bits, last head + 1 (0: none)
-        if (active) {
-#pragma unroll
-            for (int j = 0; j < MS_IT; ++j) {
-                const uint32_t pos = lt * MS_IT + j;
-                if (pos < tsize) {
-                    const uint64_t before = j == 0 ? prev_last : k[j > 0 ? j - 1 : 0];
-                    const uint64_t after = j == MS_IT - 1 ? next_first : k[j < MS_IT - 1 ? j + 1 : 0];
-                    const bool head = pos == 0 || k[j] != before;
-                    const bool tail = pos + 1 == tsize || k[j] != after;
-                    if (head) {
-                        hm |= 1u << j;
-                        lh = base + pos + 1;
-                    }
-                    if (!tail) fm |= 2u << j;  // bit j + 1: not the group's last row
-                    const bool final_row = (head && tail) || !emit_ok;
-                    if (!final_row) mm |= 1u << j;  // in a group of two or more, sent to the rounds
-                    // SA, compacted through shared memory (bucket after bucket,
-                    // padding dropped) for a coalesced write
-                    sI[base + pos] = v[j] | (final_row ? SA_FINAL : 0u);
-                }
-            }
-        }
-        // the barrier also tells whether the chunk holds a group of two or more
-        const bool any_member = __syncthreads_or(mm != 0u) != 0;
-        for (uint32_t i = tid; i < len; i += NT) SA[gd.start + i] = sI[i];
-        if (any_member) {  // CTA-uniform; rare on text
-            // group starts: the last head at or before each row, by a CTA
-            // max-scan of every thread's last head
-            uint32_t incl = lh;
+        // ---- 4b. rows that share a key offset: sorted again by (run, dropped
+        //      key bits, rotation), where a run is a stretch of equal offsets,
+        //      named by its first row: the last head at or before each row, by
+        //      a running value inside the thread and a CTA max-scan of every
+        //      thread's last head
+        auto heads_before = [&](uint32_t hm) {  // last head + 1 before the thread's first row (0: none)
+            uint32_t incl = hm ? first + 32u - __clz(hm) : 0u;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -1008,18 +1005,75 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
             __syncthreads();
             uint32_t cur = __shfl_up_sync(0xffffffffu, incl, 1);
             if (lane == 0) cur = 0u;
-            for (uint32_t w = 0; w < warp; ++w) cur = max(cur, s_wmax[w]);
+            for (uint32_t x = 0; x < warp; ++x) cur = max(cur, s_wmax[x]);
+            __syncthreads();
+            return cur;
+        };
+        const uint32_t real = (1u << nreal) - 1u;
+        {
+            uint32_t cur = heads_before(real & ~eq);
+#pragma unroll
+            for (int j = 0; j < MS_IT; ++j) {
+                if ((uint32_t)j < nreal) {
+                    const uint32_t slot = (uint32_t)w[j] & SLOT_MASK;
+                    if (!((eq >> j) & 1u)) cur = first + j + 1;
+                    const uint64_t low = sh ? (K[gd.start + min(slot, len - 1u)] - kfirst) & ((1ull << sh) - 1ull) : 0ull;
+                    w[j] = ((uint64_t)(cur - 1u) << 50) | (low << TAG_SHIFT) | sI[min(slot, CAP - 1u)];
+                } else {
+                    w[j] = ~0ull;
+                }
+            }
+        }
+        team_sort(w, sW, tfirst, lt, kteam, R, active);
+        // ---- 5. naming, from the registers. A rotation heads a group where
+        //      its key differs from the one before it; it ends one where the
+        //      next key differs or its bucket ends (a bucket is a key range).
+        const bool emit_ok = bi.n > 8u;   // smaller blocks: every group is final (whole equal rotations)
+        uint32_t hm = 0, fm = 0, mm = 0;  // head, not-last and member bits
+        {
+            uint64_t prev = __shfl_up_sync(0xffffffffu, w[MS_IT - 1], 1);
+            uint64_t next = __shfl_down_sync(0xffffffffu, w[0], 1);
+            if (lane == 31) s_wlast[warp] = w[MS_IT - 1];
+            if (lane == 0) s_wfirst[warp] = w[0];
+            __syncthreads();
+            if (lane == 0 && warp > 0) prev = s_wlast[warp - 1];
+            if (lane == 31 && warp + 1 < NT / 32) next = s_wfirst[warp + 1];
+#pragma unroll
+            for (int j = 0; j < MS_IT; ++j) {
+                const uint32_t pos = lt * MS_IT + j;
+                if ((uint32_t)j < nreal) {
+                    const uint64_t after = j == MS_IT - 1 ? next : w[j < MS_IT - 1 ? j + 1 : 0];
+                    const bool head = pos == 0 || (w[j] >> TAG_SHIFT) != (prev >> TAG_SHIFT);
+                    const bool tail = pos + 1 == tsize || (w[j] >> TAG_SHIFT) != (after >> TAG_SHIFT);
+                    if (head) hm |= 1u << j;
+                    if (!tail) fm |= 2u << j;  // bit j + 1: not the group's last row
+                    const bool final_row = (head && tail) || !emit_ok;
+                    if (!final_row) mm |= 1u << j;  // in a group of two or more, sent to the rounds
+                    // SA, compacted through shared memory (bucket after bucket,
+                    // padding dropped) for a coalesced write
+                    sO[first + j] = ((uint32_t)w[j] & IDX_MASK) | (final_row ? SA_FINAL : 0u);
+                }
+                prev = w[j];
+            }
+        }
+        // the barrier also tells whether the chunk holds a group of two or more
+        const bool any_member = __syncthreads_or(mm != 0u) != 0;
+        for (uint32_t i = tid; i < len; i += NT) SA[gd.start + i] = sO[i];
+        if (any_member) {  // CTA-uniform; rare on text
+            const uint32_t cur = heads_before(hm);
+            WarpEmitter em;
+            em.init(ebuf + warp * NCLS * EMIT_BUF);
             // groups of two or more: their ranks stored and the groups sent
             // to the doubling rounds, by a call taken only by warps that
             // hold a member
-            if (__any_sync(0xffffffffu, mm != 0u))
-                name_chunk_members<MS_IT>(em, bins, mm, hm, fm, cur, base + lt * MS_IT,
-                                          active ? tsize - min(tsize, lt * MS_IT) : 0u, sI, rank, bi,
-                                          gd.start - bi.off, gd.start, gd.blk, members, &ctrl[CTRL_ERR]);
+            if (__any_sync(0xffffffffu, mm != 0u)) {
+                name_chunk_members<MS_IT>(em, bins, mm, hm, fm, cur, first, nreal, sO, rank, bi, gd.start - bi.off,
+                                          gd.start, gd.blk, members, &ctrl[CTRL_ERR]);
+                em.finish(bins, &ctrl[CTRL_ERR]);
+            }
         }
         __syncthreads();
     }
-    em.finish(bins, &ctrl[CTRL_ERR]);
 }
 
 // After the chunk sorts: a bucketed block whose chunk sorts sent more than
@@ -1376,8 +1430,8 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     const bool timing = !p->events.empty() && !p->capturing && p->ev_used + 2 <= p->events.size();
     if (timing) CKL(cudaEventRecord(p->events[p->ev_used], st));
     k_chunk_sort_name<MS_NT, 4, 0><<<sms * p->chunk_sort_ctas, MS_NT, CHUNK_SORT_SMEM, st>>>(
-        p->keys[0], p->vals[0], p->blocks, aux, p->rank, bins_of(p, 0), ctrl, chunk_counter, p->bucket_count,
-        p->members);
+        p->keys[0], p->vals[0], p->blocks, aux, p->rank, bins_of(p, 0), ctrl, chunk_counter, p->bucket_count, p->route,
+        p->splitters, p->members);
     CKL(cudaGetLastError());
     if (timing) {
         CKL(cudaEventRecord(p->events[p->ev_used + 1], st));
@@ -1391,10 +1445,10 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     // and 1,024 up to BIG_CAP
     k_chunk_sort_name<MID_NT, 2, 2><<<2 * sms, MID_NT, MID_SORT_SMEM, st>>>(p->keys[0], p->vals[0], p->blocks, aux,
                                                                             p->rank, bins_of(p, 0), ctrl, mid_counter,
-                                                                            p->bucket_count, p->members);
+                                                                            p->bucket_count, p->route, p->splitters, p->members);
     k_chunk_sort_name<BIG_NT, 1, 1><<<sms, BIG_NT, BIG_SORT_SMEM, st>>>(p->keys[0], p->vals[0], p->blocks, aux,
                                                                         p->rank, bins_of(p, 0), ctrl, big_counter,
-                                                                        p->bucket_count, p->members);
+                                                                        p->bucket_count, p->route, p->splitters, p->members);
     CKL(cudaGetLastError());
     p->stats.kernel_launches += 4;
 

@@ -1,0 +1,50 @@
+"""Edges of single kernels against the oracle, byte for byte."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1109_2348_gb300 import F_GRAPH, F_LEARNED, Plan, datagen, model
+from tests.gpu_util import assert_matches_oracle, batch_from_blocks, gpu_bwt
+
+pytestmark = pytest.mark.gpu
+
+
+def _rng_bytes(seed, n, lo, hi):
+    return np.random.RandomState(seed).randint(lo, hi, n).astype(np.uint8)
+
+
+def _chunk_sort_blocks(kind):
+    if kind == "wide":  # few rotations a chunk: key ranges of up to 64 bits, whose low bits the words drop
+        return [_rng_bytes(1, n, 0, 256) for n in (9, 13, 14, 100, 3328, 3329, 5000)]
+    if kind == "last_byte":  # prefixes of 7 equal bytes, told apart by the eighth alone, and far beyond it
+        unit = _rng_bytes(2, 7, 0, 256)
+        rows = [np.concatenate([unit, _rng_bytes(10 + k, 1 + k % 3, 0, 256)]) for k in range(1500)]
+        return [np.concatenate(rows), np.concatenate(rows[:300] + [_rng_bytes(3, 40_000, 0, 256)])]
+    if kind == "repeats":  # groups of equal prefixes of every small size beside distinct ones
+        text = datagen.block(datagen.MARKOV3_Z96, 77, 30_000)
+        return [np.concatenate([text, text[100:9000], text[200:2000], text[:5000]]), np.tile(text[:700], 20)]
+    return [np.concatenate([_rng_bytes(5, 60_000, 0, 256), np.tile(_rng_bytes(6, 24, 0, 4), 150)]),
+            datagen.block(datagen.MUTATED_UNIT, 9, 120_000)]
+
+
+@pytest.mark.parametrize("kind", ["wide", "last_byte", "repeats", "mixed"])
+@pytest.mark.parametrize("table", ["equal", "coarse", "top"])
+def test_chunk_sort_words(kind, table):
+    """The chunk sort's 64-bit words: dropped key bits, ties and runs of equal
+    prefixes, under an equal-width table (52-bit ranges), a coarse one (a few
+    wide buckets, so that all three team sizes occur) and one whose splitters
+    crowd at both ends of the key space."""
+    spl = model.equal_width_splitters()
+    if table == "coarse":
+        spl = np.sort(np.repeat(spl[::256], 256)[:spl.size])
+    elif table == "top":
+        half = np.arange(spl.size // 2, dtype=np.uint64)
+        spl = np.sort(np.concatenate([half, ~np.uint64(0) - np.arange(spl.size - half.size, dtype=np.uint64)]))
+    buf, off = batch_from_blocks(_chunk_sort_blocks(kind))
+    sizes = np.diff(off.astype(np.int64))
+    with Plan(max_blocks=off.size - 1, max_total_bytes=buf.size, max_block_bytes=int(sizes.max()),
+              flags=F_LEARNED | F_GRAPH) as plan:
+        model.install(plan, spl)
+        L, prim, _ = gpu_bwt(buf, off, plan)
+    assert_matches_oracle(buf, off, L, prim, f"{kind}/{table}")
