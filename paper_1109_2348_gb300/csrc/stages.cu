@@ -15,15 +15,11 @@
 // bit, and the codewords are written there (most significant bit first;
 // each block's stream starts at a byte boundary).
 //
-// Move-to-front encoding (Section 3.3): the paper's parallelism is over
-// the list -- its 256 entries are spread over a warp's lanes, 8 a lane (kept
-// as every value's position, so a byte's position is one shuffle away and
-// the move is one byte-wise compare-and-add per lane). A block's bytes form one chain of list states, so blocks are cut
-// into chunks: a chunk's effect on the list is the chunk's distinct bytes
-// in order of last occurrence, followed by the old list without them. Pass
-// 1 finds that list for every chunk, pass 2 chains the chunks of every
-// block to get each chunk's starting list, pass 3 encodes all chunks at
-// once.
+// Move-to-front encoding (Section 3.3): the paper searches the list in
+// parallel for one byte after another. Here blocks are cut into chunks whose
+// starting lists come from the last occurrences of every byte value before
+// them (one pass over the bytes, one over the chunks), and a warp encodes 32
+// bytes of a chunk at once (below).
 //
 // GB300 layout: the prefix sums are single passes over 4,096-element tiles
 // (256 threads x 16) with decoupled look-back between tiles, so each of the
@@ -417,143 +413,266 @@ __global__ void __launch_bounds__(RT) k_vle_pack(const uint8_t* __restrict__ S, 
 }
 
 // ---- move-to-front encoding ---------------------------------------------------
-
-// Pass 1: per chunk (a first-sort tile), its distinct bytes ordered by last
-// occurrence, most recent first: mru[chunk][0 .. mcnt[chunk]).
-__global__ void __launch_bounds__(RT) k_mtf_mru(const uint8_t* __restrict__ S, const TileDesc* __restrict__ tiles,
-                                                uint32_t ntiles, uint8_t* __restrict__ mru,
-                                                uint32_t* __restrict__ mcnt) {
-    __shared__ int32_t last[256];
-    __shared__ uint8_t sb[RTILE];
-    __shared__ uint32_t s_cnt;
-    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const TileDesc td = tiles[t];
-        last[threadIdx.x] = -1;
-        if (threadIdx.x == 0) s_cnt = 0;
-        for (uint32_t q = threadIdx.x; q < td.len; q += RT) sb[q] = S[td.start + q];
-        __syncthreads();
-        const uint32_t q0 = threadIdx.x * RI;
-        for (int j = RI - 1; j >= 0; --j) {  // the last occurrence inside this thread's range only
-            const uint32_t q = q0 + j;
-            if (q >= td.len) continue;
-            const uint8_t x = sb[q];
-            bool later = false;
-            for (int k = j + 1; k < RI && q0 + k < td.len; ++k) later |= sb[q0 + k] == x;
-            if (!later) atomicMax(&last[x], (int32_t)q);
-        }
-        __syncthreads();
-        const int32_t mine = last[threadIdx.x];
-        if (mine >= 0) {
-            uint32_t rank = 0;
-            for (int u = 0; u < 256; ++u) rank += last[u] > mine;
-            mru[(size_t)t * 256 + rank] = (uint8_t)threadIdx.x;
-            atomicAdd(&s_cnt, 1u);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) mcnt[t] = s_cnt;
-        __syncthreads();
-    }
-}
-
-// Pass 2: one warp per block chains its chunks: the list before chunk c
-// goes to tlist[c]; the next list is mru[c] followed by the list without
-// mru[c]'s bytes. A lane holds list entries 8 lane .. 8 lane + 7 (byte k of
-// its 64-bit word is entry 8 lane + k).
-__global__ void __launch_bounds__(256) k_mtf_chain(const uint32_t* __restrict__ tfirst, uint32_t nb,
-                                                   const uint8_t* __restrict__ mru, const uint32_t* __restrict__ mcnt,
-                                                   uint8_t* __restrict__ tlist) {
-    __shared__ uint32_t member[8][8];
-    __shared__ __align__(8) uint8_t nlist[8][256];
-    const uint32_t lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const uint32_t lt = lanemask_lt();
-    for (uint32_t b = blockIdx.x * 8 + wl; b < nb; b += gridDim.x * 8) {
-        uint64_t L = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) L |= (uint64_t)(lane * 8 + k) << (8 * k);
-        for (uint32_t c = tfirst[b]; c < tfirst[b + 1]; ++c) {
-            reinterpret_cast<uint64_t*>(tlist + (size_t)c * 256)[lane] = L;
-            if (lane < 8) member[wl][lane] = 0u;
-            __syncwarp();
-            const uint32_t cnt = mcnt[c];
-            const uint8_t* m = mru + (size_t)c * 256;
-            for (uint32_t i = lane; i < cnt; i += 32) {
-                const uint32_t v = m[i];
-                atomicOr(&member[wl][v >> 5], 1u << (v & 31));
-                nlist[wl][i] = (uint8_t)v;
-            }
-            __syncwarp();
-            uint32_t keep = 0;  // bit k: entry 8 lane + k stays (not among the chunk's bytes)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const uint32_t v = (uint32_t)(L >> (8 * k)) & 0xffu;
-                keep |= (uint32_t)(((member[wl][v >> 5] >> (v & 31)) & 1u) == 0u) << k;
-            }
-            uint32_t n = __popc(keep), x = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= (uint32_t)o) x += y;
-            }
-            uint32_t pos = cnt + x - n;
-            (void)lt;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if ((keep >> k) & 1u) nlist[wl][pos++] = (uint8_t)(L >> (8 * k));
-            __syncwarp();
-            L = reinterpret_cast<const uint64_t*>(nlist[wl])[lane];
-            __syncwarp();
-        }
-    }
-}
-
-// Pass 3: one warp per chunk encodes it from its starting list. The warp
-// keeps every byte value's position in the list instead of the list itself:
-// lane l holds the positions of values 8 l .. 8 l + 7, one byte each. Byte x
-// at position p: output p; every position below p moves up by one (a byte-
-// wise compare and add on the lane's two words) and x's becomes 0. A byte
-// already at the front costs one compare. The chunk sits in the warp's
-// shared buffer and every byte is replaced there by its position.
+//
+// Three launches over chunks of `mc` bytes (512 .. 4,096; chunks never cross
+// blocks): the last occurrence of every byte value in every chunk, its
+// running maximum over each block's chunks, and the encoding of all chunks
+// at once, a warp each. A byte's code is the number of distinct bytes since
+// its last occurrence, so a warp encodes 32 bytes a step from the list
+// before them, with ballots in place of 32 list updates in a row.
+//
+// Measured on 38.5 M run bytes (64 mixed blocks): 2,117 us (one list update a
+// byte, a chain of shuffles) -> 485 us for the encoding, 476 -> 24 us for the
+// chunks' starting lists, 198 -> 48 us for the last occurrences. The encoding
+// is bound by issue (68%, 311 warp instructions a step of 32 bytes). Chunk
+// sizes: a chunk's starting list costs about 12 steps, so large batches take
+// 4,096-byte chunks (565 us in all; at most twice as many chunks: 588, five
+// times: 870); five CTAs an SM at 48 registers and four at 64 took the same.
 constexpr int MTF_WARPS = 8;
+constexpr uint32_t MTF_MIN = 512, MTF_MAX = 4096;  // chunk sizes
+constexpr uint32_t MTF_CHUNKS = 16384;             // chunks shorter than MTF_MAX: at most this many
 
-__global__ void __launch_bounds__(MTF_WARPS * 32) k_mtf_encode(const uint8_t* __restrict__ S,
-                                                               const TileDesc* __restrict__ tiles, uint32_t ntiles,
-                                                               const uint8_t* __restrict__ tlist,
-                                                               uint8_t* __restrict__ out) {
-    __shared__ __align__(16) uint8_t buf[MTF_WARPS][RTILE];
-    __shared__ __align__(16) uint8_t posb[MTF_WARPS][256];
+
+struct MtfChunk {
+    uint32_t start, len, rel, n;  // global start, bytes, block-relative start, bytes of the block
+};
+
+// Chunk c: cfirst[b] = first chunk of block b (cfirst[nb] = chunks).
+__device__ __forceinline__ MtfChunk mtf_chunk(const BlockInfo* __restrict__ blocks, const uint32_t* __restrict__ cfirst,
+                                              uint32_t nb, uint32_t c, uint32_t mc) {
+    uint32_t lo = 0, hi = nb;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (cfirst[mid] <= c) lo = mid; else hi = mid;
+    }
+    const BlockInfo bi = blocks[lo];
+    const uint32_t rel = (c - cfirst[lo]) * mc;
+    return MtfChunk{bi.off + rel, min(mc, bi.n - rel), rel, bi.n};
+}
+
+// One warp stages S[g0 .. g0 + len) at buf[shift ..), shift = the address
+// modulo 16 (returned): 16-byte loads where the aligned words around the
+// range lie inside S[0 .. N), else bytes. buf is 16-byte aligned and holds
+// len + 31 bytes.
+__device__ __forceinline__ uint32_t warp_stage(const uint8_t* __restrict__ S, uint32_t g0, uint32_t len, uint32_t N,
+                                               uint8_t* buf) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t shift = (uint32_t)(reinterpret_cast<uintptr_t>(S + g0) & 15u);
+    const uint32_t nvec = (shift + len + 15) >> 4;
+    if (g0 >= shift && (uint64_t)g0 - shift + 16ull * nvec <= N) {
+        const uint4* src = reinterpret_cast<const uint4*>(S + g0 - shift);
+        for (uint32_t v = lane; v < nvec; v += 32) reinterpret_cast<uint4*>(buf)[v] = __ldg(src + v);
+    } else {
+        for (uint32_t q = lane; q < len; q += 32) buf[shift + q] = S[g0 + q];
+    }
+    __syncwarp();
+    return shift;
+}
+
+// Pass 1: tab[chunk][x] = block-relative position + 1 of the last x in the
+// chunk, 0 if it holds none. A warp walks its chunk backwards, 32 bytes a
+// step; a step whose bytes were all seen costs a look-up and a ballot.
+__global__ void __launch_bounds__(MTF_WARPS * 32) k_mtf_last(const uint8_t* __restrict__ S, uint32_t N,
+                                                             const BlockInfo* __restrict__ blocks, uint32_t nb,
+                                                             const uint32_t* __restrict__ cfirst, uint32_t mc,
+                                                             uint32_t* __restrict__ tab) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_last[MTF_WARPS][256];
     const uint32_t lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    uint8_t* bw = buf[wl];
-    for (uint32_t t = blockIdx.x * MTF_WARPS + wl; t < ntiles; t += gridDim.x * MTF_WARPS) {
-        const TileDesc td = tiles[t];
-        for (uint32_t q = lane; q < td.len; q += 32) bw[q] = S[td.start + q];
-        const uint8_t* T = tlist + (size_t)t * 256;  // starting list: T[j] = value at position j
-        for (uint32_t j = lane; j < 256; j += 32) posb[wl][T[j]] = (uint8_t)j;
-        __syncwarp();
-        uint32_t lo = reinterpret_cast<const uint32_t*>(posb[wl])[2 * lane];      // positions of 8 l .. 8 l + 3
-        uint32_t hi = reinterpret_cast<const uint32_t*>(posb[wl])[2 * lane + 1];  // positions of 8 l + 4 .. 8 l + 7
-        uint32_t front = T[0];
-        __syncwarp();
-        for (uint32_t i = 0; i < td.len; ++i) {
-            const uint32_t x = bw[i];
-            if (x == front) {  // warp-uniform: x and front are the same in every lane
-                if (lane == 0) bw[i] = 0;
-                continue;
+    uint8_t* buf = smem + wl * (mc + 32);
+    uint32_t* last = s_last[wl];
+    const uint32_t nc = cfirst[nb];
+    for (uint32_t c = blockIdx.x * MTF_WARPS + wl; c < nc; c += gridDim.x * MTF_WARPS) {
+        const MtfChunk ch = mtf_chunk(blocks, cfirst, nb, c, mc);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) last[k * 32 + lane] = 0u;
+        const uint32_t shift = warp_stage(S, ch.start, ch.len, N, buf);
+        for (uint32_t b = (ch.len - 1) & ~31u;; b -= 32) {
+            const uint32_t q = b + lane;
+            const uint32_t x = q < ch.len ? buf[shift + q] : 256u;
+            const bool fresh = x < 256u && last[x] == 0u;
+            if (__any_sync(0xffffffffu, fresh)) {
+                const uint32_t peers = __match_any_sync(0xffffffffu, fresh ? x : 256u);
+                if (fresh && (peers >> lane) == 1u) last[x] = ch.rel + q + 1;  // the highest lane of its value
+                __syncwarp();
             }
-            const uint32_t owner = x >> 3, k = x & 7u;
-            const uint32_t word = __shfl_sync(0xffffffffu, k < 4 ? lo : hi, owner);
-            const uint32_t p = (word >> (8 * (k & 3))) & 0xffu;
-            const uint32_t p4 = p * 0x01010101u;
-            lo += __vcmpltu4(lo, p4) & 0x01010101u;  // positions below p move up (they stay <= 255)
-            hi += __vcmpltu4(hi, p4) & 0x01010101u;
-            if (lane == owner) {
-                const uint32_t clear = ~(0xffu << (8 * (k & 3)));
-                if (k < 4) lo &= clear; else hi &= clear;
-            }
-            if (lane == 0) bw[i] = (uint8_t)p;
-            front = x;
+            if (b == 0) break;
         }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) tab[(size_t)c * 256 + k * 32 + lane] = last[k * 32 + lane];
         __syncwarp();
-        for (uint32_t q = lane; q < td.len; q += 32) out[td.start + q] = bw[q];
+    }
+}
+
+// Pass 2, in place: tab[chunk][x] = position + 1 of the last x before the
+// chunk in its block, 0 if there is none. One CTA a block, a thread a value;
+// 16 chunks' loads are in flight at once.
+__global__ void __launch_bounds__(256) k_mtf_scan(const uint32_t* __restrict__ cfirst, uint32_t nb,
+                                                  uint32_t* __restrict__ tab) {
+    for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
+        uint32_t run = 0;
+        const uint32_t c1 = cfirst[b + 1];
+        for (uint32_t c = cfirst[b]; c < c1; c += 16) {
+            uint32_t v[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = c + k < c1 ? tab[(size_t)(c + k) * 256 + threadIdx.x] : 0u;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                if (c + k < c1) tab[(size_t)(c + k) * 256 + threadIdx.x] = run;
+                if (v[k]) run = v[k];  // later chunks hold later positions
+            }
+        }
+    }
+}
+
+// The list before a chunk: the byte values by last occurrence, latest first,
+// then those not seen yet in ascending order. A warp sorts (recency, value)
+// descending, bitonic, eight values a lane; KeyT holds recency << 8 | value.
+template <typename KeyT>
+__device__ __forceinline__ void mtf_start_list(const uint32_t* __restrict__ row, uint8_t* list, uint8_t* pos) {
+    const uint32_t lane = threadIdx.x & 31;
+    KeyT k[8];
+    const uint4 r0 = reinterpret_cast<const uint4*>(row)[lane * 2], r1 = reinterpret_cast<const uint4*>(row)[lane * 2 + 1];
+    const uint32_t rec[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t x = lane * 8 + i, r = rec[i];
+        k[i] = ((KeyT)(r ? r + 255u : 255u - x) << 8) | x;
+    }
+#pragma unroll
+    for (uint32_t kk = 2; kk <= 256; kk <<= 1) {
+#pragma unroll
+        for (uint32_t j = kk >> 1; j > 0; j >>= 1) {
+            if (j >= 8) {  // across lanes
+#pragma unroll
+                for (uint32_t i = 0; i < 8; ++i) {
+                    const KeyT o = __shfl_xor_sync(0xffffffffu, k[i], j >> 3);
+                    const bool down = ((lane * 8) & kk) == 0, lower = ((lane * 8) & j) == 0;
+                    k[i] = (lower == down) == (k[i] > o) ? k[i] : o;
+                }
+            } else {
+#pragma unroll
+                for (uint32_t i = 0; i < 8; ++i) {
+                    if ((i & j) == 0) {
+                        const bool down = ((lane * 8 + i) & kk) == 0;
+                        const KeyT a = k[i], b = k[i | j];
+                        const bool keep = (a > b) == down;
+                        k[i] = keep ? a : b;
+                        k[i | j] = keep ? b : a;
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t x = (uint32_t)k[i] & 255u;
+        list[lane * 8 + i] = (uint8_t)x;
+        pos[x] = (uint8_t)(lane * 8 + i);
+    }
+}
+
+// Pass 3: one warp encodes a chunk from its starting list, 32 bytes a step.
+// With p = a byte's position in the list before the step: a byte's first
+// occurrence in the step is encoded as p plus the distinct bytes of the step
+// before it that stood behind p (they have moved in front of it); a later
+// occurrence as the distinct bytes since the previous one, which are the
+// first ones of that stretch: those whose own previous occurrence is no
+// later than its start. Both compare a small number of every lane with this
+// lane's, for all lanes at once, by one ballot a bit. Then the step's bytes
+// move to the front by last occurrence, and the others up to the last
+// position touched move back by the step's bytes behind them.
+__global__ void __launch_bounds__(MTF_WARPS * 32, 5) k_mtf_encode(const uint8_t* __restrict__ S, uint32_t N,
+                                                               const BlockInfo* __restrict__ blocks, uint32_t nb,
+                                                               const uint32_t* __restrict__ cfirst, uint32_t mc,
+                                                               const uint32_t* __restrict__ tab,
+                                                               uint8_t* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint8_t s_list[MTF_WARPS][256], s_pos[MTF_WARPS][256];
+    const uint32_t lane = threadIdx.x & 31, wl = threadIdx.x >> 5, lt = lanemask_lt(), gt_lanes = ~(lt | (1u << lane));
+    uint8_t* buf = smem + wl * (mc + 32);
+    uint8_t *list = s_list[wl], *pos = s_pos[wl];
+    const uint32_t nc = cfirst[nb];
+    for (uint32_t c = blockIdx.x * MTF_WARPS + wl; c < nc; c += gridDim.x * MTF_WARPS) {
+        const MtfChunk ch = mtf_chunk(blocks, cfirst, nb, c, mc);
+        if (ch.n < (1u << 24) - 256u) mtf_start_list<uint32_t>(tab + (size_t)c * 256, list, pos);
+        else mtf_start_list<uint64_t>(tab + (size_t)c * 256, list, pos);
+        const uint32_t shift = warp_stage(S, ch.start, ch.len, N, buf);
+        for (uint32_t b = 0; b < ch.len; b += 32) {
+            // lanes past the end repeat the last byte: they change nothing
+            const uint32_t q = min(b + lane, ch.len - 1);
+            const uint32_t x = buf[shift + q];
+            const uint32_t p = pos[x];
+            const uint32_t maxp = __reduce_max_sync(0xffffffffu, p);
+            uint32_t r = 0;
+            if (maxp > 0u) {  // else 32 times the byte at the front
+                // lanes with this lane's byte, and lanes whose position is greater
+                uint32_t eq = 0xffffffffu, gt = 0u;
+#pragma unroll
+                for (int k = 7; k >= 0; --k) {
+                    if (maxp >> k) {  // warp-uniform
+                        const bool one = (p >> k) & 1u;
+                        const uint32_t B = __ballot_sync(0xffffffffu, one);
+                        const uint32_t m = one ? 0u : 0xffffffffu;
+                        gt |= eq & B & m;
+                        eq &= B ^ m;
+                    }
+                }
+                const uint32_t before = eq & lt;
+                const bool first = before == 0u;
+                const uint32_t F = __ballot_sync(0xffffffffu, first);
+                r = p + __popc(gt & F & lt);
+                if (F != 0xffffffffu) {
+                    const uint32_t prev = 32u - __clz(before);  // lane of the previous occurrence + 1, 0: none
+                    uint32_t e2 = 0xffffffffu, less = 0u;       // lanes with an equal prev, with a smaller one
+#pragma unroll
+                    for (int k = 4; k >= 0; --k) {
+                        const bool one = (prev >> k) & 1u;
+                        const uint32_t B = __ballot_sync(0xffffffffu, one);
+                        const uint32_t m = one ? 0xffffffffu : 0u;
+                        less |= e2 & ~B & m;
+                        e2 &= ~(B ^ m);
+                    }
+                    if (!first) r = __popc(less & lt & (0xffffffffu << prev));
+                }
+                const bool last = (eq & gt_lanes) == 0u;
+                const uint32_t La = __ballot_sync(0xffffffffu, last);
+                const uint32_t D = __popc(F);
+                uint32_t below = D;  // the step's positions below word w
+                for (int w = (int)(maxp >> 5); w >= 0; --w) {
+                    const uint32_t mine = first && (int)(p >> 5) == w ? 1u << (p & 31u) : 0u;
+                    const uint32_t m = __reduce_or_sync(0xffffffffu, mine);
+                    below -= __popc(m);
+                    const uint32_t j = w * 32 + lane;
+                    const uint32_t v = list[j];
+                    __syncwarp();  // the word is read before its entries move up (into this word and the next)
+                    if (j <= maxp && !((m >> lane) & 1u)) {
+                        const uint32_t np = j + D - below - __popc(m & lt);
+                        list[np] = (uint8_t)v;
+                        pos[v] = (uint8_t)np;
+                    }
+                }
+                if (last) {
+                    const uint32_t np = __popc(La & gt_lanes);
+                    list[np] = (uint8_t)x;
+                    pos[x] = (uint8_t)np;
+                }
+                __syncwarp();
+            }
+            if (b + lane < ch.len) buf[shift + b + lane] = (uint8_t)r;
+            __syncwarp();  // the last byte is read by the lanes past the end
+        }
+        // out, by 16-byte words where its address has the staged alignment
+        uint8_t* o = out + ch.start;
+        uint32_t q0 = 0, q1 = 0;  // bytes [q0, q1) go as whole words
+        if ((reinterpret_cast<uintptr_t>(o) & 15u) == shift && shift + ch.len >= 32u) {
+            q0 = (16u - shift) & 15u;
+            q1 = ((shift + ch.len) & ~15u) - shift;
+            for (uint32_t q = q0 + lane * 16; q < q1; q += 512)
+                *reinterpret_cast<uint4*>(o + q) = *reinterpret_cast<const uint4*>(buf + shift + q);
+        }
+        for (uint32_t q = lane; q < q0; q += 32) o[q] = buf[shift + q];
+        for (uint32_t q = q1 + lane; q < ch.len; q += 32) o[q] = buf[shift + q];
         __syncwarp();
     }
 }
@@ -655,26 +774,31 @@ extern "C" bwt_status bwt_mtf_encode(bwt_plan* p, const uint8_t* d_in, const uin
     std::memset(&p->stats, 0, sizeof(p->stats));
     bwt_status s = prepare_batch(p, offsets, num_blocks, st);
     if (s != BWT_OK) return p->last = s;
-    if (p->tile > (int)RTILE) return p->last = BWT_EINVAL;
-    const uint32_t nb = p->nb, nt = p->ntiles0;
-    // scratch (first use): per chunk its list of last occurrences, its count and its starting list;
-    // per block its first chunk
-    if (!p->mtf_lists) CKS(cudaMalloc(&p->mtf_lists, (size_t)p->cap_tiles0 * (512 + 4) + 4 * ((size_t)p->cap_b + 1)));
-    uint8_t* mru = p->mtf_lists;
-    uint8_t* tlist = mru + (size_t)p->cap_tiles0 * 256;
-    uint32_t* mcnt = reinterpret_cast<uint32_t*>(tlist + (size_t)p->cap_tiles0 * 256);
-    uint32_t* tfirst = mcnt + p->cap_tiles0;
+    const uint32_t nb = p->nb, N = p->total;
+    // chunk size: the smallest that leaves at most MTF_CHUNKS of them (a
+    // small batch is latency: more and shorter chunks), 4,096 for large batches
+    uint32_t mc = MTF_MIN;
+    while (mc < MTF_MAX && N / mc > MTF_CHUNKS) mc <<= 1;
+    // scratch (first use): 256 words a chunk, per block its first chunk
+    const size_t cap_chunks = std::min<size_t>(p->cap_n / MTF_MIN, std::max<size_t>(MTF_CHUNKS, p->cap_n / MTF_MAX)) +
+                              (size_t)p->cap_b + 1;
+    if (!p->mtf_lists) CKS(cudaMalloc(&p->mtf_lists, cap_chunks * 1024 + 4 * ((size_t)p->cap_b + 1)));
+    uint32_t* tab = reinterpret_cast<uint32_t*>(p->mtf_lists);
+    uint32_t* cfirst = tab + cap_chunks * 256;
     uint32_t* h_first = p->h_inv_items;  // pinned staging, free outside the inverse
-    for (uint32_t t = 0, b = 0; t < nt; ++t)
-        if (t == 0 || p->h_tiles[t].blk != p->h_tiles[t - 1].blk) h_first[b++] = t;
-    h_first[nb] = nt;
-    CKS(cudaMemcpyAsync(tfirst, h_first, sizeof(uint32_t) * (nb + 1), cudaMemcpyHostToDevice, st));
+    uint32_t nc = 0;
+    for (uint32_t b = 0; b < nb; ++b) {
+        h_first[b] = nc;
+        nc += (uint32_t)((p->h_off[b + 1] - p->h_off[b] + mc - 1) / mc);
+    }
+    h_first[nb] = nc;
+    CKS(cudaMemcpyAsync(cfirst, h_first, sizeof(uint32_t) * (nb + 1), cudaMemcpyHostToDevice, st));
     const int sms = num_sms();
-    k_mtf_mru<<<std::max(1, std::min<int>(nt, sms * 8)), RT, 0, st>>>(d_in, p->tiles0, nt, mru, mcnt);
-    k_mtf_chain<<<std::max(1u, std::min<uint32_t>((nb + 7) / 8, (uint32_t)sms * 8)), 256, 0, st>>>(tfirst, nb, mru,
-                                                                                                 mcnt, tlist);
-    k_mtf_encode<<<std::max(1, std::min<int>((nt + MTF_WARPS - 1) / MTF_WARPS, sms * 6)), MTF_WARPS * 32, 0, st>>>(
-        d_in, p->tiles0, nt, tlist, d_out);
+    const size_t smem = (size_t)MTF_WARPS * (mc + 32);
+    const int grid = std::max(1, std::min<int>((nc + MTF_WARPS - 1) / MTF_WARPS, sms * 8));
+    k_mtf_last<<<grid, MTF_WARPS * 32, smem, st>>>(d_in, N, p->blocks, nb, cfirst, mc, tab);
+    k_mtf_scan<<<std::min<uint32_t>(nb, (uint32_t)sms * 8), 256, 0, st>>>(cfirst, nb, tab);
+    k_mtf_encode<<<grid, MTF_WARPS * 32, smem, st>>>(d_in, N, p->blocks, nb, cfirst, mc, tab, d_out);
     CKS(cudaGetLastError());
     p->stats.kernel_launches = 3;
     CKS(cudaStreamSynchronize(st));

@@ -4,8 +4,10 @@ from __future__ import annotations
 import numpy as np
 import pytest
 
+import oracle
+
 from paper_1109_2348_gb300 import F_GRAPH, F_LEARNED, Plan, datagen, model
-from tests.gpu_util import assert_matches_oracle, batch_from_blocks, gpu_bwt
+from gpu_util import assert_matches_oracle, batch_from_blocks, gpu_bwt
 
 pytestmark = pytest.mark.gpu
 
@@ -48,3 +50,39 @@ def test_chunk_sort_words(kind, table):
         model.install(plan, spl)
         L, prim, _ = gpu_bwt(buf, off, plan)
     assert_matches_oracle(buf, off, L, prim, f"{kind}/{table}")
+
+
+def _mtf_blocks(kind):
+    r = np.random.RandomState(21)
+    if kind == "edges":  # sizes around a step, a chunk and a chunk's last step, over alphabets of every size
+        return [r.randint(0, a, n).astype(np.uint8) for a in (1, 2, 33, 256)
+                for n in (1, 31, 32, 33, 63, 511, 512, 513, 1024, 1535, 4097)]
+    if kind == "large_chunks":  # 9 MB: 1,024-byte chunks; runs, then every byte value in turn
+        b = r.randint(0, 90, 9_000_000).astype(np.uint8)
+        b[1_000_000:1_200_000] = 7
+        b[5_000_000:5_002_560] = np.tile(np.arange(255, -1, -1), 10)
+        return [b, b[:70_001]]
+    # over 2^24 bytes: recencies that need more than 24 bits; a byte value last seen at the very start
+    b = (datagen.block(datagen.RUNS16, 5, 17_000_000) + 1).astype(np.uint8)
+    b[:300] = np.arange(300) % 256
+    b[-300:] = np.arange(300)[::-1] % 256
+    return [b]
+
+
+@pytest.mark.parametrize("shift_in, shift_out", [(0, 0), (5, 5), (3, 8)])
+@pytest.mark.parametrize("kind", ["edges", "large_chunks", "over_24_bits"])
+def test_mtf_steps_and_chunks(kind, shift_in, shift_out):
+    """Move-to-front by 32-byte steps: sizes around steps and chunks, every
+    chunk size, and buffers of equal and of different alignment."""
+    import torch
+    buf, off = batch_from_blocks(_mtf_blocks(kind))
+    sizes = np.diff(off.astype(np.int64))
+    d_in = torch.zeros(buf.size + 16, dtype=torch.uint8, device="cuda")
+    d_in[shift_in:shift_in + buf.size] = torch.from_numpy(buf).cuda()
+    d_out = torch.full((buf.size + 32,), 0xEE, dtype=torch.uint8, device="cuda")
+    with Plan(max_blocks=off.size - 1, max_total_bytes=buf.size, max_block_bytes=int(sizes.max())) as plan:
+        plan.mtf_encode_into(d_in[shift_in:shift_in + buf.size], off, d_out[shift_out:shift_out + buf.size])
+    got = d_out.cpu().numpy()
+    want = np.concatenate([oracle.mtf_encode(buf[int(off[b]):int(off[b + 1])]) for b in range(off.size - 1)])
+    assert np.array_equal(got[shift_out:shift_out + buf.size], want)
+    assert (got[:shift_out] == 0xEE).all() and (got[shift_out + buf.size:] == 0xEE).all()  # nothing written outside
