@@ -165,8 +165,9 @@ bwt_status bwt_inverse_check(const uint8_t* L, uint64_t n, int32_t primary, cons
  *   d_primary   device, int32[num_blocks]: the primary index of every block.
  *   d_out       device, uint8[offsets[num_blocks]]: receives the blocks.
  *   stream      cudaStream_t to run on (NULL = the legacy default stream).
- * Uses the plan's scratch plus about 1.5 bytes per byte of max_total_bytes
- * allocated on the first call. Returns BWT_EINVAL for bad arguments and for a primary
+ * Uses the plan's scratch plus about 0.75 bytes per byte of max_total_bytes
+ * (and 44 a block; 4 bytes per byte and 64 a block more in a plan whose
+ * blocks average under 16 bytes) allocated on the first call. Returns BWT_EINVAL for bad arguments and for a primary
  * outside [0, n) (found on the device; that block's output is undefined).
  * The call synchronises `stream` before it returns. d_out must not alias
  * d_L. For any L that is a permutation of some block's bytes the result is

@@ -250,6 +250,48 @@ __device__ __forceinline__ uint32_t stage_tile_bytes(const uint8_t* __restrict__
     return 0;
 }
 
+// Decoupled look-back of one digit of a radix tile: the number of keys with
+// digit d in the segment's tiles before t (t > first). `status` holds
+// [tile][radix] words (ST_AGG / ST_INC | count). Walks back LB predecessors a
+// step: their words are loaded together, then added in order until an
+// inclusive one. When the tiles of a segment run at once (a small batch),
+// their words are mostly aggregates, and the walk is a chain of L2 round trips
+// that this shortens LB-fold. A wait that runs past spin_limit polls sets
+// ERR_TIMEOUT in *err and counts an inclusive zero: the prefix is short, but
+// stays inside the segment.
+__device__ __forceinline__ uint32_t lookback_digit(const uint32_t* status, uint32_t radix, uint32_t t, uint32_t first,
+                                                   uint32_t d, uint32_t spin_limit, uint32_t* err) {
+    constexpr uint32_t LB = 4;
+    uint32_t excl = 0, q = t - 1;  // the next predecessor to add (>= first)
+    for (;;) {
+        const uint32_t m = min(LB, q - first + 1);
+        uint32_t v[LB];
+#pragma unroll
+        for (uint32_t k = 0; k < LB; ++k) v[k] = k < m ? ld_volatile(status + (size_t)(q - k) * radix + d) : 0u;
+        bool done = false;
+#pragma unroll
+        for (uint32_t k = 0; k < LB; ++k) {
+            if (k >= m || done) break;
+            uint32_t it = 0;
+            while ((v[k] & (ST_AGG | ST_INC)) == 0u) {
+                if (++it > spin_limit) {
+                    atomicOr(err, ERR_TIMEOUT);
+                    v[k] = ST_INC;  // give up: proceed with a short prefix (stays in bounds)
+                    break;
+                }
+                if (it > 32) __nanosleep(64);
+                v[k] = ld_volatile(status + (size_t)(q - k) * radix + d);
+            }
+            excl += v[k] & ST_VALUE;
+            if (v[k] & ST_INC) done = true;
+        }
+        // the segment's first tile is always inclusive: reaching it ends the walk
+        if (done || q + 1 - m == first) break;
+        q -= m;
+    }
+    return excl;
+}
+
 // ---- single-pass scan of one 64-bit count per tile -------------------------
 //
 // Decoupled look-back: tile t publishes its own total (AGG) at once and its

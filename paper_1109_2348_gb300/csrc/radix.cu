@@ -239,40 +239,7 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
                 const int d = tid;
                 uint32_t excl = 0;
                 if (!first) {
-                    // Walk back LB predecessors a step: their words are loaded
-                    // together, then added in order until an inclusive one. When
-                    // the tiles of a segment run at once (a small batch), their
-                    // words are mostly aggregates, and the walk is a chain of
-                    // L2 round trips that this shortens LB-fold.
-                    constexpr uint32_t LB = 4;
-                    uint32_t q = t - 1;  // the next predecessor to add (>= firstTile)
-                    for (;;) {
-                        const uint32_t m = min(LB, q - td.firstTile + 1);
-                        uint32_t v[LB];
-#pragma unroll
-                        for (uint32_t k = 0; k < LB; ++k)
-                            v[k] = k < m ? ld_volatile(p.status + (size_t)(q - k) * RADIX + d) : 0u;
-                        bool done = false;
-#pragma unroll
-                        for (uint32_t k = 0; k < LB; ++k) {
-                            if (k >= m || done) break;
-                            uint32_t it = 0;
-                            while ((v[k] & (ST_AGG | ST_INC)) == 0u) {
-                                if (++it > spin_limit) {
-                                    atomicOr(&p.ctrl[CTRL_ERR], ERR_TIMEOUT);
-                                    v[k] = ST_INC;  // give up: proceed with a short prefix (stays in bounds)
-                                    break;
-                                }
-                                if (it > 32) __nanosleep(64);
-                                v[k] = ld_volatile(p.status + (size_t)(q - k) * RADIX + d);
-                            }
-                            excl += v[k] & ST_VALUE;
-                            if (v[k] & ST_INC) done = true;
-                        }
-                        // the segment's first tile is always inclusive: reaching it ends the walk
-                        if (done || q + 1 - m == td.firstTile) break;
-                        q -= m;
-                    }
+                    excl = lookback_digit(p.status, RADIX, t, td.firstTile, d, spin_limit, &p.ctrl[CTRL_ERR]);
                     st_volatile(p.status + (size_t)t * RADIX + d, ST_INC | ((excl + cnt[0]) & ST_VALUE));
                 }
                 gbase[d] = td.segStart + p.seg_base[(size_t)td.seg * p.seg_base_stride + d] + excl - digit_start[d];
@@ -343,8 +310,9 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
 // ---- histograms ------------------------------------------------------------
 
 // d = 8: byte histogram of every block. Each thread counts a run of 16
-// consecutive bytes and adds whole runs of equal bytes, so run-heavy blocks
-// do not serialise on one shared-memory counter.
+// consecutive bytes (one 16-byte load where they are aligned) and adds whole
+// runs of equal bytes, so run-heavy blocks do not serialise on one shared-
+// memory counter.
 __global__ void __launch_bounds__(256) k_hist_bytes(const uint8_t* __restrict__ S, const BlockInfo* __restrict__ blocks,
                                                     const TileDesc* __restrict__ tiles, uint32_t num_tiles,
                                                     const uint32_t* __restrict__ num_tiles_dev,
@@ -357,14 +325,23 @@ __global__ void __launch_bounds__(256) k_hist_bytes(const uint8_t* __restrict__ 
         const TileDesc td = tiles[t];
         for (uint32_t c0 = threadIdx.x * 16; c0 < td.len; c0 += 256 * 16) {
             const uint32_t c1 = min(c0 + 16, td.len);
-            uint32_t prev = S[td.start + c0], run = 1;
-            for (uint32_t q = c0 + 1; q < c1; ++q) {
-                const uint32_t b = S[td.start + q];
-                if (b == prev) {
+            const uint8_t* src = S + td.start + c0;
+            __align__(16) uint8_t by[16];
+            if (c1 - c0 == 16 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0u) {
+                *reinterpret_cast<uint4*>(by) = __ldg(reinterpret_cast<const uint4*>(src));
+            } else {
+#pragma unroll
+                for (uint32_t q = 0; q < 16; ++q) by[q] = c0 + q < c1 ? src[q] : (uint8_t)0;
+            }
+            uint32_t prev = by[0], run = 1;
+#pragma unroll
+            for (uint32_t q = 1; q < 16; ++q) {
+                if (c0 + q >= c1) break;
+                if (by[q] == prev) {
                     ++run;
                 } else {
                     atomicAdd(&h[prev], run);
-                    prev = b;
+                    prev = by[q];
                     run = 1;
                 }
             }

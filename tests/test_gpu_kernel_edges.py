@@ -86,3 +86,39 @@ def test_mtf_steps_and_chunks(kind, shift_in, shift_out):
     want = np.concatenate([oracle.mtf_encode(buf[int(off[b]):int(off[b + 1])]) for b in range(off.size - 1)])
     assert np.array_equal(got[shift_out:shift_out + buf.size], want)
     assert (got[:shift_out] == 0xEE).all() and (got[shift_out + buf.size:] == 0xEE).all()  # nothing written outside
+
+
+def _inverse_blocks(kind):
+    r = np.random.RandomState(31)
+    if kind == "tiny":  # blocks of a few bytes: more samples than the plan's key buffer holds
+        return [r.randint(0, 3, n).astype(np.uint8) for n in r.randint(1, 12, 700)]
+    if kind == "strides":  # around a sample (8 rows), a super (64), the stored bytes of a sample (24)
+        return [r.randint(0, a, n).astype(np.uint8) for a in (2, 256)
+                for n in (1, 7, 8, 9, 23, 24, 25, 63, 64, 65, 127, 129, 511, 513, 4095, 4097)]
+    if kind == "periods":  # several cycles; walks far longer than a sample stores
+        return [np.tile(r.randint(0, 256, p).astype(np.uint8), k) for p, k in ((1, 3000), (3, 1001), (64, 65), (700, 9))]
+    if kind == "many_supers":  # above and below the supers that one CTA ranks in shared memory
+        return [r.randint(0, 100, n).astype(np.uint8) for n in (1_048_560, 1_048_640, 1_400_003)]
+    return [r.randint(0, 256, (1 << 24) + 77).astype(np.uint8), r.randint(0, 256, 1000).astype(np.uint8)]
+
+
+@pytest.mark.parametrize("tile", [1024, 2048, 4096])
+@pytest.mark.parametrize("kind", ["tiny", "strides", "periods", "many_supers", "over_24_bits"])
+def test_inverse_samples_and_supers(kind, tile):
+    """GPU forward, then the inverse into a buffer of odd alignment: the
+    blocks come back and nothing outside them is written."""
+    import torch
+    if kind in ("many_supers", "over_24_bits") and tile != 4096:
+        pytest.skip("large blocks: one tile size")
+    buf, off = batch_from_blocks(_inverse_blocks(kind))
+    sizes = np.diff(off.astype(np.int64))
+    d_in = torch.from_numpy(buf).cuda()
+    out = torch.full((buf.size + 32,), 0xEE, dtype=torch.uint8, device="cuda")
+    with Plan(max_blocks=off.size - 1, max_total_bytes=buf.size, max_block_bytes=int(sizes.max()),
+              tile_keys=tile) as plan:
+        L, prim = plan.forward(d_in, off)
+        if kind not in ("many_supers", "over_24_bits"):
+            assert_matches_oracle(buf, off, L.cpu().numpy(), prim.cpu().numpy(), kind)
+        plan.inverse_into(L, off, prim, out[5:5 + buf.size])
+    assert torch.equal(out[5:5 + buf.size], d_in)
+    assert bool((out[:5] == 0xEE).all()) and bool((out[5 + buf.size:] == 0xEE).all())
