@@ -3,9 +3,8 @@
 //
 // Encode: a byte ends a run if the next byte differs or starts another block
 // (runs never cross blocks); an exclusive prefix sum of these flags gives
-// every run its output slot; the run's byte and its end index (global, one
-// past the last byte) go to that slot; a run's length is the difference of
-// consecutive end indices. Decode: the inclusive prefix sum of the lengths
+// every run its output slot; a run's length is the difference of consecutive
+// end indices (the end before a tile's first run comes from the tiles before). Decode: the inclusive prefix sum of the lengths
 // gives every run's end; flags at the last byte of every run, prefix-summed
 // over the output, give every output byte its run; the byte is copied.
 //
@@ -66,75 +65,156 @@ __device__ __forceinline__ uint32_t next_tile(uint32_t* s_tile, uint32_t* counte
     return t;
 }
 
-// Encode steps 1-3: run-end flags, their prefix sum, and the scatter of
-// (byte, end index) to the run's slot. run_off[b] = the first run of block b
-// (run_off[nb] = the number of runs).
+// The 16 bytes at S[t0 + 16 tid ..] of a tile of `len` bytes, as four words:
+// one 16-byte load where the tile is whole and aligned, else through sb
+// (RTILE bytes, 16-byte aligned; bytes past the tile are undefined). All
+// threads call; sb is free again after the next barrier.
+__device__ __forceinline__ uint4 tile_words(const uint8_t* __restrict__ S, uint32_t t0, uint32_t len, uint8_t* sb) {
+    if (len == RTILE && (reinterpret_cast<uintptr_t>(S + t0) & 15u) == 0u)
+        return __ldg(reinterpret_cast<const uint4*>(S + t0) + threadIdx.x);
+    for (uint32_t q = threadIdx.x; q < len; q += RT) sb[q] = S[t0 + q];
+    __syncthreads();
+    return reinterpret_cast<const uint4*>(sb)[threadIdx.x];
+}
+
+// Bit j: byte j of a and of b differ.
+__device__ __forceinline__ uint32_t bytes_differ(uint32_t a, uint32_t b) {
+    return (__vsetne4(a, b) * 0x01020408u) >> 24;
+}
+
+// The last run end before tile t, from the tiles' published ones (`tail`:
+// LB_INC | end index, 0 for a tile without one, per tile; zero = not yet
+// published): the nearest tile with one, 32 tiles a step. 0 before the first.
+// All 32 lanes of a warp call; bounded like the look-back.
+__device__ __forceinline__ uint32_t last_end_before(const uint64_t* tail, uint32_t t, uint32_t spin_limit, uint32_t* err) {
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t end = t; end > 0; end = end > 32 ? end - 32 : 0) {
+        uint64_t v = 0;
+        if (lane < end) {
+            uint32_t it = 0;
+            while (((v = ld_volatile64(tail + (end - 1 - lane))) & LB_INC) == 0ull) {
+                if (++it > spin_limit) {
+                    atomicOr(err, ERR_TIMEOUT);
+                    break;
+                }
+                if (it > 32) __nanosleep(64);
+            }
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, (uint32_t)v != 0u);
+        if (m) return __shfl_sync(0xffffffffu, (uint32_t)v, __ffs(m) - 1);
+    }
+    return 0u;
+}
+
+// Encode, one pass: run-end flags, their prefix sum (block scan and look-back
+// over the tiles), and every run's byte and length -- the difference of
+// consecutive end indices -- compacted through shared memory so that they are
+// written in rows. run_off[b] = the first run of block b (run_off[nb] = the
+// number of runs). 64 mixed blocks (57.6 MB, 38.5 M runs): 388 us with byte
+// loads and every thread writing its own runs, and 72 us for a second pass
+// over the end indices -> 147 us. Bound by the look-back: 1,200 tiles in
+// flight poll each other's words. Measured for the whole call (177 us): the
+// look-back by 128 words a warp 211, by the whole CTA 204, tiles of 16,384
+// bytes 181, five CTAs an SM 244.
 __global__ void __launch_bounds__(RT) k_rle_encode(const uint8_t* __restrict__ S, uint32_t N,
                                                    const BlockInfo* __restrict__ blocks, uint32_t nb,
-                                                   uint8_t* __restrict__ chars, uint32_t* __restrict__ ends,
+                                                   uint8_t* __restrict__ chars, uint32_t* __restrict__ lens,
                                                    uint64_t* __restrict__ run_off, uint64_t* __restrict__ status,
-                                                   uint32_t* __restrict__ counter, uint32_t* ctrl) {
-    __shared__ __align__(16) uint8_t sb[RTILE + 16];
-    __shared__ uint32_t s_tile, scan_tmp[32];
+                                                   uint64_t* __restrict__ tail, uint32_t* __restrict__ counter,
+                                                   uint32_t* ctrl) {
+    __shared__ __align__(16) uint8_t sb[RTILE];  // staged bytes, then the tile's run bytes
+    __shared__ uint16_t se[RTILE];               // the runs' end positions in the tile
+    __shared__ uint8_t s_first[RT / 32 + 1];     // each warp's first byte (and the next tile's)
+    __shared__ uint32_t s_tile, s_last, s_prev, scan_tmp[32];
     __shared__ uint64_t s_excl;
     const uint32_t ntiles = (N + RTILE - 1) / RTILE;
     const uint32_t spin = ctrl[CTRL_SPIN], withhold = ctrl[CTRL_WITHHOLD];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (;;) {
         const uint32_t t = next_tile(&s_tile, counter);
         if (t >= ntiles) break;
         const uint32_t t0 = t * RTILE, len = min(RTILE, N - t0);
-        for (uint32_t q = threadIdx.x; q < len + 1 && t0 + q < N; q += RT) sb[q] = S[t0 + q];
+        const uint4 v = tile_words(S, t0, len, sb);
+        const uint32_t b0 = block_at(blocks, nb, t0), bend0 = blocks[b0].off + blocks[b0].n;
+        if (lane == 0) s_first[warp] = (uint8_t)v.x;
+        if (threadIdx.x == 0) {
+            s_first[RT / 32] = t0 + len < N ? S[t0 + len] : (uint8_t)0;
+            s_last = 0u;
+        }
+        uint32_t after = __shfl_down_sync(0xffffffffu, v.x, 1);  // its low byte follows this thread's
         __syncthreads();
+        if (lane == 31) after = s_first[warp + 1];
         const uint32_t q0 = threadIdx.x * RI, i0 = t0 + q0;
-        uint32_t flags = 0;  // bit j: element q0 + j ends a run
-        uint32_t b = i0 < N ? block_at(blocks, nb, i0) : 0u;
-        {
-            uint32_t bend = i0 < N ? blocks[b].off + blocks[b].n : 0u, bb = b;
+        uint32_t flags = bytes_differ(v.x, __funnelshift_r(v.x, v.y, 8)) |
+                         bytes_differ(v.y, __funnelshift_r(v.y, v.z, 8)) << 4 |
+                         bytes_differ(v.z, __funnelshift_r(v.z, v.w, 8)) << 8 |
+                         bytes_differ(v.w, __funnelshift_r(v.w, after, 8)) << 12;
+        // block ends: none inside most tiles
+        const bool inside = bend0 < t0 + len;  // CTA-uniform: another block starts in the tile
+        uint32_t starts = 0;                   // bit j: element q0 + j starts a block
+        uint32_t b = b0;
+        if (inside) {
+            b = i0 < N ? block_at(blocks, nb, i0) : 0u;
+            uint32_t bb = b, bend = i0 < N ? blocks[b].off + blocks[b].n : 0u;
+            if (i0 < N && blocks[b].off == i0) starts |= 1u;
 #pragma unroll
             for (int j = 0; j < RI; ++j) {
-                const uint32_t i = i0 + j;
-                if (i >= N) break;
-                while (i >= bend) {
+                if (i0 + j >= N) break;
+                if (i0 + j == bend) {
                     ++bb;
                     bend = blocks[bb].off + blocks[bb].n;
+                    starts |= 1u << j;
                 }
-                const bool end = i + 1 == N || i + 1 == bend || sb[q0 + j + 1] != sb[q0 + j];
-                flags |= (uint32_t)end << j;
+                if (i0 + j + 1 == bend) flags |= 1u << j;
             }
+        } else {
+            if (threadIdx.x == 0 && blocks[b0].off == t0) starts = 1u;
+            if (bend0 == t0 + len && bend0 - 1 - i0 < (uint32_t)RI) flags |= 1u << (bend0 - 1 - i0);
         }
+        if (q0 + RI > len) flags &= q0 < len ? (1u << (len - q0)) - 1u : 0u;
         uint32_t total;
         const uint32_t pre = block_exclusive_scan<RT>(__popc(flags), scan_tmp, &total);
-        if (threadIdx.x < 32) {
-            const uint64_t e = lookback_u64(status, t, 0, total, spin, &ctrl[CTRL_ERR], withhold);
-            if (threadIdx.x == 0) s_excl = e;
+        // the tile's runs, compacted (every thread holds its bytes in registers)
+        {
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            uint32_t k = pre;
+#pragma unroll
+            for (int j = 0; j < RI; ++j) {
+                if ((flags >> j) & 1u) {
+                    sb[k] = (uint8_t)(w[j / 4] >> (8 * (j % 4)));
+                    se[k] = (uint16_t)(q0 + j + 1);
+                    ++k;
+                }
+            }
+            const uint32_t last = __reduce_max_sync(0xffffffffu, flags ? t0 + q0 + 32u - __clz(flags) : 0u);
+            if (lane == 0 && last) atomicMax(&s_last, last);
         }
         __syncthreads();
-        uint64_t k = s_excl + pre;
-#pragma unroll
-        for (int j = 0; j < RI; ++j) {
-            const uint32_t i = i0 + j;
-            if (i >= N) break;
-            while (b + 1 < nb && blocks[b + 1].off <= i) ++b;
-            if (blocks[b].off == i) run_off[b] = k;  // runs before the block's first byte
-            if ((flags >> j) & 1u) {
-                if (k < N) {
-                    chars[k] = sb[q0 + j];
-                    ends[k] = i + 1;
-                }
-                ++k;
+        if (warp == 0) {
+            const uint64_t e = lookback_u64(status, t, 0, total, spin, &ctrl[CTRL_ERR], withhold);
+            if (lane == 0) s_excl = e;
+        } else if (warp == 1) {
+            if (lane == 0) st_volatile64(tail + t, LB_INC | s_last);
+            const uint32_t e = total ? last_end_before(tail, t, spin, &ctrl[CTRL_ERR]) : 0u;
+            if (lane == 0) s_prev = e;
+        }
+        __syncthreads();
+        const uint64_t k0 = s_excl;
+        while (starts) {  // runs before the block's first byte
+            const int j = __ffs(starts) - 1;
+            starts &= starts - 1;
+            while (blocks[b].off < i0 + j) ++b;
+            run_off[b] = k0 + pre + __popc(flags & ((1u << j) - 1u));
+        }
+        if (t + 1 == ntiles && threadIdx.x == 0) run_off[nb] = k0 + total;
+        for (uint32_t i = threadIdx.x; i < total; i += RT) {
+            if (k0 + i < N) {
+                chars[k0 + i] = sb[i];
+                lens[k0 + i] = i ? (uint32_t)(se[i] - se[i - 1]) : t0 + se[0] - s_prev;
             }
-            if (i + 1 == N) run_off[nb] = k;
         }
         __syncthreads();
     }
-}
-
-// Encode step 4: run lengths from consecutive end indices.
-__global__ void k_rle_lengths(const uint32_t* __restrict__ ends, const uint64_t* __restrict__ run_off, uint32_t nb,
-                              uint32_t* __restrict__ lens) {
-    const uint64_t R = run_off[nb];
-    for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < R; k += (uint64_t)gridDim.x * blockDim.x)
-        lens[k] = ends[k] - (k ? ends[k - 1] : 0u);
 }
 
 // Decode step 1: B[k] = end of run k (inclusive prefix sum of the lengths,
@@ -147,18 +227,34 @@ __global__ void __launch_bounds__(RT) k_rle_scan(const uint32_t* __restrict__ le
     __shared__ uint64_t s_excl;
     const uint64_t R = min(run_off[nb], (uint64_t)N);  // a run holds at least one byte
     const uint32_t ntiles = (uint32_t)((R + RTILE - 1) / RTILE);
+    const bool vec = (reinterpret_cast<uintptr_t>(lens) & 15u) == 0u;
     const uint32_t spin = ctrl[CTRL_SPIN], withhold = ctrl[CTRL_WITHHOLD];
     for (;;) {
         const uint32_t t = next_tile(&s_tile, counter);
         if (t >= ntiles) break;
         const uint64_t k0 = (uint64_t)t * RTILE + threadIdx.x * RI;
+        const bool whole = vec && k0 + RI <= R;
         uint32_t v[RI], sum = 0;
+        if (whole) {
+#pragma unroll
+            for (int j = 0; j < RI; j += 4) {
+                const uint4 x = __ldg(reinterpret_cast<const uint4*>(lens + k0 + j));
+                v[j] = x.x;
+                v[j + 1] = x.y;
+                v[j + 2] = x.z;
+                v[j + 3] = x.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < RI; ++j) v[j] = k0 + j < R ? lens[k0 + j] : 0u;
+        }
+        bool zero = false;
 #pragma unroll
         for (int j = 0; j < RI; ++j) {
-            v[j] = k0 + j < R ? lens[k0 + j] : 0u;
-            if (k0 + j < R && v[j] == 0u) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
+            zero |= v[j] == 0u && k0 + j < R;
             sum += v[j];
         }
+        if (zero) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
         uint32_t total;
         const uint32_t pre = block_exclusive_scan<RT>(sum, scan_tmp, &total);
         if (threadIdx.x < 32) {
@@ -170,7 +266,16 @@ __global__ void __launch_bounds__(RT) k_rle_scan(const uint32_t* __restrict__ le
 #pragma unroll
         for (int j = 0; j < RI; ++j) {
             acc += v[j];
-            if (k0 + j < R) B[k0 + j] = (uint32_t)acc;
+            v[j] = (uint32_t)acc;
+        }
+        if (k0 + RI <= R) {  // B is the plan's, 16-byte aligned
+#pragma unroll
+            for (int j = 0; j < RI; j += 4)
+                *reinterpret_cast<uint4*>(B + k0 + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < RI; ++j)
+                if (k0 + j < R) B[k0 + j] = v[j];
         }
         __syncthreads();
     }
@@ -186,54 +291,92 @@ __global__ void k_rle_check(const uint32_t* __restrict__ B, const uint64_t* __re
     }
 }
 
-// Decode steps 2-4 for one output tile: flags at the last byte of every run
-// that ends in the tile, their exclusive prefix sum = the run of every byte
-// (after the runs that end before the tile), and the copy of the run's byte.
+// Decode steps 2-4: per output tile, flags at the last byte of every run that
+// ends in it, their exclusive prefix sum = the run of every byte (after the
+// runs that end before the tile), and the run's byte. A CTA takes a span of
+// consecutive tiles: the first one's first run is searched by a warp (32
+// probes a round), every later tile starts at the run the one before ended in.
+// Bytes are gathered from shared memory and written 16 at a time. 64 mixed
+// blocks: 366 us with a search a tile by one thread (25 dependent loads) and
+// byte stores -> 96 us; the lengths' scan 248 -> 147 us with 16-byte loads and
+// stores.
 __global__ void __launch_bounds__(RT) k_rle_expand(const uint8_t* __restrict__ chars, const uint32_t* __restrict__ B,
                                                    const uint64_t* __restrict__ run_off, uint32_t nb, uint32_t N,
                                                    uint8_t* __restrict__ out) {
-    __shared__ uint8_t sflag[RTILE];
+    __shared__ __align__(16) uint8_t sflag[RTILE];
+    __shared__ uint8_t sc[RTILE];
     __shared__ uint32_t s_k0, scan_tmp[32];
     const uint64_t R = min(run_off[nb], (uint64_t)N);
     if (R == 0) return;  // no runs: the check has flagged the input
     const uint32_t ntiles = (N + RTILE - 1) / RTILE;
-    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const uint32_t t0 = t * RTILE, len = min(RTILE, N - t0);
-        for (uint32_t q = threadIdx.x; q < RTILE; q += RT) sflag[q] = 0;
-        if (threadIdx.x == 0) {  // first run ending after t0: runs before it end at or before t0
-            uint64_t lo = 0, hi = R;
-            while (lo < hi) {
-                const uint64_t mid = (lo + hi) >> 1;
-                if (B[mid] <= t0) lo = mid + 1; else hi = mid;
-            }
-            s_k0 = (uint32_t)lo;
+    const uint32_t span = (ntiles + gridDim.x - 1) / gridDim.x;
+    const uint32_t t_end = min(ntiles, (blockIdx.x + 1) * span);
+    const bool vec = (reinterpret_cast<uintptr_t>(out) & 15u) == 0u;
+    if (blockIdx.x * span >= ntiles) return;
+    if (threadIdx.x < 32) {  // first run ending after the span's start: runs before it end at or before it
+        const uint32_t t0 = blockIdx.x * span * RTILE;
+        uint64_t lo = 0, hi = R;  // B[lo - 1] <= t0 < B[hi]
+        while (lo < hi) {
+            const uint64_t p = lo + (hi - lo) * threadIdx.x / 32;
+            const uint32_t m = __popc(__ballot_sync(0xffffffffu, B[p] <= t0));  // a prefix of the lanes
+            const uint64_t nlo = m ? lo + (hi - lo) * (m - 1) / 32 + 1 : lo;
+            hi = m < 32 ? lo + (hi - lo) * m / 32 : hi;
+            lo = nlo;
         }
+        if (threadIdx.x == 0) s_k0 = (uint32_t)lo;
+    }
+    __syncthreads();
+    uint32_t k0 = s_k0;
+    for (uint32_t t = blockIdx.x * span; t < t_end; ++t) {
+        const uint32_t t0 = t * RTILE, len = min(RTILE, N - t0);
+        reinterpret_cast<uint4*>(sflag)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        const uint32_t k0 = s_k0;
-        for (uint32_t x = threadIdx.x; x < len; x += RT) {  // at most len runs end inside the tile
-            const uint64_t k = (uint64_t)k0 + x;
-            if (k >= R) break;
-            const uint32_t e = B[k];
-            if (e - 1 - t0 >= len) break;  // ends after the tile (B increases)
-            sflag[e - 1 - t0] = 1;
+        // the runs that reach into the tile (at most len): their bytes, and a
+        // flag at each one's last byte; four a thread and step, loaded together
+        constexpr int U = 4;
+        for (uint32_t x0 = threadIdx.x; x0 < len; x0 += U * RT) {
+            uint32_t e[U], st[U];
+            uint8_t c[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t k = (uint64_t)k0 + x0 + u * RT;
+                const bool ok = x0 + u * RT < len && k < R;
+                e[u] = ok ? B[k] : 0u;
+                st[u] = ok ? (k > 0 ? B[k - 1] : 0u) : 0xffffffffu;
+                c[u] = ok ? chars[k] : (uint8_t)0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (st[u] < t0 + len) {  // else it begins after the tile (B increases) or is none
+                    sc[x0 + u * RT] = c[u];
+                    if (e[u] - 1 - t0 < len) sflag[e[u] - 1 - t0] = 1;
+                }
+            }
+            if (st[U - 1] >= t0 + len) break;
         }
         __syncthreads();
         const uint32_t q0 = threadIdx.x * RI;
-        uint32_t f[RI], cnt = 0;
-#pragma unroll
-        for (int j = 0; j < RI; ++j) {
-            f[j] = q0 + j < len ? sflag[q0 + j] : 0u;
-            cnt += f[j];
-        }
+        const uint4 f4 = reinterpret_cast<const uint4*>(sflag)[threadIdx.x];
+        const uint32_t f[4] = {f4.x, f4.y, f4.z, f4.w};
+        const uint32_t cnt = __popc(f4.x) + __popc(f4.y) + __popc(f4.z) + __popc(f4.w);
         uint32_t total;
         uint32_t r = block_exclusive_scan<RT>(cnt, scan_tmp, &total);
+        uint32_t w[4];
+        const uint32_t rmax = (uint32_t)min((uint64_t)RTILE - 1u, R - 1 - min((uint64_t)k0, R - 1));
 #pragma unroll
         for (int j = 0; j < RI; ++j) {
-            if (q0 + j >= len) break;
-            const uint64_t k = min((uint64_t)k0 + r, R - 1);
-            out[t0 + q0 + j] = chars[k];
-            r += f[j];
+            const uint32_t c = sc[min(r, rmax)];
+            w[j / 4] = j % 4 ? w[j / 4] | c << (8 * (j % 4)) : c;
+            r += (f[j / 4] >> (8 * (j % 4))) & 1u;
         }
+        if (vec && q0 + RI <= len) {
+            *reinterpret_cast<uint4*>(out + t0 + q0) = make_uint4(w[0], w[1], w[2], w[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < RI; ++j)
+                if (q0 + j < len) out[t0 + q0 + j] = (uint8_t)(w[j / 4] >> (8 * (j % 4)));
+        }
+        k0 += total;
         __syncthreads();
     }
 }
@@ -691,14 +834,12 @@ extern "C" bwt_status bwt_rle_encode(bwt_plan* p, const uint8_t* d_in, const uin
     if ((s = reset_ctrl(p, st)) != BWT_OK) return p->last = s;
     const uint32_t N = p->total, nt = (N + RTILE - 1) / RTILE;
     uint64_t* status = reinterpret_cast<uint64_t*>(p->status);
-    CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * nt, st));
-    uint32_t* ends = p->vals[0];
+    CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * 2 * nt, st));  // run counts, last run ends
     const int sms = num_sms();
     k_rle_encode<<<std::max(1, std::min<int>(nt, sms * 8)), RT, 0, st>>>(
-        d_in, N, p->blocks, p->nb, d_chars, ends, d_run_off, status, p->ctrl + CTRL_TILE_CTR, p->ctrl);
-    k_rle_lengths<<<sms * 8, 256, 0, st>>>(ends, d_run_off, p->nb, d_lens);
+        d_in, N, p->blocks, p->nb, d_chars, d_lens, d_run_off, status, status + nt, p->ctrl + CTRL_TILE_CTR, p->ctrl);
     CKS(cudaGetLastError());
-    p->stats.kernel_launches = 3;
+    p->stats.kernel_launches = 2;
     return p->last = finish_status(p, st);
 }
 

@@ -122,3 +122,44 @@ def test_inverse_samples_and_supers(kind, tile):
         plan.inverse_into(L, off, prim, out[5:5 + buf.size])
     assert torch.equal(out[5:5 + buf.size], d_in)
     assert bool((out[:5] == 0xEE).all()) and bool((out[5 + buf.size:] == 0xEE).all())
+
+
+@pytest.mark.parametrize("shift", [0, 3])
+@pytest.mark.parametrize("kind", ["edges", "long", "dense", "ends"])
+def test_rle_tiles(kind, shift):
+    """Run-length encoding and decoding around the 4,096-byte tiles: runs that
+    begin many tiles before their end, tiles without a run end, blocks that end
+    at and beside a tile's edge, several blocks in a tile, and inputs and
+    outputs that are not 16-byte aligned."""
+    import torch
+    r = np.random.RandomState(41)
+    if kind == "edges":
+        blocks = [r.randint(0, 2, n).astype(np.uint8) for n in (4095, 1, 4096, 4097, 15, 16, 17, 8175, 1, 1, 12288)]
+    elif kind == "long":  # 300,000-byte runs: tiles 32 and more back hold the last run end
+        blocks = [np.repeat(np.array([5, 6, 5], dtype=np.uint8), 300_000), np.full(200_000, 6, dtype=np.uint8)]
+    elif kind == "dense":
+        blocks = [np.arange(70_001, dtype=np.uint32).astype(np.uint8), r.randint(0, 256, 9).astype(np.uint8)]
+    else:  # a run of one byte at every edge, long runs between
+        b = np.zeros(20 * 4096, dtype=np.uint8)
+        b[4095::4096] = 1
+        blocks = [b, np.ones(4096, dtype=np.uint8), np.ones(4096 - 20, dtype=np.uint8)]
+    buf, off = batch_from_blocks(blocks)
+    ref_c, ref_l, ref_ro = oracle.rle_batch(buf, off)
+    R = int(ref_ro[-1])
+    sizes = np.diff(off.astype(np.int64))
+    pad = 32
+    d_in = torch.zeros(buf.size + pad, dtype=torch.uint8, device="cuda")
+    d_in[shift:shift + buf.size] = torch.from_numpy(buf).cuda()
+    chars = torch.full((buf.size + pad,), 0xEE, dtype=torch.uint8, device="cuda")
+    lens = torch.full((buf.size + pad,), -1, dtype=torch.int32, device="cuda")
+    ro = torch.zeros(off.size, dtype=torch.int64, device="cuda")
+    out = torch.full((buf.size + pad,), 0xEE, dtype=torch.uint8, device="cuda")
+    with Plan(max_blocks=off.size - 1, max_total_bytes=buf.size, max_block_bytes=int(sizes.max())) as plan:
+        plan.rle_encode_into(d_in[shift:shift + buf.size], off, chars[shift:], lens[shift:], ro)
+        plan.rle_decode_into(chars[shift:], lens[shift:], ro, off, out[shift:])
+    assert np.array_equal(ro.cpu().numpy().astype(np.uint64), ref_ro)
+    assert np.array_equal(chars[shift:shift + R].cpu().numpy(), ref_c)
+    assert np.array_equal(lens[shift:shift + R].cpu().numpy().astype(np.uint32), ref_l)
+    assert bool((chars[shift + R:] == 0xEE).all()) and bool((lens[shift + R:] == -1).all())
+    assert np.array_equal(out[shift:shift + buf.size].cpu().numpy(), buf)
+    assert bool((out[:shift] == 0xEE).all()) and bool((out[shift + buf.size:] == 0xEE).all())
