@@ -13,11 +13,11 @@ namespace bwt {
 
 // One radix tile: `len` consecutive keys at global position `start`, inside
 // segment `seg` (a block for the first sort, a group for a doubling round).
-// Tiles never straddle segments; a segment's tiles are consecutive and
-// `firstTile` is the index of its first one (where look-back stops).
+// Tiles never straddle segments; a segment's tiles are numbered consecutively
+// and `firstTile` is the number of its first one (where look-back stops).
 struct TileDesc {
     uint32_t start, len, seg, firstTile;
-    uint32_t segStart, blk, pad0, pad1;
+    uint32_t segStart, blk, pad0, index;  // pad0: keys of the segment; index: the tile's own number (its look-back row)
 };
 
 // A group of rotations whose sort keys are still equal: global positions

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(1024) k_build_large_tiles(Bins cur, int tile, 
                 td.segStart = g.start;
                 td.blk = g.blk;
                 td.pad0 = g.len;
-                td.pad1 = 0;
+                td.index = ti;
                 tiles[ti] = td;
             }
         }

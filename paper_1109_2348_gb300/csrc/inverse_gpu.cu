@@ -121,9 +121,9 @@ __global__ void __launch_bounds__(256, TILE >= 4096 ? 5 : 6) k_inv_sort(const ui
     for (;;) {
         if (tid == 0) s_tile = atomicAdd(counter, 1u);
         __syncthreads();
-        const uint32_t t = s_tile;
-        if (t >= num_tiles) break;
-        const TileDesc td = tiles[t];
+        if (s_tile >= num_tiles) break;
+        const TileDesc td = tiles[s_tile];
+        const uint32_t t = td.index;  // its look-back row: the table is interleaved
         const BlockInfo bi = blocks[td.blk];
         const uint32_t i0 = td.start - bi.off;
         const uint32_t shift = stage_tile_bytes(L, bi, i0, td.len, sb, tid, 256);
@@ -525,11 +525,11 @@ void launch_inv_sort(bwt_plan* p, const uint8_t* L, uint32_t* counter, PT* P, cu
     const uint32_t nt = p->ntiles0;
     const int sms = num_sms(), grid = std::max(1, std::min<int>((int)nt, sms * (p->tile >= 4096 ? 5 : 6)));
     if (p->tile == 1024)
-        k_inv_sort<PT, 1024><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles0, nt, p->hist, p->status, counter, p->ctrl, P);
+        k_inv_sort<PT, 1024><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles_il, nt, p->hist, p->status, counter, p->ctrl, P);
     else if (p->tile == 2048)
-        k_inv_sort<PT, 2048><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles0, nt, p->hist, p->status, counter, p->ctrl, P);
+        k_inv_sort<PT, 2048><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles_il, nt, p->hist, p->status, counter, p->ctrl, P);
     else
-        k_inv_sort<PT, 4096><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles0, nt, p->hist, p->status, counter, p->ctrl, P);
+        k_inv_sort<PT, 4096><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles_il, nt, p->hist, p->status, counter, p->ctrl, P);
 }
 
 }  // namespace

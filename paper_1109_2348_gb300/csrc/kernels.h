@@ -40,6 +40,14 @@ cudaError_t launch_onesweep(int key_bytes, bool from_s, int radix_bits, int tile
 int onesweep_grid(int key_bytes, bool from_s, int radix_bits, int tile);
 size_t onesweep_smem(int key_bytes, bool from_s, int radix_bits, int tile);
 
+// The first sort's tiles in the order the look-back passes take them: blocks
+// in groups of IL_BLOCKS, the tiles of a group's blocks in turn (tile 0 of
+// every block, tile 1 of every block, ...). out[k].index stays the tile's
+// number in `tiles`.
+constexpr uint32_t IL_BLOCKS = 128;
+cudaError_t launch_interleave_tiles(const TileDesc* tiles, uint32_t ntiles, const BlockInfo* blocks, uint32_t nb,
+                                    uint32_t tile, TileDesc* out, cudaStream_t st);
+
 // ---- 16-bit digits of the first sort (radix16.cu) ------------------------
 
 // Keys per part of a 16-bit pass: parts never straddle blocks, and a part's

@@ -1176,6 +1176,7 @@ __global__ void k_route_tiles(const TileDesc* __restrict__ tiles0, uint32_t ntil
         const uint32_t f = plain ? first[b] : first[nb + b];
         const uint32_t dst = f + (t - td.firstTile);
         td.firstTile = f;
+        td.index = dst;
         (plain ? tiles_p : tiles_b)[dst] = td;
     }
 }

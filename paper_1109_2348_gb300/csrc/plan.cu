@@ -125,7 +125,7 @@ void bwt::free_plan_memory(bwt_plan* p) {
         if (q) cudaFreeHost(q);
     };
     F(p->keys[0]); F(p->keys[1]); F(p->vals[0]); F(p->vals[1]); F(p->rank);
-    F(p->tiles0); F(p->ltiles); F(p->blocks); F(p->hist); F(p->status); F(p->ctrl); F(p->seg_varied);
+    F(p->tiles0); F(p->tiles_il); F(p->ltiles); F(p->blocks); F(p->hist); F(p->status); F(p->ctrl); F(p->seg_varied);
     for (int s = 0; s < 2; ++s)
         for (int c = 0; c < NCLS; ++c) F(p->bins[s][c]);
     F(p->parts16); F(p->part_first16); F(p->partcnt16); F(p->segtot16);
@@ -195,6 +195,7 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     A(dev_alloc(&p->vals[1], N, &total));
     A(dev_alloc(&p->rank, N, &total));
     A(dev_alloc(&p->tiles0, p->cap_tiles0, &total));
+    A(dev_alloc(&p->tiles_il, p->cap_tiles0, &total));
     A(dev_alloc(&p->ltiles, p->cap_ltiles, &total));
     A(dev_alloc(&p->blocks, B, &total));
     A(dev_alloc(&p->hist, p->cap_hist, &total));
@@ -402,7 +403,7 @@ bwt_status bwt::upload_tables(bwt_plan* p, const uint64_t* off, uint32_t nb, cud
             td.segStart = o;
             td.blk = b;
             td.pad0 = n;
-            td.pad1 = 0;
+            td.index = nt;
             p->h_tiles[nt++] = td;
         }
     }
@@ -412,6 +413,7 @@ bwt_status bwt::upload_tables(bwt_plan* p, const uint64_t* off, uint32_t nb, cud
     p->ntiles0 = nt;
     CK(cudaMemcpyAsync(p->blocks, p->h_blocks, sizeof(BlockInfo) * nb, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(p->tiles0, p->h_tiles, sizeof(TileDesc) * nt, cudaMemcpyHostToDevice, st));
+    CK(launch_interleave_tiles(p->tiles0, nt, p->blocks, nb, T, p->tiles_il, st));
     p->nparts = 0;
     if (p->rbits == 16) {
         // parts of the 16-bit passes: up to PART16_KEYS consecutive rotations of one block
@@ -550,7 +552,7 @@ bwt_status bwt::enqueue_initial_sort(bwt_plan* p, const uint8_t* d_in, cudaStrea
         a.vout = p->vals[ps & 1];
         a.S = d_in;
         a.blocks = p->blocks;
-        a.tiles = p->tiles0;
+        a.tiles = p->tiles_il;
         a.num_tiles = ctrl + CTRL_NTILES0;
         a.seg_base = p->hist + (rb == 8 ? 0 : ps * 2048);
         a.seg_base_stride = seg_stride;

@@ -92,6 +92,7 @@ struct bwt_plan {
     uint32_t* vals[2] = {nullptr, nullptr};
     uint32_t* rank = nullptr;
     bwt::TileDesc* tiles0 = nullptr;
+    bwt::TileDesc* tiles_il = nullptr;  // the same tiles, interleaved for the look-back passes
     bwt::TileDesc* ltiles = nullptr;
     bwt::BlockInfo* blocks = nullptr;
     uint32_t* hist = nullptr;

@@ -495,9 +495,10 @@ __global__ void __launch_bounds__(RT) k_vle_pack(const uint8_t* __restrict__ S, 
     const uint32_t spin = ctrl[CTRL_SPIN], withhold = ctrl[CTRL_WITHHOLD];
     if (ld_volatile(&ctrl[CTRL_ERR]) & (ERR_INPUT | ERR_CAPACITY)) return;  // bad table or too small a buffer
     for (;;) {
-        const uint32_t t = next_tile(&s_tile, counter);
-        if (t >= ntiles) break;
-        const TileDesc td = tiles[t];
+        const uint32_t at = next_tile(&s_tile, counter);
+        if (at >= ntiles) break;
+        const TileDesc td = tiles[at];
+        const uint32_t t = td.index;  // its look-back row: the table is interleaved
         const uint32_t q0 = threadIdx.x * RI;
         uint32_t lsum = 0;
         uint32_t c[RI];
@@ -899,7 +900,7 @@ extern "C" bwt_status bwt_vle_encode(bwt_plan* p, const uint8_t* d_in, const uin
     uint64_t* status = reinterpret_cast<uint64_t*>(p->status);
     CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * nt, st));
     k_vle_pack<<<std::max(1, std::min<int>(nt, sms * 6)), RT, VLE_WORDS * 4 + 256 * 5, st>>>(
-        d_in, p->tiles0, nt, d_code, d_len, d_byte_off, cap_words, reinterpret_cast<uint32_t*>(d_out), status,
+        d_in, p->tiles_il, nt, d_code, d_len, d_byte_off, cap_words, reinterpret_cast<uint32_t*>(d_out), status,
         p->ctrl + CTRL_TILE_CTR, p->ctrl);
     CKS(cudaGetLastError());
     p->stats.kernel_launches = 5;

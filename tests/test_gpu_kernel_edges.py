@@ -163,3 +163,20 @@ def test_rle_tiles(kind, shift):
     assert bool((chars[shift + R:] == 0xEE).all()) and bool((lens[shift + R:] == -1).all())
     assert np.array_equal(out[shift:shift + buf.size].cpu().numpy(), buf)
     assert bool((out[:shift] == 0xEE).all()) and bool((out[shift + buf.size:] == 0xEE).all())
+
+
+@pytest.mark.parametrize("tile", [1024, 4096])
+@pytest.mark.parametrize("flags", [0, F_GRAPH])
+def test_interleaved_tiles(tile, flags):
+    """The radix passes take the tiles of 128 blocks in turn: more blocks than
+    one group, with no two neighbours of the same number of tiles, and a plan
+    whose layout changes between calls."""
+    r = np.random.RandomState(51)
+    sizes = [int(n) for n in np.concatenate([r.randint(1, 30_000, 140), [1, 4096, 4097, 60_000], r.randint(1, 9, 120)])]
+    blocks = [r.randint(0, 256, n).astype(np.uint8) for n in sizes]
+    with Plan(max_blocks=len(blocks), max_total_bytes=sum(sizes), max_block_bytes=max(sizes), tile_keys=tile,
+              flags=flags) as plan:
+        for part in (blocks, blocks[100:150], blocks[::-1], blocks[:1]):
+            buf, off = batch_from_blocks(part)
+            L, prim, _ = gpu_bwt(buf, off, plan)
+            assert_matches_oracle(buf, off, L, prim, f"{len(part)} blocks")
