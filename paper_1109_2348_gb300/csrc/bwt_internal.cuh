@@ -47,6 +47,10 @@ constexpr uint32_t ERR_BOUNDS = 8u; // a bounds check of the debug build failed 
 // (LazyRanks below). Readers of SA mask the bit.
 constexpr uint32_t SA_FINAL = 0x80000000u;
 
+// Marks of the rows whose bytes of L the gather writes after a learned first
+// stage: bit (pos >> 7) & 31 of word pos >> 12.
+constexpr uint32_t LG_ROW_SHIFT = 7, LG_WORD_SHIFT = LG_ROW_SHIFT + 5;
+
 // Bounds checks of the debug build (-DBWT_DEBUG): index < n for every
 // SA-derived index, destinations inside their segment. A failed check sets
 // ERR_BOUNDS in the error word *err (the call then returns BWT_EINTERNAL) and
@@ -111,12 +115,12 @@ struct Bins {
 // bucket's rows (already sorted). A row marked SA_FINAL is the rotation's
 // rank; otherwise the rotation is a group member with its rank stored.
 constexpr int LR_BUCKETS = 4096;  // learned buckets (the library's BWT_BUCKETS)
-constexpr int IDX_BITS = 16;      // splitter index on a key's first two bytes
+constexpr int IDX_BITS = 15;      // splitter index on a key's first 15 bits (64 KB: two counting CTAs an SM)
 constexpr int IDX_CELLS = 1 << IDX_BITS;
 constexpr int IDX_WORDS = IDX_CELLS + 8;  // u16 entries (first[IDX_CELLS] = #splitters), padded to 16 bytes
 
-// Bucket of a key: #{j : spl[j] <= key}. first[c] = #{j : spl[j] < c << 48}
-// narrows the search to the splitters that share the key's first two bytes
+// Bucket of a key: #{j : spl[j] <= key}. first[c] = #{j : spl[j] < c << 49}
+// narrows the search to the splitters that share the key's first 15 bits
 // (the ones below all count, the ones above none).
 __device__ __forceinline__ uint32_t bucket_of(const uint64_t* spl, const uint16_t* first, uint64_t key) {
     const uint32_t c = (uint32_t)(key >> (64 - IDX_BITS));
@@ -135,7 +139,7 @@ struct LazyRanks {
     const uint32_t* route = nullptr;     // [block] 0 learned buckets, 2 equal-width buckets
     const uint32_t* starts = nullptr;    // [block][LR_BUCKETS] block-relative first row of every bucket
     const uint64_t* splitters = nullptr; // learned splitters
-    const uint16_t* index = nullptr;     // their two-byte-prefix index
+    const uint16_t* index = nullptr;     // their prefix index
     uint32_t own_cap = 0;                // largest bucket the chunk sorts name (larger: named in full)
 };
 

@@ -771,42 +771,81 @@ __global__ void __launch_bounds__(256) k_rename_large(const uint32_t* __restrict
 }
 
 // Tiles in order from an atomic counter (zeroed before the launch): the
-// blocks whose bytes are gathered stay few, so their S stays in L2.
+// blocks whose bytes are gathered stay few, so their S stays in L2. Bound by
+// the random byte reads (about 280 G/s, L2).
+//
+// MARKED (after a learned first stage): the chunk sorts have written
+// most of L and primary themselves: only plain-routed blocks and the marked
+// granules of the others are gathered. A CTA then takes `batch` tiles at a
+// time (up to 16, as long as every CTA has some) and looks at their marks
+// together.
+
+template <bool MARKED>
 __global__ void __launch_bounds__(256) k_gather_L(const uint8_t* __restrict__ S, const uint32_t* __restrict__ SA,
                                                   const BlockInfo* __restrict__ blocks,
                                                   const TileDesc* __restrict__ tiles, uint32_t num_tiles,
                                                   uint8_t* __restrict__ L, int32_t* __restrict__ primary,
-                                                  uint32_t* __restrict__ tile_counter, uint32_t* err) {
-    __shared__ uint32_t s_t;
+                                                  uint32_t* __restrict__ tile_counter, uint32_t* err,
+                                                  const uint32_t* __restrict__ route,
+                                                  const uint32_t* __restrict__ marks, uint32_t batch) {
+    __shared__ uint32_t s_t, s_need;
+    uint32_t need = 0, t0 = 0;  // tiles of the batch still to gather (bit k: tile t0 + k)
     for (;;) {
-        if (threadIdx.x == 0) s_t = atomicAdd(tile_counter, 1u);
-        __syncthreads();
-        const uint32_t t = s_t;
-        if (t >= num_tiles) break;
+        if (need == 0u) {
+            if (threadIdx.x == 0) s_t = atomicAdd(tile_counter, batch);
+            __syncthreads();
+            t0 = s_t;
+            if (t0 >= num_tiles) break;
+            if (MARKED && threadIdx.x < 32) {
+                const uint32_t t = t0 + threadIdx.x;
+                bool mine = threadIdx.x < batch && t < num_tiles;
+                if (mine) {
+                    const TileDesc td = tiles[t];
+                    if (route[td.blk] != 1u) {
+                        // a tile holds at most 4,096 rows: two words at most
+                        mine = (marks[td.start >> LG_WORD_SHIFT] | marks[(td.start + td.len - 1) >> LG_WORD_SHIFT]) != 0u;
+                    }
+                }
+                const uint32_t m = __ballot_sync(0xffffffffu, mine);
+                if (threadIdx.x == 0) s_need = m;
+            }
+            if constexpr (MARKED) {
+                __syncthreads();
+                need = s_need;
+                if (need == 0u) continue;
+            } else {
+                need = 1u;
+            }
+        }
+        const uint32_t t = t0 + __ffs(need) - 1;
+        need &= need - 1;
         const TileDesc td = tiles[t];
         const BlockInfo bi = blocks[td.blk];
+        const bool all = !MARKED || route[td.blk] == 1u;
         // four elements a thread per step: their SA loads, then their byte
         // gathers, are all in flight at once
         constexpr int PI = 4;
         for (uint32_t q0 = 0; q0 < td.len; q0 += 256u * PI) {
             uint32_t sa[PI];
             uint8_t c[PI];
+            bool want[PI];
 #pragma unroll
             for (int j = 0; j < PI; ++j) {
-                const uint32_t q = q0 + j * 256u + threadIdx.x;
-                sa[j] = q < td.len ? SA[td.start + q] : 1u;
+                const uint32_t q = q0 + j * 256u + threadIdx.x, pos = td.start + q;
+                want[j] = q < td.len && (all || (marks[pos >> LG_WORD_SHIFT] >> ((pos >> LG_ROW_SHIFT) & 31u)) & 1u);
+                sa[j] = want[j] ? SA[pos] : 1u;
             }
 #pragma unroll
             for (int j = 0; j < PI; ++j) {
                 sa[j] &= ~SA_FINAL;
-                BWT_DCHECK(q0 + j * 256u + threadIdx.x >= td.len || sa[j] < bi.n, err);
+                BWT_DCHECK(!want[j] || sa[j] < bi.n, err);
                 const uint32_t src = sa[j] == 0 || sa[j] > bi.n ? bi.n - 1 : sa[j] - 1;
-                c[j] = S[bi.off + src];
+                c[j] = want[j] ? S[bi.off + src] : (uint8_t)0;
             }
 #pragma unroll
             for (int j = 0; j < PI; ++j) {
                 const uint32_t q = q0 + j * 256u + threadIdx.x;
-                if (q < td.len) {
+                if (want[j]) {
                     L[td.start + q] = c[j];
                     if (sa[j] == 0) primary[td.blk] = (int32_t)q + (int32_t)(td.start - bi.off);
                 }
@@ -916,7 +955,7 @@ cudaError_t launch_large_prologue(const uint32_t* SA, const uint32_t* rank, cons
 
 cudaError_t launch_sort_small(uint32_t* SA, uint32_t* key2, uint32_t* rank, const BlockInfo* blocks, Bins cur,
                               Bins next, const uint32_t* depth, const uint32_t* host_counts, uint32_t* ctrl,
-                              cudaStream_t st, int* launched) {
+                              cudaStream_t st, cudaStream_t med, int* launched) {
     int g[4] = {num_sms() * 8, num_sms() * 16, num_sms() * 8, num_sms() * 8};
     if (host_counts) {
         g[0] = host_counts[0] ? grid_for(host_counts[0], 256, 8) : 0;
@@ -938,7 +977,7 @@ cudaError_t launch_sort_small(uint32_t* SA, uint32_t* key2, uint32_t* rank, cons
         ++*launched;
     }
     if (g[3]) {
-        k_sort_med<<<g[3], 256, 0, st>>>(SA, key2, rank, blocks, cur, next, depth, ctrl);
+        k_sort_med<<<g[3], 256, 0, med>>>(SA, key2, rank, blocks, cur, next, depth, ctrl);
         ++*launched;
     }
     return cudaGetLastError();
@@ -953,12 +992,19 @@ cudaError_t launch_rename_large(const uint32_t* SA, const uint32_t* key2, uint32
 }
 
 cudaError_t launch_gather_L(const uint8_t* S, const uint32_t* SA, const BlockInfo* blocks, const TileDesc* tiles,
-                            uint32_t num_tiles, uint8_t* L, int32_t* primary, uint32_t* ctrl, cudaStream_t st) {
+                            uint32_t num_tiles, uint8_t* L, int32_t* primary, uint32_t* ctrl, cudaStream_t st,
+                            const uint32_t* route, const uint32_t* marks) {
     if (!num_tiles) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(ctrl + GATHER_L_CTR, 0, 4, st);
     if (e != cudaSuccess) return e;
-    k_gather_L<<<grid_for(num_tiles, 1, 16), 256, 0, st>>>(S, SA, blocks, tiles, num_tiles, L, primary,
-                                                           ctrl + GATHER_L_CTR, ctrl + CTRL_ERR);
+    const uint32_t batch = route ? std::max(1u, std::min(16u, num_tiles / ((uint32_t)num_sms() * 16u))) : 1u;
+    const int grid = grid_for(num_tiles, batch, 16);
+    if (route)
+        k_gather_L<true><<<grid, 256, 0, st>>>(S, SA, blocks, tiles, num_tiles, L, primary, ctrl + GATHER_L_CTR,
+                                               ctrl + CTRL_ERR, route, marks, batch);
+    else
+        k_gather_L<false><<<grid, 256, 0, st>>>(S, SA, blocks, tiles, num_tiles, L, primary, ctrl + GATHER_L_CTR,
+                                                ctrl + CTRL_ERR, nullptr, nullptr, 1u);
     return cudaGetLastError();
 }
 
@@ -996,6 +1042,7 @@ __global__ void k_round_end(uint32_t* ctrl, int par, uint32_t max_n, cudaGraphCo
         ctrl[CTRL_DEPTH] *= 2u;
         ctrl[CTRL_ROUNDS] += 1u;
     }
+    for (int i = 0; i < NCLS; ++i) ctrl[CTRL_BINS + NCLS * par + i] = 0u;  // the bins the next round fills
     if (flags & 4) ctrl[CTRL_BODY_ITERS] += 1u;
     if (flags & 3) {
         const bool more = any_groups(nxt) && ctrl[CTRL_DEPTH] < max_n && ctrl[CTRL_ROUNDS] < 40u &&

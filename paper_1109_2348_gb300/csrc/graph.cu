@@ -100,8 +100,9 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     }
 
     bwt_status status = BWT_OK;
-    // capture streams: the main graph, the loop body, the body's second round
-    cudaStream_t cs = nullptr, bs = nullptr, rs = nullptr;
+    // capture streams: the main graph, the loop body, the body's second round,
+    // and two branches of each
+    cudaStream_t cs = nullptr, bs = nullptr, rs = nullptr, br[6] = {};
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t launched = nullptr;
@@ -117,6 +118,7 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     CKG(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     CKG(cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking));
     CKG(cudaStreamCreateWithFlags(&rs, cudaStreamNonBlocking));
+    for (auto& s : br) CKG(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     CKG(cudaGraphCreate(&g, 0));
     CKG(cudaGraphConditionalHandleCreate(&cond, g, 0, 0));
     p->capturing = true;
@@ -124,7 +126,9 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     k0 = p->stats.kernel_launches;
     r0 = p->stats.radix_launches;
     CKS(reset_ctrl(p, cs));
-    if (learned) CKS(enqueue_learned(p, d_in, cs));
+    p->br[0] = br[4];
+    p->br[1] = br[5];
+    if (learned) CKS(enqueue_learned(p, d_in, d_L, d_primary, cs));
     else CKS(enqueue_initial_sort(p, d_in, cs));
     CKG(launch_set_cond_initial(p->ctrl, p->max_n, cond, cs));
     p->stats.kernel_launches++;
@@ -140,12 +144,16 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     // loop body: a round on bins[0]; then, if another round is due, a round
     // on bins[1] (an IF node, so a finished batch skips it)
     CKG(cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    p->br[0] = br[0];
+    p->br[1] = br[1];
     CKS(enqueue_round(p, 0, nullptr, bs));
     CKG(cudaGraphConditionalHandleCreate(&cond_r1, body, 0, 0));
     CKG(launch_round_end(p->ctrl, 0, p->max_n, cond, cond_r1, 1 | 2 | 4, bs));
     p->stats.kernel_launches++;
     k2 = p->stats.kernel_launches;
     CKS(begin_if_capture(bs, rs, cond_r1));
+    p->br[0] = br[2];
+    p->br[1] = br[3];
     CKS(enqueue_round(p, 1, nullptr, rs));
     CKG(launch_round_end(p->ctrl, 1, p->max_n, cond, 0, 1 | 4, rs));
     p->stats.kernel_launches++;
@@ -155,19 +163,25 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     r3 = p->stats.radix_launches;
     {
         NvtxRange nv("gather");
-        CKG(launch_gather_L(d_in, p->sa, p->blocks, p->tiles0, p->ntiles0, d_L, d_primary, p->ctrl, cs));
+        CKG(launch_gather_L(d_in, p->sa, p->blocks, p->tiles0, p->ntiles0, d_L, d_primary, p->ctrl, cs,
+                            learned ? p->route : nullptr, learned ? p->lgather : nullptr));
     }
     p->stats.kernel_launches++;
     k4 = p->stats.kernel_launches;
     r4 = p->stats.radix_launches;
     CKG(cudaStreamEndCapture(cs, &g));
     p->capturing = false;
+    p->br[0] = p->br[1] = nullptr;
     CKG(cudaGraphInstantiate(&exec, g, 0));
     CKG(cudaEventCreateWithFlags(&launched, cudaEventDisableTiming));
     cudaStreamDestroy(cs);
     cudaStreamDestroy(bs);
     cudaStreamDestroy(rs);
     cs = bs = rs = nullptr;
+    for (auto& s : br) {
+        cudaStreamDestroy(s);
+        s = nullptr;
+    }
     {
         // the least recently used graph makes room (its last launch may still run)
         if (p->graphs.size() >= kGraphCache) {
@@ -201,12 +215,15 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
 
 fail:
     p->capturing = false;
+    p->br[0] = p->br[1] = nullptr;
     for (cudaStream_t s : {rs, bs, cs}) {  // innermost captures first
         if (!s) continue;
         cudaGraph_t t = nullptr;
         cudaStreamEndCapture(s, &t);
         cudaStreamDestroy(s);
     }
+    for (cudaStream_t s : br)  // their captures ended with the streams they branched from
+        if (s) cudaStreamDestroy(s);
     if (launched) cudaEventDestroy(launched);
     if (exec) cudaGraphExecDestroy(exec);
     if (g) cudaGraphDestroy(g);

@@ -23,7 +23,8 @@ struct OneSweepParams {
     const uint32_t* num_tiles;    // device count of tiles
     const uint32_t* seg_base;     // per segment, per digit: exclusive digit offset in the segment
     uint32_t seg_base_stride;     // words between consecutive segments' rows
-    uint32_t* status;             // [tile][radix] look-back words, zeroed before the pass
+    uint32_t* status;             // look-back words, zeroed before the pass: tile t's at t * status_stride
+    uint32_t status_stride;       // words between consecutive tiles' (radix, or radix * passes cleared together)
     uint32_t* tile_counter;       // zeroed before the pass
     uint32_t* ctrl;               // device control words (spin limit, error)
     int shift;                    // digit = (key >> shift) & (radix - 1)
@@ -89,9 +90,20 @@ cudaError_t launch_hist_keys11(const uint8_t* S, const BlockInfo* blocks, const 
 cudaError_t launch_scan_rows(uint32_t* hist, int radix, const uint32_t* num_rows_dev, uint32_t rows_mult,
                              uint32_t rows_host, uint32_t max_rows, cudaStream_t st);
 
-// Zero count * words_per_unit words (count read on the device).
-cudaError_t launch_zero_by_count(uint32_t* p, const uint32_t* count, uint32_t words_per_unit, uint32_t max_words,
-                                 cudaStream_t st);
+// Words to clear: [p, p + *count * per), at most `max` (count null: none).
+struct ZeroRange {
+    uint32_t* p = nullptr;
+    const uint32_t* count = nullptr;
+    uint32_t per = 0;
+    uint64_t max = 0;
+    __device__ uint64_t words() const {
+        const uint64_t n = count ? (uint64_t)(*count) * per : 0ull;
+        return n < max ? n : max;
+    }
+};
+
+// Clears two counted ranges and c[0, nc) (nc <= 256) in one launch.
+cudaError_t launch_zero_by_count(ZeroRange a, ZeroRange b, uint32_t* c, uint32_t nc, cudaStream_t st);
 
 // ---- naming, doubling rounds, L gather (doubling.cu) --------------------
 
@@ -137,7 +149,7 @@ cudaError_t launch_large_prologue(const uint32_t* SA, const uint32_t* rank, cons
 // refined groups.
 cudaError_t launch_sort_small(uint32_t* SA, uint32_t* key2, uint32_t* rank, const BlockInfo* blocks, Bins cur,
                               Bins next, const uint32_t* depth, const uint32_t* host_counts, uint32_t* ctrl,
-                              cudaStream_t st, int* launched);
+                              cudaStream_t st, cudaStream_t med, int* launched);
 
 // Large groups after their radix sort: rename and emit refined groups; a
 // group with seg_varied[group] == 0 (all key2 equal, skipped by the radix)
@@ -164,9 +176,12 @@ cudaError_t launch_set_cond_initial(const uint32_t* ctrl, uint32_t max_n, cudaGr
                                     cudaStream_t st);
 
 // L[k] = S[(SA[k] + n - 1) mod n]; primary[b] = the k with SA[k] = 0.
-// ctrl: its tile-counter word for the gather is zeroed and used.
+// ctrl: its tile-counter word for the gather is zeroed and used. route, marks
+// (after a learned first stage, else null): only the tiles of plain-routed
+// blocks and the marked granules of the others (LG_ROW_SHIFT).
 cudaError_t launch_gather_L(const uint8_t* S, const uint32_t* SA, const BlockInfo* blocks, const TileDesc* tiles,
-                            uint32_t num_tiles, uint8_t* L, int32_t* primary, uint32_t* ctrl, cudaStream_t st);
+                            uint32_t num_tiles, uint8_t* L, int32_t* primary, uint32_t* ctrl, cudaStream_t st,
+                            const uint32_t* route = nullptr, const uint32_t* marks = nullptr);
 
 int num_sms();
 

@@ -163,7 +163,7 @@ extern "C" bwt_status bwt_model_samples(bwt_plan* p, const uint8_t* d_in, const 
 //
 //   count:   bucket b(i) = #{j : splitter[j] <= K_i} of every rotation, counted
 //            per block (a search of the splitters in shared memory from an
-//            index on the key's first two bytes), the bucket stored per
+//            index on the key's first 15 bits), the bucket stored per
 //            rotation;
 //   route:   a block whose over-capacity buckets hold more than a quarter of
 //            its rotations is counted again with equal-width buckets (the top
@@ -189,11 +189,10 @@ namespace {
 constexpr int NBK = BWT_BUCKETS;
 constexpr int NSP = BWT_SPLITTERS;
 
-// The splitter search (bucket_of) starts from an index on the key's first
-// two bytes: text keys use a few thousand of the 65,536 two-byte prefixes
-// and the splitters spread over them, so a search takes one or two steps
-// (five or six with an index on the top 12 bits, whose bank conflicts bound
-// the counting kernel).
+// The splitter search (bucket_of) starts from an index on the key's first 15
+// bits: text keys use a few thousand of the cells and the splitters spread
+// over them, so a search takes one to three steps (five or six with an index
+// on the top 12 bits, whose bank conflicts bounded the counting kernel).
 static_assert(NBK == LR_BUCKETS, "the lazy rank lookup indexes bucket starts by learned bucket");
 
 // The index of a splitter table (built once when the table is installed).
@@ -223,11 +222,15 @@ __device__ __forceinline__ void load_splitters(const uint64_t* __restrict__ spli
     __syncthreads();
 }
 
-constexpr size_t SPL_BYTES = 4096 * 8 + IDX_WORDS * 2;  // splitters + two-byte-prefix index
-constexpr size_t CNT_BYTES = 4096 * 4;
+constexpr size_t SPL_BYTES = 4096 * 8 + IDX_WORDS * 2;  // splitters + prefix index
+constexpr size_t CNT_BYTES = 4096 * 2;
 constexpr size_t TILE_BYTES = 4096 + 48;
 constexpr size_t COUNT_SMEM = SPL_BYTES + CNT_BYTES + TILE_BYTES;
-constexpr int COUNT_THREADS = 1024;  // one CTA an SM: its shared memory holds the splitters and the index
+// Two CTAs an SM: an index on 15 key bits, 16-bit counts and 512 threads make
+// room for both (one CTA of 1,024 threads with a 16-bit index: 728 us per 240
+// blocks of 900,000 bytes; two of 512: 662; two of 768 or 1,024 threads, which
+// leave 32 registers: 690 and 720).
+constexpr int COUNT_THREADS = 512;
 
 // Counts every rotation's bucket. FLAT = false: the learned bucketing of
 // every block, storing each rotation's learned bucket in fb (u16 per
@@ -235,23 +238,24 @@ constexpr int COUNT_THREADS = 1024;  // one CTA an SM: its shared memory holds t
 // 12 key bits) of the blocks marked in `need` only (those the learned
 // buckets do not fit). Text keys crowd a few of the equal-width buckets, so
 // their shared-memory atomics conflict: counting them only where the routing
-// needs them keeps them off the common path. Counts gather in one shared-
-// memory word per bucket (learned in the low half, equal-width in the high
-// half), so a CTA counts at most 65535 rotations (`span` tiles) before it
+// needs them keeps them off the common path. Counts gather in 16 bits a bucket
+// (bucket b in the low half of word b, b + 2,048 in its high half), so a CTA
+// counts at most 65535 rotations (`span` tiles) before it
 // adds them to the block's rows: one global atomic per non-empty bucket and
 // span; a span that crosses into the next block flushes at the boundary.
 // counts: [2][block][4096] (learned rows, then equal-width rows).
-__device__ __forceinline__ void flush_counts(uint32_t* h, uint32_t* __restrict__ counts, uint32_t nb, uint32_t blk) {
-    for (int i = threadIdx.x; i < NBK; i += blockDim.x) {
+__device__ __forceinline__ void flush_counts(uint32_t* h, uint32_t* __restrict__ counts, uint32_t nb, uint32_t blk, bool flat) {
+    for (int i = threadIdx.x; i < NBK / 2; i += blockDim.x) {
         const uint32_t c = h[i];
         h[i] = 0;
-        if (c & 0xffffu) atomicAdd(&counts[(size_t)blk * NBK + i], c & 0xffffu);
-        if (c >> 16) atomicAdd(&counts[((size_t)nb + blk) * NBK + i], c >> 16);
+        uint32_t* row = counts + ((size_t)(flat ? nb : 0u) + blk) * NBK;
+        if (c & 0xffffu) atomicAdd(&row[i], c & 0xffffu);
+        if (c >> 16) atomicAdd(&row[i + NBK / 2], c >> 16);
     }
 }
 
 template <bool FLAT>
-__global__ void __launch_bounds__(COUNT_THREADS, 1) k_bucket_count(const uint8_t* __restrict__ S,
+__global__ void __launch_bounds__(COUNT_THREADS, 2) k_bucket_count(const uint8_t* __restrict__ S,
                                                                     const BlockInfo* __restrict__ blocks,
                                                                     const TileDesc* __restrict__ tiles,
                                                                     uint32_t ntiles, uint32_t span,
@@ -266,7 +270,7 @@ __global__ void __launch_bounds__(COUNT_THREADS, 1) k_bucket_count(const uint8_t
     uint32_t* h = reinterpret_cast<uint32_t*>(smem + SPL_BYTES);
     uint8_t* sb = smem + SPL_BYTES + CNT_BYTES;
     if (!FLAT) load_splitters(splitters, index, spl, first);
-    for (int i = threadIdx.x; i < NBK; i += blockDim.x) h[i] = 0;
+    for (int i = threadIdx.x; i < NBK / 2; i += blockDim.x) h[i] = 0;
     __syncthreads();
     const uint32_t nspan = (ntiles + span - 1) / span;
     // One CTA an SM, so nothing else hides a tile's load: the next tile's
@@ -307,7 +311,7 @@ __global__ void __launch_bounds__(COUNT_THREADS, 1) k_bucket_count(const uint8_t
         for (uint32_t t = t0; t < t1; ++t) {
             const TileDesc td = tiles[t];
             if (td.blk != cur) {  // CTA-uniform; the histogram is complete (synced after the last tile)
-                flush_counts(h, counts, nb, cur);
+                flush_counts(h, counts, nb, cur, FLAT);
                 cur = td.blk;
             }
             if (FLAT && need[td.blk] == 0u) {  // CTA-uniform: a block the learned buckets fit
@@ -327,16 +331,17 @@ __global__ void __launch_bounds__(COUNT_THREADS, 1) k_bucket_count(const uint8_t
             for (uint32_t q = threadIdx.x; q < td.len; q += blockDim.x) {
                 const uint64_t key = pack8_smem(sb, shift + q);
                 if (FLAT) {
-                    atomicAdd(&h[(uint32_t)(key >> 52)], 1u << 16);
+                    const uint32_t b = (uint32_t)(key >> 52);
+                    atomicAdd(&h[b & (NBK / 2 - 1)], b < NBK / 2 ? 1u : 1u << 16);
                 } else {
                     const uint32_t b = bucket_of(spl, first, key);
                     fb[td.start + q] = (uint16_t)b;
-                    atomicAdd(&h[b], 1u);
+                    atomicAdd(&h[b & (NBK / 2 - 1)], b < NBK / 2 ? 1u : 1u << 16);
                 }
             }
             __syncthreads();
         }
-        flush_counts(h, counts, nb, cur);
+        flush_counts(h, counts, nb, cur, FLAT);
         __syncthreads();
     }
 }
@@ -419,16 +424,51 @@ __host__ __device__ constexpr uint32_t padded(uint32_t s) { return (s + MS_IT - 
 constexpr uint16_t CM_OWN = 0x8000;
 constexpr uint32_t TAG_SHIFT = 24, IDX_MASK = (1u << TAG_SHIFT) - 1u;
 
+// The keys buckets [b0, b0 + nbk) of a block may hold: learned buckets by the
+// splitters, equal-width ones (flat) by their top 12 bits.
+__device__ __forceinline__ void chunk_keys(bool flat, const uint64_t* __restrict__ splitters, uint32_t b0, uint32_t nbk,
+                                           uint64_t& first, uint64_t& last) {
+    const uint32_t b1 = min(b0 + nbk, (uint32_t)NBK);  // one past the last bucket
+    if (flat) {
+        first = (uint64_t)b0 << 52;
+        last = ((uint64_t)b1 << 52) - 1ull;  // b1 = 4096: 2^64 - 1
+    } else {
+        first = b0 > 0 ? splitters[b0 - 1] : 0ull;
+        last = b1 < (uint32_t)NBK ? splitters[b1 - 1] - 1ull : ~0ull;
+    }
+}
+
+// A chunk whose keys differ in their low 56 bits alone (modulo 2^56 they keep
+// their order above the first) is written with the byte before each rotation
+// -- its byte of L -- in the place of the key's top byte: key << 8 | byte. Its
+// sort then writes L itself (a byte a row in order, instead of one random read
+// a row by the L gather), and the gather is left the rows of groups. The chunks
+// of wider ranges (CB_WIDE in their start) and the buckets sorted by the
+// overflow radix keep whole keys; a wide chunk's sort reads the bytes from S.
+// Measured per 240 blocks of 900,000 bytes: the gather 767 -> 28 us, for
+// 1,151 -> 1,278 us in the scatter and 2,614 -> 2,735 us in the chunk sort; the
+// call 5,690 -> 5,234 us.
+constexpr uint64_t KEY56 = (1ull << 56) - 1ull;
+__device__ __forceinline__ bool wide_keys(uint64_t first, uint64_t last) { return (last - first) > KEY56; }
+constexpr uint32_t CB_WIDE = 0x80000000u;
+
+// Rows whose bytes of L the gather has to write, in granules of 128 global
+// positions: a bit each, 32 to a word, zeroed before the chunk plan.
+__device__ __forceinline__ void mark_lgather(uint32_t* __restrict__ marks, uint32_t pos) {
+    atomicOr(&marks[pos >> LG_WORD_SHIFT], 1u << ((pos >> LG_ROW_SHIFT) & 31u));
+}
+
 struct ChunkTables {
     uint16_t* cmap;        // [block][4096] chunk of each fine bucket (| CM_OWN: a bucket sorted on its own)
-    uint32_t* cbase;       // [block][MAXCH] block-relative start of each chunk
+    uint32_t* cbase;       // [block][MAXCH] block-relative start of each chunk (| CB_WIDE)
     uint32_t* ccur;        // [block][MAXCH] slots taken by the scatter
 };
 
 __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__ starts,
                                                     const BlockInfo* __restrict__ blocks,
-                                                    const uint32_t* __restrict__ route, uint32_t nb, ChunkTables ct,
-                                                    Bins out, uint32_t* ctrl) {
+                                                    const uint32_t* __restrict__ route,
+                                                    const uint64_t* __restrict__ splitters, uint32_t nb, ChunkTables ct,
+                                                    Bins out, uint32_t* __restrict__ lgather, uint32_t* ctrl) {
     __shared__ uint32_t st[NBK + 1];
     __shared__ uint16_t cm[NBK];
     __shared__ uint32_t cb[MAXCH];
@@ -452,8 +492,9 @@ __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__
                 if (len > 0) {
                     if (lane == 0 && nch < MAXCH) {
                         cb[nch] = cstart;
-                        // pad: the chunk's first fine bucket and its number of buckets
-                        chunks[nemit] = GroupDesc{bi.off + cstart, len, blk, cb0 | (nbo << 16)};
+                        // pad: the chunk's first fine bucket and its number of buckets;
+                        // blk: the chunk's number, until it is emitted
+                        chunks[nemit] = GroupDesc{bi.off + cstart, len, nch, cb0 | (nbo << 16)};
                     }
                     if (nch < MAXCH) ++nemit;
                     ++nch;
@@ -469,9 +510,15 @@ __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__
                     close();
                     if (lane == 0) {
                         cm[b] = (uint16_t)(min(nch, MAXCH - 1) | CM_OWN);
-                        if (nch < MAXCH) cb[nch] = st[b];
                         // the 512- or 1,024-thread sort, else the overflow radix
                         const int li = sz <= MID_CAP ? 2 : sz <= BIG_CAP ? 1 : CLS_LARGE;
+                        uint64_t k0, k1;
+                        chunk_keys(route[blk] == 2u, splitters, b, 1u, k0, k1);
+                        if (nch < MAXCH) cb[nch] = st[b] | (li == CLS_LARGE || wide_keys(k0, k1) ? CB_WIDE : 0u);
+                        if (li == CLS_LARGE)  // its sort does not write L
+                            for (uint32_t g = (bi.off + st[b]) >> LG_ROW_SHIFT;
+                                 g <= (bi.off + st[b] + sz - 1) >> LG_ROW_SHIFT; ++g)
+                                mark_lgather(lgather, g << LG_ROW_SHIFT);
                         const uint32_t slot = atomicAdd(&out.count[li], 1u);
                         if (slot < out.cap[li]) out.list[li][slot] = GroupDesc{bi.off + st[b], sz, blk, b | (1u << 16)};
                         else atomicOr(&ctrl[CTRL_ERR], ERR_CAPACITY);
@@ -517,6 +564,13 @@ __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__
             }
         }
         __syncthreads();
+        for (uint32_t i = threadIdx.x; i < s_n[0]; i += blockDim.x) {
+            uint64_t k0, k1;
+            chunk_keys(route[blk] == 2u, splitters, chunks[i].pad & 0xffffu, chunks[i].pad >> 16, k0, k1);
+            if (wide_keys(k0, k1)) cb[chunks[i].blk] |= CB_WIDE;
+            chunks[i].blk = blk;
+        }
+        __syncthreads();
         for (int i = threadIdx.x; i < NBK; i += blockDim.x) ct.cmap[(size_t)blk * NBK + i] = cm[i];
         for (uint32_t i = threadIdx.x; i < MAXCH; i += blockDim.x) {
             ct.cbase[(size_t)blk * MAXCH + i] = cb[i];
@@ -560,6 +614,7 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
     uint32_t* dbase = pre + MAXCH;                                       // [MAXCH] destination of pre[c]
     uint32_t* stQC = dbase + MAXCH;  // [4096] by rank: tile position (low 16 bits) | fine bucket (high 16)
     __shared__ uint32_t scan_tmp[32];
+    __shared__ uint8_t s_before;  // the byte before the tile's first rotation
     const uint32_t ntiles = *ntiles_dev;
     const uint32_t span = max(1u, min(16u, ntiles / (gridDim.x * 4u)));
     const uint32_t nspan = (ntiles + span - 1) / span;
@@ -588,6 +643,7 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
                 }
             }
             const uint32_t shift = stage_tile_bytes(S, bi, i0, td.len, sb, threadIdx.x, 256);
+            if (threadIdx.x == 0) s_before = S[bi.off + (i0 ? i0 : bi.n) - 1];
             __syncthreads();
             // chunk (low 10 bits) | slot within the tile's share of the chunk << 10;
             // every item's chunk is looked up before the first count, so the
@@ -622,8 +678,8 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
 #pragma unroll
                 for (int i = 0; i < PER; ++i) {
                     const uint32_t c = threadIdx.x * PER + i;
-                    pre[c] = ex;
-                    if (v[i]) dbase[c] = bi.off + cb[c] + g[i];
+                    pre[c] = ex | (cb[c] & CB_WIDE);
+                    if (v[i]) dbase[c] = bi.off + (cb[c] & ~CB_WIDE) + g[i];
                     ex += v[i];
                 }
             }
@@ -632,16 +688,18 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
             for (int j = 0; j < ITEMS; ++j) {
                 if (cs[j] != 0xffffffffu) {
                     const uint32_t c = cs[j] & (MAXCH - 1);
-                    const uint32_t pos = pre[c] + (cs[j] >> 10);
+                    const uint32_t pos = (pre[c] & ~CB_WIDE) + (cs[j] >> 10);
                     stQC[pos] = (j * 256 + threadIdx.x) | (bk[j] << 16);
                 }
             }
             __syncthreads();
             for (uint32_t r = threadIdx.x; r < td.len; r += blockDim.x) {
                 const uint32_t qc = stQC[r], q = qc & 0xffffu, b = qc >> 16, e = cm[b], c = e & (MAXCH - 1);
-                const uint32_t dst = dbase[c] + (r - pre[c]);
+                const uint32_t pc = pre[c];
+                const uint32_t dst = dbase[c] + (r - (pc & ~CB_WIDE));
                 BWT_DCHECK(dst - bi.off < bi.n, err);  // inside the tile's block
-                K[dst] = pack8_smem(sb, shift + q);
+                const uint64_t key = pack8_smem(sb, shift + q);
+                K[dst] = pc & CB_WIDE ? key : (key << 8) | (q ? sb[shift + q - 1] : s_before);
                 I[dst] = (i0 + q) | ((e & CM_OWN) ? 0u : (b & 0xffu) << TAG_SHIFT);
             }
             __syncthreads();
@@ -826,7 +884,9 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
                                                               const uint32_t* __restrict__ starts,
                                                               const uint32_t* __restrict__ route,
                                                               const uint64_t* __restrict__ splitters,
-                                                              uint32_t* __restrict__ members) {
+                                                              uint32_t* __restrict__ members,
+                                                              const uint8_t* __restrict__ S, uint8_t* __restrict__ L, int32_t* __restrict__ primary,
+                                                              uint32_t* __restrict__ lgather) {
     constexpr uint32_t CAP = NT * MS_IT;
     constexpr int SB = NT == 256 ? 12 : NT == 512 ? 13 : 14;  // slot bits of a word
     static_assert(CAP < (1u << SB), "a real word's slot is below the padding's");
@@ -873,14 +933,10 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
         // the chunk's keys are [kfirst, klast]: a word holds the offset from
         // kfirst, its low `sh` bits dropped if it needs more than 64 - SB bits
         uint64_t kfirst, klast;
-        const uint32_t b1 = min(b0 + nbk, (uint32_t)NBK);  // one past the last bucket
-        if (route[gd.blk] == 2u) {
-            kfirst = (uint64_t)b0 << 52;
-            klast = ((uint64_t)b1 << 52) - 1ull;  // b1 = 4096: 2^64 - 1
-        } else {
-            kfirst = b0 > 0 ? splitters[b0 - 1] : 0ull;
-            klast = b1 < (uint32_t)NBK ? splitters[b1 - 1] - 1ull : ~0ull;
-        }
+        chunk_keys(route[gd.blk] == 2u, splitters, b0, nbk, kfirst, klast);
+        const bool wide = wide_keys(kfirst, klast);
+        const uint32_t kshift = wide ? 0u : 8u;  // else the byte of L below 56 key bits
+        const uint64_t kmask = wide ? ~0ull : KEY56;
         const uint32_t sh = (uint32_t)max(SB - __clzll((long long)(klast - kfirst)), 0);
         __syncthreads();
         if (warp == 0) {
@@ -950,10 +1006,10 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
                     const uint32_t sa = v[j] & IDX_MASK;
                     BWT_DCHECK(lb < nbk && sa < bi.n, &ctrl[CTRL_ERR]);
                     lb = min(lb, nbk - 1);
-                    sI[i] = sa;
+                    sI[i] = sa | (uint32_t)w[j] << TAG_SHIFT;  // with the byte of L (of the key, if wide)
                     // any order inside the run: the sort decides it
                     const uint32_t slot = min(atomicAdd(&bcur[lb], 1u), CAP - 1u);
-                    sW[slot] = ((w[j] - kfirst) >> sh << SB) | i;
+                    sW[slot] = (((w[j] >> kshift) - kfirst) & kmask) >> sh << SB | i;
                 }
             }
         }
@@ -983,9 +1039,14 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
             // ---- 4a. every key of the chunk is its own (nearly every chunk of text): all rows are final
 #pragma unroll
             for (int j = 0; j < MS_IT; ++j)
-                if ((uint32_t)j < nreal) sO[first + j] = sI[(uint32_t)w[j] & SLOT_MASK] | SA_FINAL;
+                if ((uint32_t)j < nreal) sO[first + j] = sI[(uint32_t)w[j] & SLOT_MASK];
             __syncthreads();
-            for (uint32_t i = tid; i < len; i += NT) SA[gd.start + i] = sO[i];
+            for (uint32_t i = tid; i < len; i += NT) {
+                const uint32_t x = sO[i], sa = x & IDX_MASK;
+                SA[gd.start + i] = sa | SA_FINAL;
+                L[gd.start + i] = wide ? S[bi.off + (sa ? sa : bi.n) - 1u] : (uint8_t)(x >> TAG_SHIFT);
+                if (sa == 0u) primary[gd.blk] = (int32_t)(cstart + i);
+            }
             __syncthreads();
             continue;
         }
@@ -1017,8 +1078,9 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
                 if ((uint32_t)j < nreal) {
                     const uint32_t slot = (uint32_t)w[j] & SLOT_MASK;
                     if (!((eq >> j) & 1u)) cur = first + j + 1;
-                    const uint64_t low = sh ? (K[gd.start + min(slot, len - 1u)] - kfirst) & ((1ull << sh) - 1ull) : 0ull;
-                    w[j] = ((uint64_t)(cur - 1u) << 50) | (low << TAG_SHIFT) | sI[min(slot, CAP - 1u)];
+                    const uint64_t key = sh ? K[gd.start + min(slot, len - 1u)] >> kshift : 0ull;
+                    const uint64_t low = (key - kfirst) & ((1ull << sh) - 1ull);
+                    w[j] = ((uint64_t)(cur - 1u) << 50) | (low << TAG_SHIFT) | (sI[min(slot, CAP - 1u)] & IDX_MASK);
                 } else {
                     w[j] = ~0ull;
                 }
@@ -1058,7 +1120,20 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
         }
         // the barrier also tells whether the chunk holds a group of two or more
         const bool any_member = __syncthreads_or(mm != 0u) != 0;
-        for (uint32_t i = tid; i < len; i += NT) SA[gd.start + i] = sO[i];
+        for (uint32_t i = tid; i < len; i += NT) {
+            const uint32_t x = sO[i], sa = min(x & IDX_MASK, bi.n - 1u);
+            SA[gd.start + i] = x;
+            // this sort has dropped the bytes of L; the members' rows are
+            // gathered after the rounds
+            if (x & SA_FINAL) {
+                L[gd.start + i] = S[bi.off + (sa ? sa : bi.n) - 1u];
+                if (sa == 0u) primary[gd.blk] = (int32_t)(cstart + i);
+            }
+        }
+        if (mm) {  // a thread's rows lie in two granules at most
+            mark_lgather(lgather, gd.start + first + __ffs(mm) - 1u);
+            mark_lgather(lgather, gd.start + first + 31u - __clz(mm));
+        }
         if (any_member) {  // CTA-uniform; rare on text
             const uint32_t cur = heads_before(hm);
             WarpEmitter em;
@@ -1249,6 +1324,7 @@ bwt_status bwt::ensure_learned_buffers(bwt_plan* p) {
     if (!p->route_first) CKL(cudaMalloc(&p->route_first, sizeof(uint32_t) * 2 * p->cap_b));
     if (!p->members) CKL(cudaMalloc(&p->members, sizeof(uint32_t) * p->cap_b));
     if (!p->lazy) CKL(cudaMalloc(&p->lazy, sizeof(uint32_t) * p->cap_b));
+    if (!p->lgather) CKL(cudaMalloc(&p->lgather, sizeof(uint32_t) * ((size_t)(p->cap_n >> LG_WORD_SHIFT) + 2)));
     if (!p->bstats) CKL(cudaMalloc(&p->bstats, sizeof(unsigned long long) * 10 * p->cap_b));
     if (!p->tiles_aux) CKL(cudaMalloc(&p->tiles_aux, sizeof(TileDesc) * 2 * (size_t)p->cap_tiles0));
     if (!p->splitters_flat) {
@@ -1293,7 +1369,7 @@ bwt_status bwt::build_splitter_index(bwt_plan* p) {
     return BWT_OK;
 }
 
-bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t st) {
+bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st) {
     const uint32_t nb = p->nb, nt = p->ntiles0;
     const int sms = num_sms();
     uint32_t* ctrl = p->ctrl;
@@ -1316,8 +1392,8 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     CKL(cudaMemsetAsync(p->bucket_count, 0, sizeof(uint32_t) * 2 * NBK * nb, st));
     {
         const uint32_t span_max = 65535u / T;  // packed 16-bit counts per span
-        const uint32_t span = std::max(1u, std::min(span_max, nt / (uint32_t)(sms * 4)));
-        const int grid = std::max(1, std::min<int>((nt + span - 1) / span, sms));
+        const uint32_t span = std::max(1u, std::min(span_max, nt / (uint32_t)(sms * 8)));
+        const int grid = std::max(1, std::min<int>((nt + span - 1) / span, 2 * sms));
         k_bucket_count<false><<<grid, COUNT_THREADS, COUNT_SMEM, st>>>(
             d_in, p->blocks, p->tiles0, nt, span, p->splitters, p->splitter_index, nb, p->bucket_count, fb, nullptr);
         k_bucket_stats<<<std::min<uint32_t>(nb, 65535), 256, 0, st>>>(p->bucket_count, CHUNK_CAP, nb, p->bstats);
@@ -1353,8 +1429,9 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     k_select_rows<<<std::min<uint32_t>(nb, 65535), 256, 0, st>>>(p->bucket_count, p->route, nb);
     CKL(launch_scan_rows(p->bucket_count, NBK, nullptr, 0, nb, nb, st));  // counts -> starts in place
     ChunkTables ct{p->chunk_map, p->chunk_base, p->bucket_cursor};
-    k_chunk_plan<<<std::min<uint32_t>(nb, 65535), 256, 0, st>>>(p->bucket_count, p->blocks, p->route, nb, ct, aux,
-                                                                ctrl);
+    CKL(cudaMemsetAsync(p->lgather, 0, sizeof(uint32_t) * ((size_t)(p->total >> LG_WORD_SHIFT) + 1), st));
+    k_chunk_plan<<<std::min<uint32_t>(nb, 65535), 256, 0, st>>>(p->bucket_count, p->blocks, p->route, p->splitters, nb,
+                                                                ct, aux, p->lgather, ctrl);
     {
         const int g = sms * 4;
         if (T <= 1024)
@@ -1370,6 +1447,25 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     CKL(cudaGetLastError());
     p->stats.kernel_launches += 4;
 
+    uint32_t* chunk_counter = ctrl + CTRL_TILE_CTR + 58;  // control words no radix pass uses
+    uint32_t* big_counter = ctrl + CTRL_TILE_CTR + 59;
+    uint32_t* mid_counter = ctrl + CTRL_TILE_CTR + 50;  // no radix pass of a learned call uses it either
+    CKL(cudaMemsetAsync(chunk_counter, 0, 8, st));
+    CKL(cudaMemsetAsync(mid_counter, 0, 4, st));
+    CKL(cudaMemsetAsync(p->members, 0, sizeof(uint32_t) * nb, st));
+    // While a graph is captured the three kinds of block and bucket are sorted
+    // side by side on branch streams (they write disjoint rows): the chunk
+    // sorts; the over-full buckets; the plain-routed blocks and then the
+    // overflow buckets, whose launches mostly find no work on text (256 uneven
+    // blocks: 2,858 -> 2,796 us a call).
+    const bool fork = p->capturing && p->br[0] != nullptr;
+    const cudaStream_t ls = fork ? p->br[0] : st, ms = fork ? p->br[1] : st;
+    if (fork) {
+        CKL(cudaEventRecord(p->br_ev[0], st));
+        CKL(cudaStreamWaitEvent(ls, p->br_ev[0], 0));
+        CKL(cudaStreamWaitEvent(ms, p->br_ev[0], 0));
+    }
+
     // 4b. plain-routed blocks: the first sort of the plain path, ending in
     //     buffer 0, and its naming (with no plain-routed block every kernel
     //     here finds zero tiles and returns). Their tile table is only known
@@ -1377,24 +1473,29 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     //     the host) they take 8-bit onesweep passes.
     nv.next("bucket_plain");
     const int rb = p->rbits == 16 ? 8 : p->rbits, RADIX = 1 << rb;
-    const uint32_t status_cap = (uint32_t)std::min<uint64_t>(p->cap_status, 0xffffffffu);
     {
         const int P = (64 + rb - 1) / rb;
         uint32_t seg_stride;
         if (rb == 8) {
-            CKL(cudaMemsetAsync(p->hist, 0, sizeof(uint32_t) * 256 * nb, st));
-            CKL(launch_hist_bytes(d_in, p->blocks, tilesP, 0, p->hist, st, ntp));
-            CKL(launch_scan_rows(p->hist, 256, nullptr, 0, nb, nb, st));
+            CKL(cudaMemsetAsync(p->hist, 0, sizeof(uint32_t) * 256 * nb, ls));
+            CKL(launch_hist_bytes(d_in, p->blocks, tilesP, 0, p->hist, ls, ntp));
+            CKL(launch_scan_rows(p->hist, 256, nullptr, 0, nb, nb, ls));
             seg_stride = 256;
         } else {
-            CKL(cudaMemsetAsync(p->hist, 0, sizeof(uint32_t) * 6 * 2048 * nb, st));
-            CKL(launch_hist_keys11(d_in, p->blocks, tilesP, 0, p->tile, p->hist, st, ntp));
-            CKL(launch_scan_rows(p->hist, 2048, nullptr, 0, nb * 6, nb * 6, st));
+            CKL(cudaMemsetAsync(p->hist, 0, sizeof(uint32_t) * 6 * 2048 * nb, ls));
+            CKL(launch_hist_keys11(d_in, p->blocks, tilesP, 0, p->tile, p->hist, ls, ntp));
+            CKL(launch_scan_rows(p->hist, 2048, nullptr, 0, nb * 6, nb * 6, ls));
             seg_stride = 6 * 2048;
         }
         p->stats.kernel_launches += 2;
+        // the passes' look-back words side by side, cleared at once, where they fit
+        const bool one_zero = P * RADIX <= 2048;
         for (int ps = 0; ps < P; ++ps) {
-            CKL(launch_zero_by_count(p->status, ntp, (uint32_t)RADIX, status_cap, st));
+            if (ps == 0 || !one_zero) {
+                CKL(launch_zero_by_count({p->status, ntp, (uint32_t)(one_zero ? P * RADIX : RADIX), p->cap_status}, {},
+                                         nullptr, 0, ls));
+                p->stats.kernel_launches++;
+            }
             OneSweepParams a{};
             const int out = (P - 1 - ps) & 1, in = (P - ps) & 1;
             a.kin = ps == 0 ? nullptr : p->keys[in];
@@ -1407,32 +1508,27 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
             a.num_tiles = ntp;
             a.seg_base = p->hist + (rb == 8 ? 0 : ps * 2048);
             a.seg_base_stride = seg_stride;
-            a.status = p->status;
+            a.status = p->status + (one_zero ? ps * RADIX : 0);
+            a.status_stride = (uint32_t)(one_zero ? P * RADIX : RADIX);
             a.tile_counter = ctrl + CTRL_TILE_CTR + ps;
             a.ctrl = ctrl;
             a.shift = ps * rb;
-            CKL(launch_onesweep(8, ps == 0, rb, p->tile, a, 0, st));
-            p->stats.kernel_launches += 2;
+            CKL(launch_onesweep(8, ps == 0, rb, p->tile, a, 0, ls));
+            p->stats.kernel_launches++;
             p->stats.radix_launches++;
         }
         CKL(launch_name_tiles(p->keys[0], p->vals[0], p->blocks, tilesP, ntp, false, p->rank, bins_of(p, 0), ctrl,
-                              st));
+                              ls));
         p->stats.kernel_launches++;
     }
 
     // 4c. bucketed blocks: chunk sorts with naming, then the overflow buckets
     nv.next("bucket_sort");
-    uint32_t* chunk_counter = ctrl + CTRL_TILE_CTR + 58;  // control words no radix pass uses
-    uint32_t* big_counter = ctrl + CTRL_TILE_CTR + 59;
-    uint32_t* mid_counter = ctrl + CTRL_TILE_CTR + 50;  // no radix pass of a learned call uses it either
-    CKL(cudaMemsetAsync(chunk_counter, 0, 8, st));
-    CKL(cudaMemsetAsync(mid_counter, 0, 4, st));
-    CKL(cudaMemsetAsync(p->members, 0, sizeof(uint32_t) * nb, st));
     const bool timing = !p->events.empty() && !p->capturing && p->ev_used + 2 <= p->events.size();
     if (timing) CKL(cudaEventRecord(p->events[p->ev_used], st));
     k_chunk_sort_name<MS_NT, 4, 0><<<sms * p->chunk_sort_ctas, MS_NT, CHUNK_SORT_SMEM, st>>>(
         p->keys[0], p->vals[0], p->blocks, aux, p->rank, bins_of(p, 0), ctrl, chunk_counter, p->bucket_count, p->route,
-        p->splitters, p->members);
+        p->splitters, p->members, d_in, d_L, d_primary, p->lgather);
     CKL(cudaGetLastError());
     if (timing) {
         CKL(cudaEventRecord(p->events[p->ev_used + 1], st));
@@ -1444,29 +1540,35 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
     }
     // over-full buckets: one CTA each, 512 threads up to MID_CAP (two an SM)
     // and 1,024 up to BIG_CAP
-    k_chunk_sort_name<MID_NT, 2, 2><<<2 * sms, MID_NT, MID_SORT_SMEM, st>>>(p->keys[0], p->vals[0], p->blocks, aux,
-                                                                            p->rank, bins_of(p, 0), ctrl, mid_counter,
-                                                                            p->bucket_count, p->route, p->splitters, p->members);
-    k_chunk_sort_name<BIG_NT, 1, 1><<<sms, BIG_NT, BIG_SORT_SMEM, st>>>(p->keys[0], p->vals[0], p->blocks, aux,
-                                                                        p->rank, bins_of(p, 0), ctrl, big_counter,
-                                                                        p->bucket_count, p->route, p->splitters, p->members);
+    k_chunk_sort_name<MID_NT, 2, 2><<<2 * sms, MID_NT, MID_SORT_SMEM, ms>>>(
+        p->keys[0], p->vals[0], p->blocks, aux, p->rank, bins_of(p, 0), ctrl, mid_counter, p->bucket_count, p->route,
+        p->splitters, p->members, d_in, d_L, d_primary, p->lgather);
+    k_chunk_sort_name<BIG_NT, 1, 1><<<sms, BIG_NT, BIG_SORT_SMEM, ms>>>(
+        p->keys[0], p->vals[0], p->blocks, aux, p->rank, bins_of(p, 0), ctrl, big_counter, p->bucket_count, p->route,
+        p->splitters, p->members, d_in, d_L, d_primary, p->lgather);
     CKL(cudaGetLastError());
     p->stats.kernel_launches += 4;
 
     // overflow buckets: radix on the index, then on the key
     nv.next("bucket_overflow");
     const int PI = std::max(1, (bits_needed(p->max_n - 1) + 7) / 8), PK = 8, PT = PI + PK;
-    CKL(launch_build_large_tiles(aux, p->tile, p->ltiles, p->cap_ltiles, ctrl, st));
-    CKL(launch_zero_by_count(p->hist, aux.count + CLS_LARGE, (uint32_t)(PT * 256),
-                             (uint32_t)std::min<uint64_t>(p->cap_hist, 0xffffffffu), st));
-    k_seg_hist_u64<<<sms * 4, 256, PT * 256 * 4, st>>>(p->keys[0], p->vals[0], p->ltiles, ctrl + CTRL_NUM_LTILES,
+    CKL(launch_build_large_tiles(aux, p->tile, p->ltiles, p->cap_ltiles, ctrl, ls));
+    // an overflow bucket has more than BIG_CAP rotations, which bounds its tiles
+    const bool one_zero = ((uint64_t)p->total / T + p->total / (BIG_CAP + 1) + 1) * PT * 256 <= p->cap_status;
+    CKL(launch_zero_by_count({p->hist, aux.count + CLS_LARGE, (uint32_t)(PT * 256),
+                              p->cap_hist},
+                             {p->status, one_zero ? ctrl + CTRL_NUM_LTILES : nullptr, (uint32_t)(PT * 256), p->cap_status},
+                             ctrl + CTRL_TILE_CTR + 16, (uint32_t)PT, ls));
+    k_seg_hist_u64<<<sms * 4, 256, PT * 256 * 4, ls>>>(p->keys[0], p->vals[0], p->ltiles, ctrl + CTRL_NUM_LTILES,
                                                        p->hist, PI, PK);
     CKL(cudaGetLastError());
-    CKL(launch_scan_rows(p->hist, 256, aux.count + CLS_LARGE, (uint32_t)PT, 0, (uint32_t)(p->cap_hist / 256), st));
+    CKL(launch_scan_rows(p->hist, 256, aux.count + CLS_LARGE, (uint32_t)PT, 0, (uint32_t)(p->cap_hist / 256), ls));
     p->stats.kernel_launches += 4;
     for (int ps = 0; ps < PT; ++ps) {
-        CKL(launch_zero_by_count(p->status, ctrl + CTRL_NUM_LTILES, 256u, status_cap, st));
-        CKL(cudaMemsetAsync(ctrl + CTRL_TILE_CTR + 16 + ps, 0, 4, st));
+        if (!one_zero) {
+            CKL(launch_zero_by_count({p->status, ctrl + CTRL_NUM_LTILES, 256u, p->cap_status}, {}, nullptr, 0, ls));
+            p->stats.kernel_launches++;
+        }
         OneSweepParams a{};
         a.kin = p->keys[ps & 1];
         a.vin = p->vals[ps & 1];
@@ -1477,25 +1579,33 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t s
         a.num_tiles = ctrl + CTRL_NUM_LTILES;
         a.seg_base = p->hist + ps * 256;
         a.seg_base_stride = (uint32_t)(PT * 256);
-        a.status = p->status;
+        a.status = p->status + (one_zero ? ps * 256 : 0);
+        a.status_stride = (uint32_t)(one_zero ? PT * 256 : 256);
         a.tile_counter = ctrl + CTRL_TILE_CTR + 16 + ps;
         a.ctrl = ctrl;
         a.shift = ps < PI ? 8 * ps : 8 * (ps - PI);
-        CKL(launch_onesweep(ps < PI ? -8 : 8, false, 8, p->tile, a, 0, st));
-        p->stats.kernel_launches += 2;
+        CKL(launch_onesweep(ps < PI ? -8 : 8, false, 8, p->tile, a, 0, ls));
+        p->stats.kernel_launches++;
         p->stats.radix_launches++;
     }
     if (PT & 1) {
-        k_copy_tiles<<<sms * 4, 256, 0, st>>>(p->keys[1], p->vals[1], p->keys[0], p->vals[0], p->ltiles,
+        k_copy_tiles<<<sms * 4, 256, 0, ls>>>(p->keys[1], p->vals[1], p->keys[0], p->vals[0], p->ltiles,
                                               ctrl + CTRL_NUM_LTILES);
         CKL(cudaGetLastError());
         p->stats.kernel_launches++;
     }
     // overflow buckets are whole key ranges too: name them inside their own bounds
     CKL(launch_name_tiles(p->keys[0], p->vals[0], p->blocks, p->ltiles, ctrl + CTRL_NUM_LTILES, true, p->rank,
-                          bins_of(p, 0), ctrl, st));
+                          bins_of(p, 0), ctrl, ls));
     p->stats.kernel_launches++;
     p->learned_overflow_passes = (uint32_t)PT;
+    if (fork) {
+        CKL(cudaEventRecord(p->br_ev[0], ls));
+        CKL(cudaEventRecord(p->br_ev[1], ms));
+        CKL(cudaStreamWaitEvent(st, p->br_ev[0], 0));
+        CKL(cudaStreamWaitEvent(st, p->br_ev[1], 0));
+    }
+    CKL(cudaMemsetAsync(aux.count, 0, sizeof(uint32_t) * NCLS, st));  // the first round's next bins
 
     // 4d. ranks: blocks with many group members get every rank stored; the
     //     rest find the ranks of their groups of one on demand
@@ -1550,9 +1660,9 @@ bwt_status bwt::run_learned(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int3
     bwt_status s;
     if ((s = ensure_learned_buffers(p)) != BWT_OK) return s;
     if ((s = reset_ctrl(p, st)) != BWT_OK) return s;
-    if ((s = enqueue_learned(p, d_in, st)) != BWT_OK) return s;
+    if ((s = enqueue_learned(p, d_in, d_L, d_primary, st)) != BWT_OK) return s;
     if ((s = run_doubling_host_loop(p, st)) != BWT_OK) return s;
-    CKL(launch_gather_L(d_in, p->sa, p->blocks, p->tiles0, p->ntiles0, d_L, d_primary, p->ctrl, st));
+    CKL(launch_gather_L(d_in, p->sa, p->blocks, p->tiles0, p->ntiles0, d_L, d_primary, p->ctrl, st, p->route, p->lgather));
     p->stats.kernel_launches++;
     return BWT_OK;
 }

@@ -133,7 +133,7 @@ void bwt::free_plan_memory(bwt_plan* p) {
         FH(p->stage_parts[sl]);
         FH(p->stage_pfirst[sl]);
     }
-    F(p->splitters); F(p->splitter_index); F(p->splitters_flat); F(p->bucket_count); F(p->bucket_cursor); F(p->chunk_map); F(p->chunk_base); F(p->route); F(p->route_first); F(p->members); F(p->lazy); F(p->bstats); F(p->tiles_aux); F(p->inv_slots); F(p->inv_buf); F(p->inv_items); F(p->mtf_lists);
+    F(p->splitters); F(p->splitter_index); F(p->splitters_flat); F(p->bucket_count); F(p->bucket_cursor); F(p->chunk_map); F(p->chunk_base); F(p->route); F(p->route_first); F(p->members); F(p->lazy); F(p->lgather); F(p->bstats); F(p->tiles_aux); F(p->inv_slots); F(p->inv_buf); F(p->inv_items); F(p->mtf_lists);
     drop_graph(p);
     FH(p->h_ctrl); FH(p->h_off);
     for (int s = 0; s < 2; ++s) {
@@ -142,6 +142,8 @@ void bwt::free_plan_memory(bwt_plan* p) {
         if (p->stage_ev[s]) cudaEventDestroy(p->stage_ev[s]);
     }
     if (p->done_ev) cudaEventDestroy(p->done_ev);
+    for (auto& ev : p->br_ev)
+        if (ev) cudaEventDestroy(ev);
     FH(p->h_route); FH(p->h_bstats); FH(p->h_inv_items);
     for (auto& e : p->events) cudaEventDestroy(e);
     p->events.clear();
@@ -218,6 +220,8 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     p->h_tiles = p->stage_tiles[0];
     p->h_blocks = p->stage_blocks[0];
     if (s == BWT_OK && cudaEventCreateWithFlags(&p->done_ev, cudaEventDisableTiming) != cudaSuccess) s = BWT_ECUDA;
+    for (auto& ev : p->br_ev)
+        if (s == BWT_OK && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) s = BWT_ECUDA;
     A(host_alloc(&p->h_off, (size_t)B + 1));
     A(host_alloc(&p->h_inv_items, 2 * ((size_t)B + 1)));
     // the learned bucketing's tables and the 16-bit passes' scratch, so that
@@ -557,6 +561,7 @@ bwt_status bwt::enqueue_initial_sort(bwt_plan* p, const uint8_t* d_in, cudaStrea
         a.seg_base = p->hist + (rb == 8 ? 0 : ps * 2048);
         a.seg_base_stride = seg_stride;
         a.status = p->status + (one_memset ? region * ps : 0);
+        a.status_stride = (uint32_t)RADIX;
         a.tile_counter = ctrl + CTRL_TILE_CTR + ps;
         a.ctrl = ctrl;
         a.shift = ps * rb;
@@ -590,7 +595,19 @@ bwt_status bwt::enqueue_round(bwt_plan* p, int par, const uint32_t* host_counts,
     uint32_t* ctrl = p->ctrl;
     const uint32_t* depth = ctrl + CTRL_DEPTH;
     Bins cur = bins_of(p, par), nxt = bins_of(p, par ^ 1);
-    CK(cudaMemsetAsync(nxt.count, 0, sizeof(uint32_t) * NCLS, st));
+    // While a graph is captured the round's independent parts go to branch
+    // streams: the large groups' section beside the small groups' gathers, then
+    // (every gather before any rank is rewritten) its passes and renaming beside
+    // the small groups' sorts, the medium ones on a branch of their own. All
+    // write disjoint rows. Most launches of a round fill a fraction of the GPU
+    // (degenerate 5 x 900,000:
+    // 3,280 -> 2,660 us a call, with a round's clears merged into one launch).
+    const bool fork = p->capturing && p->br[0] != nullptr;
+    const cudaStream_t ls = fork ? p->br[0] : st, ms = fork ? p->br[1] : st;
+    if (fork) {
+        CK(cudaEventRecord(p->br_ev[0], st));
+        CK(cudaStreamWaitEvent(ls, p->br_ev[0], 0));
+    }
     {
         int launched = 0;
         CK(launch_gather_small(p->sa, p->rank, p->blocks, cur, depth, p->key2, host_counts, st, &launched,
@@ -599,12 +616,16 @@ bwt_status bwt::enqueue_round(bwt_plan* p, int par, const uint32_t* host_counts,
     }
     const bool large = !host_counts || host_counts[CLS_LARGE] > 0;
     const uint64_t k0 = p->stats.kernel_launches, r0 = p->stats.radix_launches;
-    const uint32_t hist_cap = (uint32_t)std::min<uint64_t>(p->cap_hist, 0xffffffffu);
-    const uint32_t status_cap = (uint32_t)std::min<uint64_t>(p->cap_status, 0xffffffffu);
+    // look-back words of every pass side by side (cleared with the histograms
+    // and the tile counters in one launch) where they fit: a large group has
+    // more than MED_MAX rotations, so cap_ltiles tiles of P2 * RADIX words
+    const bool one_zero = P2 * RADIX <= 2048;
     if (large) {
-        const cudaStream_t ls = st;
         CK(launch_build_large_tiles(cur, p->tile, p->ltiles, p->cap_ltiles, ctrl, ls, p->seg_varied));
-        CK(launch_zero_by_count(p->hist, cur.count + CLS_LARGE, (uint32_t)(P2 * RADIX), hist_cap, ls));
+        CK(launch_zero_by_count({p->hist, cur.count + CLS_LARGE, (uint32_t)(P2 * RADIX), p->cap_hist},
+                                {p->status, one_zero ? ctrl + CTRL_NUM_LTILES : nullptr, (uint32_t)(P2 * RADIX),
+                                 p->cap_status},
+                                ctrl + CTRL_TILE_CTR + 16, (uint32_t)P2, ls));
         // with one pass only, that pass would read and write SA in place: it
         // reads a copy instead
         CK(launch_large_prologue(p->sa, p->rank, p->blocks, p->ltiles, ctrl + CTRL_NUM_LTILES, depth, p->kA,
@@ -612,10 +633,21 @@ bwt_status bwt::enqueue_round(bwt_plan* p, int par, const uint32_t* host_counts,
         CK(launch_scan_rows(p->hist, RADIX, cur.count + CLS_LARGE, (uint32_t)P2, 0, (uint32_t)(p->cap_hist / RADIX),
                             ls));
         p->stats.kernel_launches += 4;
+    }
+    if (fork) {
+        CK(cudaEventRecord(p->br_ev[0], ls));
+        CK(cudaStreamWaitEvent(st, p->br_ev[0], 0));
+        CK(cudaEventRecord(p->br_ev[0], st));
+        CK(cudaStreamWaitEvent(ls, p->br_ev[0], 0));
+        CK(cudaStreamWaitEvent(ms, p->br_ev[0], 0));
+    }
+    if (large) {
         for (int ps = 0; ps < P2; ++ps) {
-            CK(launch_zero_by_count(p->status, ctrl + CTRL_NUM_LTILES, (uint32_t)RADIX, status_cap, ls));
-            CK(cudaMemsetAsync(ctrl + CTRL_TILE_CTR + 16 + ps, 0, 4, ls));
-            p->stats.kernel_launches++;
+            if (!one_zero) {
+                CK(launch_zero_by_count({p->status, ctrl + CTRL_NUM_LTILES, (uint32_t)RADIX, p->cap_status}, {}, nullptr,
+                                        0, ls));
+                p->stats.kernel_launches++;
+            }
             OneSweepParams a{};
             const bool last = ps == P2 - 1;
             a.kin = ps == 0 ? p->kA : ((ps - 1) & 1 ? p->kA : p->kB);
@@ -627,7 +659,8 @@ bwt_status bwt::enqueue_round(bwt_plan* p, int par, const uint32_t* host_counts,
             a.num_tiles = ctrl + CTRL_NUM_LTILES;
             a.seg_base = p->hist + ps * RADIX;
             a.seg_base_stride = (uint32_t)(P2 * RADIX);
-            a.status = p->status;
+            a.status = p->status + (one_zero ? ps * RADIX : 0);
+            a.status_stride = (uint32_t)(one_zero ? P2 * RADIX : RADIX);
             a.tile_counter = ctrl + CTRL_TILE_CTR + 16 + ps;
             a.ctrl = ctrl;
             a.shift = ps * rb;
@@ -638,13 +671,19 @@ bwt_status bwt::enqueue_round(bwt_plan* p, int par, const uint32_t* host_counts,
     }
     const uint64_t k1 = p->stats.kernel_launches, r1 = p->stats.radix_launches;
     int launched = 0;
-    CK(launch_sort_small(p->sa, p->key2, p->rank, p->blocks, cur, nxt, depth, host_counts, ctrl, st, &launched));
+    CK(launch_sort_small(p->sa, p->key2, p->rank, p->blocks, cur, nxt, depth, host_counts, ctrl, st, ms, &launched));
     p->stats.kernel_launches += launched;
     const uint64_t k2 = p->stats.kernel_launches;
     if (large) {
         CK(launch_rename_large(p->sa, p->key2, p->rank, p->blocks, p->ltiles, ctrl + CTRL_NUM_LTILES, nxt, depth,
-                               p->seg_varied, ctrl, st));
+                               p->seg_varied, ctrl, ls));
         p->stats.kernel_launches++;
+    }
+    if (fork) {
+        CK(cudaEventRecord(p->br_ev[0], ls));
+        CK(cudaEventRecord(p->br_ev[1], ms));
+        CK(cudaStreamWaitEvent(st, p->br_ev[0], 0));
+        CK(cudaStreamWaitEvent(st, p->br_ev[1], 0));
     }
     p->cap_large_kernels = (k1 - k0) + (p->stats.kernel_launches - k2);  // one round's large-group section
     p->cap_large_radix = r1 - r0;

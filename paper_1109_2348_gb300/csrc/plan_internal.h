@@ -113,6 +113,7 @@ struct bwt_plan {
     uint32_t* route_first = nullptr;    // [2][block] first tile of each block in its route's tile table
     uint32_t* members = nullptr;        // [block] rotations the chunk sorts sent to the doubling rounds
     uint32_t* lazy = nullptr;           // [block] 1: ranks of groups of one are found on demand
+    uint32_t* lgather = nullptr;       // learned: marks of the rows whose bytes of L the gather writes (LG_ROW_SHIFT)
     bwt::LazyRanks lazy_ranks;          // how this call's doubling rounds read ranks
     unsigned long long* bstats = nullptr;  // [2][block][5] overflow keys, overflow buckets, largest bucket,
                                            // sum of squared sizes, non-empty buckets
@@ -186,6 +187,8 @@ struct bwt_plan {
     uint64_t graph_main_radix = 0, graph_large_radix = 0;
     uint64_t cap_large_kernels = 0, cap_large_radix = 0;  // one round's large-group section, as enqueued
     bool capturing = false;
+    cudaStream_t br[2] = {nullptr, nullptr};    // branch streams of the round being captured (graph.cu)
+    cudaEvent_t br_ev[2] = {nullptr, nullptr};
 
     bwt_stats stats{};
     bwt_status last = BWT_OK;
@@ -225,7 +228,7 @@ bwt_status run_learned(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* 
 // Learned first stage (bucket count, device-side routing, scatter, chunk sorts
 // with naming, overflow radix, plain radix of plain-routed blocks) with no
 // host synchronisation, so it can be captured; ctrl must have been reset.
-bwt_status enqueue_learned(bwt_plan* p, const uint8_t* d_in, cudaStream_t st);
+bwt_status enqueue_learned(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st);
 // After the call has synchronised: routing and bucket statistics from the
 // per-block counters the learned stage copied to the host.
 void learned_stats(bwt_plan* p);

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
         if (owner) {
 #pragma unroll
             for (int i = 0; i < DPT; ++i) {
-                uint32_t* mine = p.status + (size_t)t * RADIX + tid * DPT + i;
+                uint32_t* mine = p.status + (size_t)t * p.status_stride + tid * DPT + i;
                 if (first) {
                     if (!(withhold && t == 0)) st_volatile(mine, ST_INC | cnt[i]);
                 } else {
@@ -240,8 +240,8 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
                 const int d = tid;
                 uint32_t excl = 0;
                 if (!first) {
-                    excl = lookback_digit(p.status, RADIX, t, td.firstTile, d, spin_limit, &p.ctrl[CTRL_ERR]);
-                    st_volatile(p.status + (size_t)t * RADIX + d, ST_INC | ((excl + cnt[0]) & ST_VALUE));
+                    excl = lookback_digit(p.status, p.status_stride, t, td.firstTile, d, spin_limit, &p.ctrl[CTRL_ERR]);
+                    st_volatile(p.status + (size_t)t * p.status_stride + d, ST_INC | ((excl + cnt[0]) & ST_VALUE));
                 }
                 gbase[d] = td.segStart + p.seg_base[(size_t)td.seg * p.seg_base_stride + d] + excl - digit_start[d];
             }
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
                 uint32_t v[DPT];
 #pragma unroll
                 for (int i = 0; i < DPT; ++i)
-                    v[i] = (pending >> i) & 1u ? ld_volatile(p.status + (size_t)q[i] * RADIX + tid * DPT + i) : 0u;
+                    v[i] = (pending >> i) & 1u ? ld_volatile(p.status + (size_t)q[i] * p.status_stride + tid * DPT + i) : 0u;
                 bool progress = false;
 #pragma unroll
                 for (int i = 0; i < DPT; ++i) {
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
 #pragma unroll
                 for (int i = 0; i < DPT; ++i) {
                     const int d = tid * DPT + i;
-                    if (!first) st_volatile(p.status + (size_t)t * RADIX + d, ST_INC | ((excl[i] + cnt[i]) & ST_VALUE));
+                    if (!first) st_volatile(p.status + (size_t)t * p.status_stride + d, ST_INC | ((excl[i] + cnt[i]) & ST_VALUE));
                     gbase[d] = td.segStart + p.seg_base[(size_t)td.seg * p.seg_base_stride + d] + excl[i] -
                                digit_start[d];
                 }
@@ -419,12 +419,14 @@ __global__ void __launch_bounds__(256) k_scan_rows(uint32_t* __restrict__ hist, 
     }
 }
 
-__global__ void k_zero_by_count(uint32_t* __restrict__ p, const uint32_t* __restrict__ count, uint32_t per_unit,
-                                uint32_t max_words) {
-    uint64_t n = (uint64_t)(*count) * per_unit;
-    if (n > max_words) n = max_words;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        p[i] = 0u;
+// Zeroes a[0, *a_count * a_per), b[0, *b_count * b_per) (up to their limits)
+// and c[0, nc): what the large-group section of a round clears, in one launch.
+__global__ void k_zero_by_count(ZeroRange a, ZeroRange b, uint32_t* __restrict__ c, uint32_t nc) {
+    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t na = a.words(), nb = b.words();
+    for (uint64_t i = i0; i < na; i += stride) a.p[i] = 0u;
+    for (uint64_t i = i0; i < nb; i += stride) b.p[i] = 0u;
+    if (i0 < nc) c[i0] = 0u;
 }
 
 // A pass's tiles start in table order, and a tile looks back over its block's
@@ -590,9 +592,8 @@ cudaError_t launch_scan_rows(uint32_t* hist, int radix, const uint32_t* num_rows
     return cudaGetLastError();
 }
 
-cudaError_t launch_zero_by_count(uint32_t* p, const uint32_t* count, uint32_t words_per_unit, uint32_t max_words,
-                                 cudaStream_t st) {
-    k_zero_by_count<<<num_sms() * 4, 256, 0, st>>>(p, count, words_per_unit, max_words);
+cudaError_t launch_zero_by_count(ZeroRange a, ZeroRange b, uint32_t* c, uint32_t nc, cudaStream_t st) {
+    k_zero_by_count<<<num_sms() * 4, 256, 0, st>>>(a, b, c, nc);
     return cudaGetLastError();
 }
 
