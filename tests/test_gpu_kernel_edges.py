@@ -180,3 +180,56 @@ def test_interleaved_tiles(tile, flags):
             buf, off = batch_from_blocks(part)
             L, prim, _ = gpu_bwt(buf, off, plan)
             assert_matches_oracle(buf, off, L, prim, f"{len(part)} blocks")
+
+
+@pytest.mark.parametrize("count", [1, 31, 63, 64, 65, 200])
+def test_mlp_gradient_of_partial_ctas(count):
+    """Four threads a sample, 64 samples a CTA: counts around a warp and a CTA
+    against the float64 oracle, to the relative 1e-4 / absolute 1e-6 the
+    gradient check uses."""
+    import ctypes
+
+    import torch
+    from paper_1109_2348_gb300 import _lib
+    r = np.random.RandomState(count)
+    params = model.init_params(7)
+    x = r.rand(count, 8).astype(np.float32)
+    t = r.rand(count).astype(np.float32)
+    loss, want = oracle.mlp_loss_grad(params.astype(np.float64), x.astype(np.float64), t.astype(np.float64))
+    d = [torch.from_numpy(a).cuda() for a in (params, x, t)]
+    grad, got_loss = torch.zeros(params.size, device="cuda"), torch.zeros(1, device="cuda")
+    vp = [ctypes.c_void_p(a.data_ptr()) for a in (*d, grad, got_loss)]
+    lib = _lib.load()
+    _lib.check(lib.bwt_mlp_loss_grad(vp[0], vp[1], vp[2], count, vp[3], vp[4], ctypes.c_void_p(0)), "loss_grad")
+    np.testing.assert_allclose(grad.cpu().numpy(), want, rtol=1e-4, atol=1e-6)
+    np.testing.assert_allclose(got_loss.item(), loss, rtol=1e-4, atol=1e-6)
+
+
+def test_spread_of_equal_splitters():
+    """A model whose output jumps where the first byte does gives runs of equal
+    splitters: the compiled table is sorted and spreads each run evenly up to
+    the next distinct splitter."""
+    import ctypes
+
+    import torch
+    from paper_1109_2348_gb300 import _lib
+    p = np.zeros(model.NPARAMS, dtype=np.float32)  # y = x0 through one unit a layer
+    p[0] = p[288] = p[1344] = 1.0
+    norm = np.repeat(np.arange(8, dtype=np.float32) / 8, 32)  # eight steps over the first byte
+    d_p, d_n = torch.from_numpy(p).cuda(), torch.from_numpy(norm).cuda()
+    d_s = torch.zeros(model.SPLITTERS, dtype=torch.int64, device="cuda")
+    vp = [ctypes.c_void_p(a.data_ptr()) for a in (d_p, d_n, d_s)]
+    lib = _lib.load()
+    _lib.check(lib.bwt_model_compile(*vp, ctypes.c_void_p(0)), "compile")
+    got = d_s.cpu().numpy().view(np.uint64)
+    want = []
+    for j in range(model.SPLITTERS):  # the smallest key whose first byte's step reaches (j + 1) / 4096
+        step = -(-(j + 1) * 8 // 4096)
+        want.append((step * 32) << 56 if step < 8 else (1 << 64) - 1)
+    want = sorted(want)
+    out = []
+    for i, w in enumerate(want):
+        first, end = want.index(w), len(want) - want[::-1].index(w)
+        nxt = want[end] if end < len(want) else (1 << 64) - 1
+        out.append(w + (nxt - w) * (i - first) // (end - first))
+    assert np.array_equal(got, np.array(out, dtype=np.uint64))
