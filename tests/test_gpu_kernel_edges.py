@@ -233,3 +233,30 @@ def test_spread_of_equal_splitters():
         nxt = want[end] if end < len(want) else (1 << 64) - 1
         out.append(w + (nxt - w) * (i - first) // (end - first))
     assert np.array_equal(got, np.array(out, dtype=np.uint64))
+
+
+@pytest.mark.parametrize("shift", [0, 1, 7])
+@pytest.mark.parametrize("longest", [1, 13, 26, 27, 32])
+def test_vle_word_packing(longest, shift):
+    """Variable-length encoding by whole words: codes of one length up to the
+    one that shares a word with its length, just above it and of 32 bits, mixed
+    with 1-bit ones, blocks of every size around a thread's 16 bytes and a tile,
+    unaligned input."""
+    import torch
+    r = np.random.RandomState(61)
+    length = np.where(np.arange(256) % 3 == 0, longest, r.randint(1, longest + 1, 256)).astype(np.uint8)
+    code = r.randint(0, 1 << 32, 256, dtype=np.uint64).astype(np.uint32)
+    blocks = [r.randint(0, a, n).astype(np.uint8) for a in (1, 256) for n in (1, 15, 16, 17, 31, 4095, 4096, 4097, 9001)]
+    buf, off = batch_from_blocks(blocks)
+    sizes = np.diff(off.astype(np.int64))
+    d_in = torch.zeros(buf.size + 16, dtype=torch.uint8, device="cuda")
+    d_in[shift:shift + buf.size] = torch.from_numpy(buf).cuda()
+    with Plan(max_blocks=off.size - 1, max_total_bytes=buf.size, max_block_bytes=int(sizes.max())) as plan:
+        got, byte_off, bits = plan.vle_encode(d_in[shift:shift + buf.size], off, code, length)
+    got, byte_off = got.cpu().numpy(), byte_off.cpu().numpy()
+    for b in range(off.size - 1):
+        blk = buf[int(off[b]):int(off[b + 1])]
+        want = "".join(format(int(code[x]) & ((1 << int(length[x])) - 1), "b").zfill(int(length[x])) for x in blk)
+        assert int(bits[b]) == len(want)
+        want = np.frombuffer(int(want.ljust(-(-len(want) // 8) * 8, "0"), 2).to_bytes(-(-len(want) // 8), "big"), np.uint8)
+        assert np.array_equal(got[byte_off[b]:byte_off[b + 1]], want), f"block {b}"
