@@ -71,7 +71,8 @@ typedef struct {
     int radix_bits;            /* first sort's LSD digit width: 8, 11 or 16; 0 = the default (8) or the
                                   autotuned value. 16 adds about 4.3 bytes per byte of max_total_bytes
                                   plus 256 KB per block of scratch */
-    int tile_keys;             /* keys per radix tile: 1024, 2048 or 4096; 0 = default (4096) */
+    int tile_keys;             /* keys per radix tile: 1024, 2048 or 4096; 0 = default (4096; the radix
+                                  passes of a batch of up to about 900,000 bytes then take 1024) */
     uint32_t flags;            /* BWT_F_* */
     const char* model_path;    /* splitter table for BWT_F_LEARNED (bwt_model_compile output); may be NULL */
 } bwt_plan_desc;

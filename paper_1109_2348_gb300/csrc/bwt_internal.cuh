@@ -71,8 +71,8 @@ constexpr uint32_t LG_ROW_SHIFT = 7, LG_WORD_SHIFT = LG_ROW_SHIFT + 5;
 constexpr int NCLS = 5;
 constexpr uint32_t MICRO_MAX = 4;     // one thread per group, sorting network in registers
 constexpr uint32_t TINY_MAX = 32;     // one warp per group, bitonic across the lanes
-constexpr uint32_t SMALL_MAX = 256;   // one warp per group, bitonic in shared memory
-constexpr uint32_t MED_MAX = 2048;    // one CTA per group, bitonic in shared memory
+constexpr uint32_t SMALL_MAX = 256;   // one warp per group, merged in shared memory
+constexpr uint32_t MED_MAX = 2048;    // one CTA per group, merged in shared memory
 // groups above MED_MAX (class 4, "large") are sorted by the segmented onesweep radix.
 constexpr int CLS_LARGE = 4;
 
@@ -87,7 +87,7 @@ enum : int {
     CTRL_SPIN = 16,         // spin limit for bounded waits
     CTRL_WITHHOLD = 17,     // debug: first tile withholds its look-back publish
     CTRL_DEPTH = 18,        // prefix length h the current round doubles
-    CTRL_NTILES0 = 19,      // tiles of the first sort
+    CTRL_NTILES0 = 19,      // tiles of the first sort's passes
     CTRL_BODY_ITERS = 20,   // graph mode: doubling rounds whose launches ran (a round skipped by its condition is not counted)
     CTRL_AUX0 = 21,         // learned: tiles of plain-routed blocks
     CTRL_AUX1 = 22,         // learned: tiles of bucketed blocks

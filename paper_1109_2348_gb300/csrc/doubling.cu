@@ -18,7 +18,7 @@
 //   large_prologue (large groups, by tile)
 //   -> sorts: micro (sorting network in registers), tiny (bitonic across a
 //      warp's lanes), small (warp: 33..64 bitonic in registers by shuffles,
-//      larger in shared memory), medium (CTA bitonic in shared memory),
+//      larger merged in shared memory), medium (CTA, merged in shared memory),
 //      large (segmented onesweep radix)
 //   -> renames (fused into the small sorts; rename_large for large groups).
 // Refined groups are appended to the next round's size-class bins. A group
@@ -190,19 +190,43 @@ __global__ void __launch_bounds__(256) k_gather_micro(const uint32_t* __restrict
     }
 }
 
-// tiny, small and medium groups: one warp per group
+// tiny and small groups: one warp per group; medium groups: one CTA per group,
+// eight elements a thread in flight at once (by a warp their 2,048 elements
+// were 16 steps of two dependent loads: a launch 19 -> 6 us on 24 small blocks,
+// 22 -> 14 on the degenerate ones)
 __global__ void __launch_bounds__(256) k_gather_small(const uint32_t* __restrict__ SA, const uint32_t* __restrict__ rank,
                                                       const BlockInfo* __restrict__ blocks, Bins cur,
                                                       const uint32_t* __restrict__ depth, uint32_t* __restrict__ key2,
                                                       const LazyRanks lz) {
     const uint32_t h = *depth;
     const uint32_t c1 = bin_count(cur, 1), c2 = bin_count(cur, 2), c3 = bin_count(cur, 3);
-    const uint32_t total = c1 + c2 + c3;
+    const uint32_t total = c1 + c2;
     const int lane = threadIdx.x & 31;
     const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
-    auto desc = [&](uint32_t g) {
-        return g < c1 ? cur.list[1][g] : (g < c1 + c2 ? cur.list[2][g - c1] : cur.list[3][g - c1 - c2]);
-    };
+    for (uint32_t g = blockIdx.x; g < c3; g += gridDim.x) {
+        const GroupDesc gd = cur.list[3][g];
+        const BlockInfo bi = blocks[gd.blk];
+        constexpr int U = MED_MAX / 256;
+        uint32_t s[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t e = threadIdx.x + 256 * u;
+            s[u] = e < gd.len ? SA[gd.start + e] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t e = threadIdx.x + 256 * u;
+            uint32_t r = s[u] + h;
+            if (r >= bi.n) r -= bi.n;
+            s[u] = e < gd.len && r < bi.n ? rank_at(lz, rank, bi, gd.blk, r) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t e = threadIdx.x + 256 * u;
+            if (e < gd.len) key2[gd.start + e] = s[u];
+        }
+    }
+    auto desc = [&](uint32_t g) { return g < c1 ? cur.list[1][g] : cur.list[2][g - c1]; };
     // two groups a warp (g and g + nwarps), their chains of loads interleaved:
     // the gather is bound by the latency of descriptor -> SA -> rank
     for (uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < total; g += 2 * nwarps) {
@@ -212,8 +236,8 @@ __global__ void __launch_bounds__(256) k_gather_small(const uint32_t* __restrict
         const BlockInfo b0 = blocks[gd0.blk];
         const BlockInfo b1 = blocks[gd1.blk];
         const uint32_t len = max(gd0.len, gd1.len);
-        // U elements of each group a lane per step (medium groups run to
-        // 2,048): all their SA loads, then all their rank gathers, in flight
+        // U elements of each group a lane per step: all their SA loads, then
+        // all their rank gathers, in flight
         constexpr int U = 4;
         for (uint32_t e0 = lane; e0 < len; e0 += 32 * U) {
             uint32_t s0[U], s1[U];
@@ -325,12 +349,17 @@ __global__ void __launch_bounds__(256) k_large_prologue(const uint32_t* __restri
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* sh = reinterpret_cast<uint32_t*>(smem);
     const int lane = threadIdx.x & 31;
-    const uint32_t nt = *num_tiles;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+    // With few tiles a CTA takes a quarter of one: a tile's four steps, each a
+    // chain of two loads, then run side by side (24 small blocks: a launch
+    // 18 -> 8.5 us).
+    const uint32_t nt = *num_tiles, parts = nt * 4u <= gridDim.x ? 4u : 1u;
+    for (uint32_t u = blockIdx.x; u < nt * parts; u += gridDim.x) {
         for (int i = threadIdx.x; i < passes * RADIX; i += blockDim.x) sh[i] = 0;
         __syncthreads();
-        const TileDesc td = tiles[t];
+        const TileDesc td = tiles[u / parts];
         const BlockInfo bi = blocks[td.blk];
+        const uint32_t qa = parts == 1u ? 0u : min(td.len, (u % parts) * 1024u);
+        const uint32_t qe = parts == 1u ? td.len : min(td.len, qa + 1024u);
         // key2 of the group's first member: the group does not move this
         // round if every member has it
         uint32_t k0;
@@ -343,18 +372,18 @@ __global__ void __launch_bounds__(256) k_large_prologue(const uint32_t* __restri
         // PI elements a thread per step: their SA loads, then their rank
         // gathers, are all in flight at once
         constexpr int PI = 4;
-        for (uint32_t q0 = 0; q0 < td.len; q0 += 256u * PI) {
+        for (uint32_t q0 = qa; q0 < qe; q0 += 256u * PI) {
             uint32_t sa[PI], k2[PI];
 #pragma unroll
             for (int j = 0; j < PI; ++j) {
                 const uint32_t q = q0 + j * 256u + threadIdx.x;
-                sa[j] = q < td.len ? SA[td.start + q] : 0u;
+                sa[j] = q < qe ? SA[td.start + q] : 0u;
             }
 #pragma unroll
             for (int j = 0; j < PI; ++j) {
                 const uint32_t q = q0 + j * 256u + threadIdx.x;
                 k2[j] = 0u;
-                if (q < td.len) {
+                if (q < qe) {
                     uint32_t r = sa[j] + h;
                     if (r >= bi.n) r -= bi.n;
                     k2[j] = r < bi.n ? rank_at(lz, rank, bi, td.blk, r) : 0u;
@@ -363,7 +392,7 @@ __global__ void __launch_bounds__(256) k_large_prologue(const uint32_t* __restri
 #pragma unroll
             for (int j = 0; j < PI; ++j) {
                 const uint32_t q = q0 + j * 256u + threadIdx.x;
-                const bool valid = q < td.len;
+                const bool valid = q < qe;
                 if (valid) {
                     kbuf[td.start + q] = k2[j];
                     if (vbuf) vbuf[td.start + q] = sa[j];
@@ -515,28 +544,71 @@ __device__ __forceinline__ void coop_sync() {
     if constexpr (NT == 32) __syncwarp(); else __syncthreads();
 }
 
-// Sorts comp[0..P) (P a power of two) by bitonic merging; NT threads
-// cooperate (a warp or the CTA), t is the thread's index among them. Each
-// step has P/2 compare-exchanges; thread t takes pairs t, t + NT, ..: pair
-// p is (i, i + j) with i = p with a zero bit inserted at j's position.
+// Sorts comp[0..m) ascending; NT threads cooperate (a warp or the CTA), t is
+// the thread's index among them, m <= 8 NT, comp holds CS_IT * NT + 1 words.
+// Every thread sorts CS_IT words in registers (odd-even transposition), then
+// merge-path rounds double the sorted runs: at most 8 for a CTA, each two
+// barriers, against the 66 compare-exchange steps of a bitonic sort of 2,048
+// (degenerate 5 x 900,000: medium groups 489 -> 417 us a call, small ones
+// 289 -> 221). CS_IT is odd, so that the threads' runs start in different
+// banks. Words past m are padded with all ones; a head may be read one word
+// past its run and is then never chosen.
+constexpr int CS_IT = 9;
+
 template <int NT>
-__device__ __forceinline__ void coop_bitonic(uint64_t* comp, uint32_t P, uint32_t t) {
-    const uint32_t half = P >> 1;
-    for (uint32_t kk = 2; kk <= P; kk <<= 1) {
-        for (uint32_t j = kk >> 1; j > 0; j >>= 1) {
-            for (uint32_t pr = t; pr < half; pr += NT) {
-                const uint32_t i = ((pr & ~(j - 1)) << 1) | (pr & (j - 1));
-                const uint32_t ixj = i | j;
-                const uint64_t a = comp[i], b = comp[ixj];
-                const bool up = (i & kk) == 0;
-                if ((a > b) == up) {
-                    comp[i] = b;
-                    comp[ixj] = a;
-                }
+__device__ __forceinline__ void coop_sort(uint64_t* comp, uint32_t m, uint32_t t) {
+    const uint32_t nth = (m + CS_IT - 1) / CS_IT;  // threads with words
+    if (t < nth * CS_IT - m) comp[m + t] = ~0ull;
+    coop_sync<NT>();
+    const bool active = t < nth;
+    uint64_t w[CS_IT];
+    if (active) {
+#pragma unroll
+        for (int j = 0; j < CS_IT; ++j) w[j] = comp[t * CS_IT + j];
+#pragma unroll
+        for (int r = 0; r < CS_IT; ++r) {
+#pragma unroll
+            for (int j = r & 1; j + 1 < CS_IT; j += 2) {
+                const uint64_t a = w[j], b = w[j + 1];
+                const bool sw = b < a;
+                w[j] = sw ? b : a;
+                w[j + 1] = sw ? a : b;
             }
-            coop_sync<NT>();
         }
     }
+    for (uint32_t h = 1; h < nth; h <<= 1) {  // threads per input run
+        if (active) {
+#pragma unroll
+            for (int j = 0; j < CS_IT; ++j) comp[t * CS_IT + j] = w[j];
+        }
+        coop_sync<NT>();
+        if (active) {
+            const uint32_t f = t & ~(2 * h - 1);  // the merged run's first thread
+            const uint32_t la = min(h, nth - f) * CS_IT, lb = (min(2 * h, nth - f)) * CS_IT - la;
+            const uint64_t *A = comp + f * CS_IT, *B = A + la;
+            const uint32_t diag = (t - f) * CS_IT;
+            uint32_t lo = diag > lb ? diag - lb : 0u, hi = min(diag, la);
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (A[mid] <= B[diag - 1 - mid]) lo = mid + 1; else hi = mid;
+            }
+            uint32_t ia = lo, ib = diag - lo;
+            uint64_t ka = A[ia], kb = B[ib];
+#pragma unroll
+            for (int j = 0; j < CS_IT; ++j) {
+                const bool take_b = ib < lb && (ia >= la || kb < ka);
+                w[j] = take_b ? kb : ka;
+                if (take_b) kb = B[++ib];
+                else ka = A[++ia];
+            }
+        }
+        coop_sync<NT>();
+    }
+    if (active) {
+#pragma unroll
+        for (int j = 0; j < CS_IT; ++j) comp[t * CS_IT + j] = w[j];
+    }
+    coop_sync<NT>();
 }
 
 // Loads a group's (key2, SA) composites, sorts them, writes SA back, renames
@@ -547,8 +619,6 @@ __device__ __forceinline__ void sort_rename_group(uint64_t* comp, const GroupDes
                                                   uint32_t* __restrict__ rank, const Bins& next, uint32_t new_depth,
                                                   WarpEmitter& em, uint32_t* err, uint32_t t) {
     const uint32_t m = gd.len;
-    uint32_t P = 32;
-    while (P < m) P <<= 1;
     static_assert((NT == 32 ? SMALL_MAX : MED_MAX) <= 8 * NT, "a group fits 8 elements a thread");
     // A group whose members all have the same key2 cannot split: it stays in
     // index order with its ranks (every member already holds the group's
@@ -572,7 +642,7 @@ __device__ __forceinline__ void sort_rename_group(uint64_t* comp, const GroupDes
     }
     bool sorted = false;
     if constexpr (NT == 32) {
-        if (P == 64) {
+        if (m <= 64) {
             // 33..64 elements: element e = r * 32 + t in register c[r]; the
             // bitonic network by shuffles (its one distance-32 step pairs a
             // lane's own two elements), then the result to shared memory
@@ -603,7 +673,7 @@ __device__ __forceinline__ void sort_rename_group(uint64_t* comp, const GroupDes
         }
     }
     if (!sorted) {
-        // up to 8 elements a thread (P <= 8 NT): all loads in flight before any store
+        // up to 8 elements a thread: all loads in flight before any store
         uint32_t lk[8], ls[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -614,10 +684,9 @@ __device__ __forceinline__ void sort_rename_group(uint64_t* comp, const GroupDes
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const uint32_t i = t + j * NT;
-            if (i < P) comp[i] = i < m ? (((uint64_t)lk[j] << 32) | ls[j]) : ~0ull;
+            if (i < m) comp[i] = ((uint64_t)lk[j] << 32) | ls[j];
         }
-        coop_sync<NT>();
-        coop_bitonic<NT>(comp, P, t);
+        coop_sort<NT>(comp, m, t);
     }
     if constexpr (NT == 32) {
         // One warp: group heads by ballot, 32 elements a step. An element's
@@ -680,12 +749,12 @@ __device__ __forceinline__ void sort_rename_group(uint64_t* comp, const GroupDes
     coop_sync<NT>();
 }
 
-// small groups (33..256): one warp each, bitonic in the warp's shared memory
+// small groups (33..256): one warp each, sorted in the warp's shared memory
 __global__ void __launch_bounds__(256) k_sort_small(uint32_t* __restrict__ SA, const uint32_t* __restrict__ key2,
                                                     uint32_t* __restrict__ rank, const BlockInfo* __restrict__ blocks,
                                                     Bins cur, Bins next, const uint32_t* __restrict__ depth,
                                                     uint32_t* ctrl) {
-    __shared__ uint64_t comp[8][SMALL_MAX];
+    __shared__ uint64_t comp[8][CS_IT * 32 + 1];
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
     if (ld_volatile(&ctrl[CTRL_ERR])) return;
     const uint32_t new_depth = 2u * *depth;
@@ -702,12 +771,12 @@ __global__ void __launch_bounds__(256) k_sort_small(uint32_t* __restrict__ SA, c
     em.finish(next, &ctrl[CTRL_ERR]);
 }
 
-// medium groups (257..2048): one CTA each, bitonic in shared memory
+// medium groups (257..2048): one CTA each, sorted in shared memory
 __global__ void __launch_bounds__(256) k_sort_med(uint32_t* __restrict__ SA, const uint32_t* __restrict__ key2,
                                                   uint32_t* __restrict__ rank, const BlockInfo* __restrict__ blocks,
                                                   Bins cur, Bins next, const uint32_t* __restrict__ depth,
                                                   uint32_t* ctrl) {
-    __shared__ uint64_t comp[MED_MAX];
+    __shared__ uint64_t comp[CS_IT * 256 + 1];
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
     if (ld_volatile(&ctrl[CTRL_ERR])) return;
     const uint32_t new_depth = 2u * *depth;
@@ -905,8 +974,8 @@ cudaError_t launch_gather_small(const uint32_t* SA, const uint32_t* rank, const 
     int g_micro = num_sms() * 8, g_warp = num_sms() * 16;
     if (host_counts) {
         g_micro = host_counts[0] ? grid_for(std::min(host_counts[0], 0x3fffffffu) * MICRO_MAX, 256, 8) : 0;
-        const uint32_t n = host_counts[1] + host_counts[2] + host_counts[3];
-        g_warp = n ? grid_for(n, 8, 16) : 0;
+        const uint32_t n = host_counts[1] + host_counts[2];
+        g_warp = std::max(n ? grid_for(n, 8, 16) : 0, host_counts[3] ? grid_for(host_counts[3], 1, 16) : 0);
     }
     *launched = 0;
     if (g_micro) {

@@ -40,7 +40,7 @@ using namespace bwt;
 static std::vector<uint64_t> graph_key_of(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary) {
     std::vector<uint64_t> k = {(uint64_t)(uintptr_t)d_in, (uint64_t)(uintptr_t)d_L, (uint64_t)(uintptr_t)d_primary,
                                (uint64_t)p->rbits, (uint64_t)p->tile, (uint64_t)p->spin_limit,
-                               (uint64_t)p->withhold, (uint64_t)p->nb, (uint64_t)p->round_bits};
+                               (uint64_t)p->withhold, (uint64_t)p->nb, (uint64_t)p->round_bits, (uint64_t)p->rtile};
     k.insert(k.end(), p->h_off, p->h_off + p->nb + 1);
     return k;
 }
@@ -163,7 +163,8 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     r3 = p->stats.radix_launches;
     {
         NvtxRange nv("gather");
-        CKG(launch_gather_L(d_in, p->sa, p->blocks, p->tiles0, p->ntiles0, d_L, d_primary, p->ctrl, cs,
+        CKG(launch_gather_L(d_in, p->sa, p->blocks, learned ? p->tiles0 : p->tiles_seq(),
+                            learned ? p->ntiles0 : p->ntiles_seq(), d_L, d_primary, p->ctrl, cs,
                             learned ? p->route : nullptr, learned ? p->lgather : nullptr));
     }
     p->stats.kernel_launches++;

@@ -522,11 +522,11 @@ __global__ void __launch_bounds__(256) k_inv_replicate(InvCtx c, const TileDesc*
 
 template <typename PT>
 void launch_inv_sort(bwt_plan* p, const uint8_t* L, uint32_t* counter, PT* P, cudaStream_t st) {
-    const uint32_t nt = p->ntiles0;
-    const int sms = num_sms(), grid = std::max(1, std::min<int>((int)nt, sms * (p->tile >= 4096 ? 5 : 6)));
-    if (p->tile == 1024)
+    const uint32_t nt = p->ntiles_il;
+    const int sms = num_sms(), grid = std::max(1, std::min<int>((int)nt, sms * (p->rtile >= 4096 ? 5 : 6)));
+    if (p->rtile == 1024)
         k_inv_sort<PT, 1024><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles_il, nt, p->hist, p->status, counter, p->ctrl, P);
-    else if (p->tile == 2048)
+    else if (p->rtile == 2048)
         k_inv_sort<PT, 2048><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles_il, nt, p->hist, p->status, counter, p->ctrl, P);
     else
         k_inv_sort<PT, 4096><<<grid, 256, 0, st>>>(L, p->blocks, p->tiles_il, nt, p->hist, p->status, counter, p->ctrl, P);
@@ -583,7 +583,7 @@ extern "C" bwt_status bwt_inverse_batch(bwt_plan* p, const uint8_t* d_L, const u
     CKI(cudaMemsetAsync(p->hist, 0, sizeof(uint32_t) * 256 * nb, st));
     CKI(launch_hist_bytes(d_L, p->blocks, p->tiles0, nt, p->hist, st));
     CKI(launch_scan_rows(p->hist, 256, nullptr, 0, nb, nb, st));
-    CKI(cudaMemsetAsync(p->status, 0, sizeof(uint32_t) * (size_t)nt * 256, st));
+    CKI(cudaMemsetAsync(p->status, 0, sizeof(uint32_t) * (size_t)p->ntiles_il * 256, st));
     if (p32) launch_inv_sort<uint32_t>(p, d_L, counters, reinterpret_cast<uint32_t*>(p->keys[1]), st);
     else launch_inv_sort<uint64_t>(p, d_L, counters, p->keys[1], st);
     CKI(cudaGetLastError());

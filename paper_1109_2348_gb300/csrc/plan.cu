@@ -138,6 +138,7 @@ void bwt::free_plan_memory(bwt_plan* p) {
     FH(p->h_ctrl); FH(p->h_off);
     for (int s = 0; s < 2; ++s) {
         FH(p->stage_tiles[s]);
+        FH(p->stage_il[s]);
         FH(p->stage_blocks[s]);
         if (p->stage_ev[s]) cudaEventDestroy(p->stage_ev[s]);
     }
@@ -169,6 +170,8 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     p->desc.model_path = nullptr;
     p->rbits = desc->radix_bits ? desc->radix_bits : 8;
     p->tile = desc->tile_keys ? desc->tile_keys : 4096;
+    p->tile_auto = desc->tile_keys == 0;
+    p->rtile = p->tile;
     p->spin_limit = kDefaultSpin;
     const uint64_t N = desc->max_total_bytes;
     const uint32_t B = desc->max_blocks;
@@ -213,6 +216,7 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     }
     for (int sl = 0; sl < 2; ++sl) {
         A(host_alloc(&p->stage_tiles[sl], p->cap_tiles0));
+        A(host_alloc(&p->stage_il[sl], SMALL_TILES));
         A(host_alloc(&p->stage_blocks[sl], B));
         if (s == BWT_OK && cudaEventCreateWithFlags(&p->stage_ev[sl], cudaEventDisableTiming) != cudaSuccess)
             s = BWT_ECUDA;
@@ -223,6 +227,7 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     for (auto& ev : p->br_ev)
         if (s == BWT_OK && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) s = BWT_ECUDA;
     A(host_alloc(&p->h_off, (size_t)B + 1));
+    p->h_first.resize(std::min<uint32_t>(B, SMALL_TILES));
     A(host_alloc(&p->h_inv_items, 2 * ((size_t)B + 1)));
     // the learned bucketing's tables and the 16-bit passes' scratch, so that
     // no forward call allocates
@@ -315,6 +320,7 @@ extern "C" bwt_status bwt_plan_set_radix(bwt_plan* plan, int radix_bits, int til
     }
     plan->rbits = radix_bits;
     plan->tile = tile_keys;
+    plan->tile_auto = false;
     drop_graph(plan);
     return BWT_OK;
 }
@@ -381,6 +387,7 @@ bwt_status bwt::upload_tables(bwt_plan* p, const uint64_t* off, uint32_t nb, cud
     std::vector<uint64_t> key;
     key.reserve((size_t)nb + 3);
     key.push_back(T);
+    key.push_back(p->tile_auto ? 1u : 0u);
     key.push_back((uint64_t)p->rbits);  // 16-bit digits add the part table
     key.push_back(nb);
     key.insert(key.end(), off, off + nb + 1);
@@ -417,7 +424,39 @@ bwt_status bwt::upload_tables(bwt_plan* p, const uint64_t* off, uint32_t nb, cud
     p->ntiles0 = nt;
     CK(cudaMemcpyAsync(p->blocks, p->h_blocks, sizeof(BlockInfo) * nb, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(p->tiles0, p->h_tiles, sizeof(TileDesc) * nt, cudaMemcpyHostToDevice, st));
-    CK(launch_interleave_tiles(p->tiles0, nt, p->blocks, nb, T, p->tiles_il, st));
+    // A small batch takes tiles of 1,024 keys where the caller left the size
+    // open: with every tile in flight at once a pass is one tile's chain of
+    // phases, and a quarter of the keys is a shorter one (one 100,000-byte block:
+    // 190 -> 143 us a call; up to SMALL_TILES all tiles of a batch fit the GPU).
+    uint32_t small = 0;
+    if (p->tile_auto && p->rbits == 8)
+        for (uint32_t b = 0; b < nb && small <= SMALL_TILES; ++b)
+            small += (uint32_t)((off[b + 1] - off[b] + SMALL_RTILE - 1) / SMALL_RTILE);
+    if (small > 0 && small <= SMALL_TILES) {
+        TileDesc* il = p->stage_il[sl];
+        uint32_t k = 0, left = nb;
+        for (uint32_t b = 0, first = 0; b < nb; ++b) {  // first tiles, kept in the block's pinned entry below
+            p->h_first[b] = first;
+            first += (uint32_t)((off[b + 1] - off[b] + SMALL_RTILE - 1) / SMALL_RTILE);
+        }
+        for (uint32_t s = 0; left > 0; s += SMALL_RTILE) {  // tile 0 of every block, then tile 1, ...
+            left = 0;
+            for (uint32_t b = 0; b < nb; ++b) {
+                const uint32_t o = (uint32_t)off[b], n = (uint32_t)(off[b + 1] - off[b]);
+                if (s >= n) continue;
+                il[k++] = TileDesc{o + s, std::min(SMALL_RTILE, n - s), b, p->h_first[b], o, b, n,
+                                   p->h_first[b] + s / SMALL_RTILE};
+                ++left;
+            }
+        }
+        p->rtile = (int)SMALL_RTILE;
+        p->ntiles_il = k;
+        CK(cudaMemcpyAsync(p->tiles_il, il, sizeof(TileDesc) * k, cudaMemcpyHostToDevice, st));
+    } else {
+        p->rtile = p->tile;
+        p->ntiles_il = nt;
+        CK(launch_interleave_tiles(p->tiles0, nt, p->blocks, nb, T, p->tiles_il, st));
+    }
     p->nparts = 0;
     if (p->rbits == 16) {
         // parts of the 16-bit passes: up to PART16_KEYS consecutive rotations of one block
@@ -458,10 +497,10 @@ Bins bwt::bins_of(bwt_plan* p, int par) {
 // Records an event pair around a radix launch when timing is on.
 static cudaError_t timed_onesweep(bwt_plan* p, int key_bytes, bool from_s, const OneSweepParams& a,
                                   double bytes_per_key, uint64_t keys_host, int ctrl_keys_word, cudaStream_t st,
-                                  int radix_bits = 0, bool first_sort = false) {
+                                  int radix_bits, int tile, bool first_sort = false) {
     const bool timing = !p->events.empty() && !p->capturing && p->ev_used + 2 <= p->events.size();
     if (timing) cudaEventRecord(p->events[p->ev_used], st);
-    cudaError_t e = launch_onesweep(key_bytes, from_s, radix_bits ? radix_bits : p->rbits, p->tile, a, 0, st);
+    cudaError_t e = launch_onesweep(key_bytes, from_s, radix_bits, tile, a, 0, st);
     if (timing) {
         cudaEventRecord(p->events[p->ev_used + 1], st);
         EvMeta m;
@@ -480,7 +519,7 @@ static cudaError_t timed_onesweep(bwt_plan* p, int key_bytes, bool from_s, const
 
 bwt_status bwt::reset_ctrl(bwt_plan* p, cudaStream_t st) {
     p->lazy_ranks = LazyRanks{};  // every rank stored, unless a learned first stage says otherwise
-    CK(launch_reset_ctrl(p->ctrl, p->spin_limit, (uint32_t)p->withhold, p->ntiles0, st));
+    CK(launch_reset_ctrl(p->ctrl, p->spin_limit, (uint32_t)p->withhold, p->ntiles_il, st));
     p->stats.kernel_launches++;
     return BWT_OK;
 }
@@ -543,7 +582,7 @@ bwt_status bwt::enqueue_initial_sort(bwt_plan* p, const uint8_t* d_in, cudaStrea
     // 8-bit digits: every pass gets its own look-back region (8 x 256 words a
     // tile fit the status array), all zeroed by one memset; 11-bit passes
     // reuse one region, zeroed before each
-    const size_t region = (size_t)nt * RADIX;
+    const size_t region = (size_t)p->ntiles_il * RADIX;
     const bool one_memset = region * P <= p->cap_status;
     if (one_memset) CK(cudaMemsetAsync(p->status, 0, sizeof(uint32_t) * region * P, st));
     for (int ps = 0; ps < P; ++ps) {
@@ -565,7 +604,7 @@ bwt_status bwt::enqueue_initial_sort(bwt_plan* p, const uint8_t* d_in, cudaStrea
         a.tile_counter = ctrl + CTRL_TILE_CTR + ps;
         a.ctrl = ctrl;
         a.shift = ps * rb;
-        CK(timed_onesweep(p, 8, ps == 0, a, ps == 0 ? 13.0 : 24.0, p->total, -1, st, 0, true));
+        CK(timed_onesweep(p, 8, ps == 0, a, ps == 0 ? 13.0 : 24.0, p->total, -1, st, rb, p->rtile, true));
     }
     p->sa = p->vals[(P - 1) & 1];
     p->key2 = p->vals[P & 1];
@@ -579,7 +618,7 @@ bwt_status bwt::enqueue_initial_sort(bwt_plan* p, const uint8_t* d_in, cudaStrea
 bwt_status bwt::enqueue_naming(bwt_plan* p, const uint64_t* K, cudaStream_t st) {
     NvtxRange nv("name");
     CK(cudaMemsetAsync(p->ctrl + CTRL_BINS, 0, sizeof(uint32_t) * 2 * NCLS, st));
-    CK(launch_name_initial(K, p->sa, p->blocks, p->tiles0, p->ntiles0, p->rank, bins_of(p, 0), p->ctrl, st));
+    CK(launch_name_initial(K, p->sa, p->blocks, p->tiles_seq(), p->ntiles_seq(), p->rank, bins_of(p, 0), p->ctrl, st));
     p->stats.kernel_launches++;
     return BWT_OK;
 }
@@ -665,7 +704,7 @@ bwt_status bwt::enqueue_round(bwt_plan* p, int par, const uint32_t* host_counts,
             a.ctrl = ctrl;
             a.shift = ps * rb;
             a.seg_varied = p->seg_varied;  // groups whose key2 are all equal do not move
-            CK(timed_onesweep(p, 4, false, a, 16.0, 0, CTRL_LARGE_KEYS, ls, rb));
+            CK(timed_onesweep(p, 4, false, a, 16.0, 0, CTRL_LARGE_KEYS, ls, rb, p->tile));
         }
         p->pending_large_passes = (uint32_t)P2;
     }
@@ -801,7 +840,7 @@ bwt_status bwt::run_plain_host_loop(bwt_plan* p, const uint8_t* d_in, uint8_t* d
     if ((s = enqueue_initial_sort(p, d_in, st)) != BWT_OK) return s;
     if ((s = run_doubling_host_loop(p, st)) != BWT_OK) return s;
     NvtxRange nv("gather");
-    CK(launch_gather_L(d_in, p->sa, p->blocks, p->tiles0, p->ntiles0, d_L, d_primary, p->ctrl, st));
+    CK(launch_gather_L(d_in, p->sa, p->blocks, p->tiles_seq(), p->ntiles_seq(), d_L, d_primary, p->ctrl, st));
     p->stats.kernel_launches++;
     return BWT_OK;
 }

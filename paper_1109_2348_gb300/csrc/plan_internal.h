@@ -71,6 +71,10 @@ constexpr size_t kGraphCache = 4;
 
 }  // namespace bwt
 
+// Small batches (tile size left to the library): tiles of SMALL_RTILE keys while
+// there are at most SMALL_TILES of them, six an SM.
+constexpr uint32_t SMALL_RTILE = 1024, SMALL_TILES = 900;
+
 struct bwt_plan {
     int device = 0;
     bwt_plan_desc desc{};
@@ -92,7 +96,7 @@ struct bwt_plan {
     uint32_t* vals[2] = {nullptr, nullptr};
     uint32_t* rank = nullptr;
     bwt::TileDesc* tiles0 = nullptr;
-    bwt::TileDesc* tiles_il = nullptr;  // the same tiles, interleaved for the look-back passes
+    bwt::TileDesc* tiles_il = nullptr;  // tiles of rtile keys, interleaved, for the look-back passes
     bwt::TileDesc* ltiles = nullptr;
     bwt::BlockInfo* blocks = nullptr;
     uint32_t* hist = nullptr;
@@ -167,6 +171,15 @@ struct bwt_plan {
 
     // current batch
     uint32_t nb = 0, total = 0, max_n = 0, ntiles0 = 0;
+    uint32_t ntiles_il = 0;      // tiles in tiles_il
+    int rtile = 0;               // their keys: tile, or SMALL_RTILE for a small batch (upload_tables)
+    bool tile_auto = false;      // the caller left the tile size to the library
+    std::vector<uint32_t> h_first;  // small batches: first tile of every block
+    bwt::TileDesc* stage_il[2] = {nullptr, nullptr};  // pinned staging of small batches' tiles_il
+    // the tables of one tile a CTA's chain: naming and L gather take the small
+    // batch's tiles too
+    const bwt::TileDesc* tiles_seq() const { return rtile == tile ? tiles0 : tiles_il; }
+    uint32_t ntiles_seq() const { return rtile == tile ? ntiles0 : ntiles_il; }
     uint32_t* sa = nullptr;    // final SA buffer of the current batch
     uint32_t* key2 = nullptr;  // doubling keys, position-indexed
     uint32_t *kA = nullptr, *vA = nullptr, *kB = nullptr, *vB = nullptr;

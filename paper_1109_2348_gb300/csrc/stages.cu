@@ -943,7 +943,7 @@ extern "C" bwt_status bwt_vle_encode(bwt_plan* p, const uint8_t* d_in, const uin
     uint64_t* status = reinterpret_cast<uint64_t*>(p->status);
     CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * nt, st));
     k_vle_pack<<<std::max(1, std::min<int>(nt, sms * 6)), RT, VLE_SMEM, st>>>(
-        d_in, p->blocks, p->tiles_il, nt, d_code, d_len, d_byte_off, cap_words, reinterpret_cast<uint32_t*>(d_out), status,
+        d_in, p->blocks, p->rtile == p->tile ? p->tiles_il : p->tiles0, nt, d_code, d_len, d_byte_off, cap_words, reinterpret_cast<uint32_t*>(d_out), status,
         p->ctrl + CTRL_TILE_CTR, p->ctrl);
     CKS(cudaGetLastError());
     p->stats.kernel_launches = 5;

@@ -260,3 +260,49 @@ def test_vle_word_packing(longest, shift):
         assert int(bits[b]) == len(want)
         want = np.frombuffer(int(want.ljust(-(-len(want) // 8) * 8, "0"), 2).to_bytes(-(-len(want) // 8), "big"), np.uint8)
         assert np.array_equal(got[byte_off[b]:byte_off[b + 1]], want), f"block {b}"
+
+
+@pytest.mark.parametrize("flags", [0, F_GRAPH, F_LEARNED | F_GRAPH])
+def test_small_batch_tiles(flags):
+    """Batches around the largest that takes 1,024-key tiles (900 of them), a
+    call of each kind after the other on one plan, and its inverse."""
+    import torch
+    r = np.random.RandomState(71)
+    sets = [[900 * 1024], [899 * 1024 + 1, 1], [900 * 1024 + 1], [1] * 900, [2] * 901, [1023, 1024, 1025, 5000, 7],
+            [100_000]]
+    with Plan(max_blocks=1000, max_total_bytes=1_000_000, max_block_bytes=1_000_000, flags=flags) as plan:
+        if flags & F_LEARNED:
+            model.install(plan, model.equal_width_splitters())
+        for sizes in sets:
+            blocks = [r.randint(0, 60, n).astype(np.uint8) for n in sizes]
+            buf, off = batch_from_blocks(blocks)
+            L, prim, st = gpu_bwt(buf, off, plan)
+            assert st["tile_keys"] == 4096
+            assert_matches_oracle(buf, off, L, prim, str(sizes[:3]))
+            back = plan.inverse(torch.from_numpy(L).cuda(), off, torch.from_numpy(prim).cuda())
+            assert np.array_equal(back.cpu().numpy(), buf)
+
+
+def _group_blocks():
+    """Blocks whose 8-byte prefixes repeat m times each, for group sizes m at
+    the edges of the size classes, with sorted, reversed, equal and mixed
+    successors (what decides the order inside a group)."""
+    r = np.random.RandomState(81)
+    blocks = []
+    for m in (33, 64, 65, 72, 73, 255, 256, 257, 288, 289, 511, 1000, 2047, 2048, 2049):
+        for kind in range(3):
+            unit = r.randint(0, 256, 9).astype(np.uint8)
+            tails = r.randint(0, 256, (m, 6)).astype(np.uint8)
+            if kind == 1:
+                tails[:, :] = tails[0]
+            elif kind == 2:
+                tails[:, 0] = np.arange(m) // max(1, m // 7)
+            blocks.append(np.concatenate([np.concatenate([unit, t]) for t in tails]))
+    return blocks
+
+
+@pytest.mark.parametrize("flags", [0, F_GRAPH])
+def test_group_sorts_at_class_edges(flags):
+    buf, off = batch_from_blocks(_group_blocks())
+    L, prim, _ = gpu_bwt(buf, off, flags=flags)
+    assert_matches_oracle(buf, off, L, prim)
