@@ -86,6 +86,24 @@ bwt_status bwt::begin_if_capture(cudaStream_t st, cudaStream_t inner, cudaGraphC
     return e == cudaSuccess ? BWT_OK : record_cuda(e, "cudaStreamBeginCaptureToGraph");
 }
 
+// The capture's streams, kept by the plan: nine creations are most of what a
+// first call on new buffers spends beside the capture itself.
+cudaError_t bwt::create_capture_streams(bwt_plan* p) {
+    for (auto& s : p->cap_streams) {
+        if (s) continue;
+        const cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+void bwt::destroy_capture_streams(bwt_plan* p) {
+    for (auto& s : p->cap_streams) {
+        if (s) cudaStreamDestroy(s);
+        s = nullptr;
+    }
+}
+
 bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st) {
     const bool learned = (p->desc.flags & BWT_F_LEARNED) != 0;
     if (learned) {
@@ -102,7 +120,7 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     bwt_status status = BWT_OK;
     // capture streams: the main graph, the loop body, the body's second round,
     // and two branches of each
-    cudaStream_t cs = nullptr, bs = nullptr, rs = nullptr, br[6] = {};
+    cudaStream_t cs, bs, rs, *br;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t launched = nullptr;
@@ -115,10 +133,11 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     cudaGraph_t body, tmp;
     uint64_t k0, k1, k2, k3, k4, r0, r1, r3, r4;
 
-    CKG(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    CKG(cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking));
-    CKG(cudaStreamCreateWithFlags(&rs, cudaStreamNonBlocking));
-    for (auto& s : br) CKG(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    CKG(create_capture_streams(p));
+    cs = p->cap_streams[0];
+    bs = p->cap_streams[1];
+    rs = p->cap_streams[2];
+    br = p->cap_streams + 3;
     CKG(cudaGraphCreate(&g, 0));
     CKG(cudaGraphConditionalHandleCreate(&cond, g, 0, 0));
     p->capturing = true;
@@ -175,14 +194,6 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
     p->br[0] = p->br[1] = nullptr;
     CKG(cudaGraphInstantiate(&exec, g, 0));
     CKG(cudaEventCreateWithFlags(&launched, cudaEventDisableTiming));
-    cudaStreamDestroy(cs);
-    cudaStreamDestroy(bs);
-    cudaStreamDestroy(rs);
-    cs = bs = rs = nullptr;
-    for (auto& s : br) {
-        cudaStreamDestroy(s);
-        s = nullptr;
-    }
     {
         // the least recently used graph makes room (its last launch may still run)
         if (p->graphs.size() >= kGraphCache) {
@@ -217,14 +228,11 @@ bwt_status bwt::run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_
 fail:
     p->capturing = false;
     p->br[0] = p->br[1] = nullptr;
-    for (cudaStream_t s : {rs, bs, cs}) {  // innermost captures first
-        if (!s) continue;
+    for (int i : {2, 1, 0}) {  // innermost captures first; the branches' end with them
         cudaGraph_t t = nullptr;
-        cudaStreamEndCapture(s, &t);
-        cudaStreamDestroy(s);
+        if (p->cap_streams[i]) cudaStreamEndCapture(p->cap_streams[i], &t);
     }
-    for (cudaStream_t s : br)  // their captures ended with the streams they branched from
-        if (s) cudaStreamDestroy(s);
+    destroy_capture_streams(p);  // a later call starts from fresh ones
     if (launched) cudaEventDestroy(launched);
     if (exec) cudaGraphExecDestroy(exec);
     if (g) cudaGraphDestroy(g);

@@ -594,10 +594,18 @@ __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__
 // staged bytes on the way out), so each chunk's share of the tile is written
 // as one run, at a slot range reserved with one atomic per tile and chunk.
 // Values written to packed chunks carry their bucket's tag (CM_OWN above).
-constexpr size_t CHUNK_SCATTER_SMEM = NBK * 2 + 4 * MAXCH * 4 + TILE_BYTES + 4096 * 4;
+// 512 threads take up to 8,192 rotations of a block at once (two 4,096-key
+// tiles): the scan over the chunks and the slot reservations are paid once for
+// both and a chunk's runs are twice as long (30 rotations on 900,000-byte
+// blocks). Per 240 blocks the call took 5,118 us with 256 threads and 4,096
+// rotations, 4,990 with this; 512 x 12 rotations a thread 5,174, x 20 5,025, x 24
+// 5,001, three CTAs 5,118 (spills), 1,024 x 8 5,256, 1,024 x 16 5,106.
+constexpr int SC_NT = 512, SC_ITEMS = 16, SC_CTAS = 2;
+template <int NT, int ITEMS>
+constexpr size_t CHUNK_SCATTER_SMEM = NBK * 2 + 4 * MAXCH * 4 + (NT * ITEMS + 48) + NT * ITEMS * 4;
 
-template <int ITEMS>
-__global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restrict__ S,
+template <int NT, int ITEMS, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __restrict__ S,
                                                        const BlockInfo* __restrict__ blocks,
                                                        const TileDesc* __restrict__ tiles,
                                                        const uint32_t* __restrict__ ntiles_dev,
@@ -607,12 +615,12 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
                                                        uint32_t* err) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint8_t* sb = smem;                                                  // [TILE_BYTES], 16-aligned
-    uint16_t* cm = reinterpret_cast<uint16_t*>(smem + TILE_BYTES);       // [NBK] chunk of each bucket
+    uint16_t* cm = reinterpret_cast<uint16_t*>(smem + NT * ITEMS + 48);  // [NBK] chunk of each bucket
     uint32_t* cb = reinterpret_cast<uint32_t*>(cm + NBK);                // [MAXCH] chunk starts (block-relative)
     uint32_t* lcount = cb + MAXCH;                                       // [MAXCH] tile's rotations per chunk
     uint32_t* pre = lcount + MAXCH;                                      // [MAXCH] tile-local chunk offsets
     uint32_t* dbase = pre + MAXCH;                                       // [MAXCH] destination of pre[c]
-    uint32_t* stQC = dbase + MAXCH;  // [4096] by rank: tile position (low 16 bits) | fine bucket (high 16)
+    uint32_t* stQC = dbase + MAXCH;  // [NT * ITEMS] by rank: position (low 16 bits) | fine bucket (high 16)
     __shared__ uint32_t scan_tmp[32];
     __shared__ uint8_t s_before;  // the byte before the tile's first rotation
     const uint32_t ntiles = *ntiles_dev;
@@ -624,7 +632,14 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
         BlockInfo bi{};     // of block cur, with its route: read once a block, so a
         bool flat = false;  // tile's loads wait only on its own descriptor
         for (uint32_t t = t0; t < t1; ++t) {
-            const TileDesc td = tiles[t];
+            TileDesc td = tiles[t];
+            // consecutive tiles of a block are one unit as long as they fit
+            while (t + 1 < t1 && td.len < (uint32_t)(NT * ITEMS)) {
+                const TileDesc nx = tiles[t + 1];
+                if (nx.blk != td.blk || td.len + nx.len > (uint32_t)(NT * ITEMS)) break;
+                td.len += nx.len;
+                ++t;
+            }
             if (td.blk != cur) {  // CTA-uniform
                 cur = td.blk;
                 bi = blocks[cur];
@@ -638,11 +653,11 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
             if (!flat) {
 #pragma unroll
                 for (int j = 0; j < ITEMS; ++j) {
-                    const uint32_t q = j * 256 + threadIdx.x;
+                    const uint32_t q = j * NT + threadIdx.x;
                     bk[j] = q < td.len ? (uint32_t)fb[td.start + q] : 0u;
                 }
             }
-            const uint32_t shift = stage_tile_bytes(S, bi, i0, td.len, sb, threadIdx.x, 256);
+            const uint32_t shift = stage_tile_bytes(S, bi, i0, td.len, sb, threadIdx.x, NT);
             if (threadIdx.x == 0) s_before = S[bi.off + (i0 ? i0 : bi.n) - 1];
             __syncthreads();
             // chunk (low 10 bits) | slot within the tile's share of the chunk << 10;
@@ -651,7 +666,7 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
             uint32_t cs[ITEMS];
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) {
-                const uint32_t q = j * 256 + threadIdx.x;
+                const uint32_t q = j * NT + threadIdx.x;
                 cs[j] = 0xffffffffu;
                 if (q < td.len) {
                     if (flat) bk[j] = (uint32_t)(pack8_smem(sb, shift + q) >> 52);
@@ -665,7 +680,7 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
             // the global reservation (issued first: its round trip overlaps
             // the scan) and the tile-local exclusive prefix over chunks
             {
-                constexpr int PER = MAXCH / 256;
+                constexpr int PER = MAXCH / NT;
                 uint32_t v[PER], g[PER], sum = 0;
 #pragma unroll
                 for (int i = 0; i < PER; ++i) {
@@ -674,7 +689,7 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
                     sum += v[i];
                 }
                 uint32_t total;
-                uint32_t ex = block_exclusive_scan<256>(sum, scan_tmp, &total);
+                uint32_t ex = block_exclusive_scan<NT>(sum, scan_tmp, &total);
 #pragma unroll
                 for (int i = 0; i < PER; ++i) {
                     const uint32_t c = threadIdx.x * PER + i;
@@ -689,7 +704,7 @@ __global__ void __launch_bounds__(256, 4) k_chunk_scatter(const uint8_t* __restr
                 if (cs[j] != 0xffffffffu) {
                     const uint32_t c = cs[j] & (MAXCH - 1);
                     const uint32_t pos = (pre[c] & ~CB_WIDE) + (cs[j] >> 10);
-                    stQC[pos] = (j * 256 + threadIdx.x) | (bk[j] << 16);
+                    stQC[pos] = (j * NT + threadIdx.x) | (bk[j] << 16);
                 }
             }
             __syncthreads();
@@ -1433,16 +1448,14 @@ bwt_status bwt::enqueue_learned(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, 
     k_chunk_plan<<<std::min<uint32_t>(nb, 65535), 256, 0, st>>>(p->bucket_count, p->blocks, p->route, p->splitters, nb,
                                                                 ct, aux, p->lgather, ctrl);
     {
-        const int g = sms * 4;
-        if (T <= 1024)
-            k_chunk_scatter<4><<<g, 256, CHUNK_SCATTER_SMEM, st>>>(d_in, p->blocks, tilesB, ntb, fb, p->route, ct,
-                                                                   p->keys[0], p->vals[0], ctrl + CTRL_ERR);
-        else if (T <= 2048)
-            k_chunk_scatter<8><<<g, 256, CHUNK_SCATTER_SMEM, st>>>(d_in, p->blocks, tilesB, ntb, fb, p->route, ct,
-                                                                   p->keys[0], p->vals[0], ctrl + CTRL_ERR);
-        else
-            k_chunk_scatter<16><<<g, 256, CHUNK_SCATTER_SMEM, st>>>(d_in, p->blocks, tilesB, ntb, fb, p->route, ct,
-                                                                    p->keys[0], p->vals[0], ctrl + CTRL_ERR);
+        static const int ctas = [] {
+            cudaFuncSetAttribute((void*)k_chunk_scatter<SC_NT, SC_ITEMS, SC_CTAS>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)CHUNK_SCATTER_SMEM<SC_NT, SC_ITEMS>);
+            return SC_CTAS;
+        }();
+        k_chunk_scatter<SC_NT, SC_ITEMS, SC_CTAS><<<sms * ctas, SC_NT, CHUNK_SCATTER_SMEM<SC_NT, SC_ITEMS>, st>>>(
+            d_in, p->blocks, tilesB, ntb, fb, p->route, ct, p->keys[0], p->vals[0], ctrl + CTRL_ERR);
     }
     CKL(cudaGetLastError());
     p->stats.kernel_launches += 4;

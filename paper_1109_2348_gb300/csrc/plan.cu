@@ -145,6 +145,7 @@ void bwt::free_plan_memory(bwt_plan* p) {
     if (p->done_ev) cudaEventDestroy(p->done_ev);
     for (auto& ev : p->br_ev)
         if (ev) cudaEventDestroy(ev);
+    destroy_capture_streams(p);
     FH(p->h_route); FH(p->h_bstats); FH(p->h_inv_items);
     for (auto& e : p->events) cudaEventDestroy(e);
     p->events.clear();
@@ -233,6 +234,7 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     // no forward call allocates
     if (s == BWT_OK && (desc->flags & BWT_F_LEARNED)) s = ensure_learned_buffers(p);
     if (s == BWT_OK && p->rbits == 16) s = ensure_radix16(p);
+    if (s == BWT_OK && (desc->flags & BWT_F_GRAPH) && create_capture_streams(p) != cudaSuccess) s = BWT_ECUDA;
     p->device_bytes = total;
     if (s == BWT_OK && (desc->flags & BWT_F_TIMING)) {
         p->events.resize(512);
@@ -810,14 +812,14 @@ bwt_status bwt::run_doubling_host_loop(bwt_plan* p, cudaStream_t st) {
         CK(cudaMemcpyAsync(p->h_ctrl, p->ctrl, sizeof(uint32_t) * 24, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         resolve_large_keys(p, p->h_ctrl[CTRL_LARGE_KEYS]);
-        if (p->h_ctrl[CTRL_ERR]) break;
+        if (p->h_ctrl[CTRL_ERR]) return BWT_OK;
         uint32_t counts[NCLS];
         uint64_t any = 0;
         for (int c = 0; c < NCLS; ++c) {
             counts[c] = std::min(p->h_ctrl[CTRL_BINS + NCLS * par + c], p->bincap[c]);
             any += counts[c];
         }
-        if (any == 0) break;
+        if (any == 0) return BWT_OK;  // the words read here are the last round's
         bwt_status s = enqueue_round(p, par, counts, st);
         if (s != BWT_OK) return s;
         CK(launch_round_end(p->ctrl, par, p->max_n, 0, 0, 0, st));  // advance the depth only

@@ -202,6 +202,8 @@ struct bwt_plan {
     bool capturing = false;
     cudaStream_t br[2] = {nullptr, nullptr};    // branch streams of the round being captured (graph.cu)
     cudaEvent_t br_ev[2] = {nullptr, nullptr};
+    // main graph, loop body, the body's second round, then two branches of each
+    cudaStream_t cap_streams[9] = {};
 
     bwt_stats stats{};
     bwt_status last = BWT_OK;
@@ -236,6 +238,8 @@ void collect_timing(bwt_plan* p);
 bwt_status run_plain_host_loop(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st);
 bwt_status run_doubling_host_loop(bwt_plan* p, cudaStream_t st);
 bwt_status run_per_block(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st);
+cudaError_t create_capture_streams(bwt_plan* p);
+void destroy_capture_streams(bwt_plan* p);
 bwt_status run_graph(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st);
 bwt_status run_learned(bwt_plan* p, const uint8_t* d_in, uint8_t* d_L, int32_t* d_primary, cudaStream_t st);
 // Learned first stage (bucket count, device-side routing, scatter, chunk sorts

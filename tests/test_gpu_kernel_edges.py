@@ -306,3 +306,20 @@ def test_group_sorts_at_class_edges(flags):
     buf, off = batch_from_blocks(_group_blocks())
     L, prim, _ = gpu_bwt(buf, off, flags=flags)
     assert_matches_oracle(buf, off, L, prim)
+
+
+@pytest.mark.parametrize("tile", [1024, 2048, 4096])
+def test_scatter_units_of_several_tiles(tile):
+    """The chunk scatter takes consecutive tiles of a block as one unit of up
+    to 8,192 rotations: blocks around that size and its multiples, in a batch
+    large enough that a CTA gets several tiles (an equal-width table)."""
+    r = np.random.RandomState(91)
+    sizes = [8191, 8192, 8193, 4097, 12_288, 16_385, 24_577, 40_000] * 6 + [1] * 40 + [2_500_000 // 8] * 30
+    blocks = [r.randint(0, 256, n).astype(np.uint8) for n in sizes]
+    buf, off = batch_from_blocks(blocks)
+    with Plan(max_blocks=len(sizes), max_total_bytes=buf.size, max_block_bytes=max(sizes), tile_keys=tile,
+              flags=F_LEARNED | F_GRAPH) as plan:
+        model.install(plan, model.equal_width_splitters())
+        L, prim, st = gpu_bwt(buf, off, plan)
+    assert st["blocks_routed_plain"] == 0
+    assert_matches_oracle(buf, off, L, prim, f"tile {tile}")
