@@ -1079,7 +1079,9 @@ cudaError_t launch_gather_L(const uint8_t* S, const uint32_t* SA, const BlockInf
 
 // ---- control kernels --------------------------------------------------------
 
-__global__ void k_reset_ctrl(uint32_t* ctrl, uint32_t spin, uint32_t withhold, uint32_t ntiles0) {
+__global__ void k_reset_ctrl(uint32_t* ctrl, uint32_t spin, uint32_t withhold, uint32_t ntiles0,
+                             uint32_t* __restrict__ zero, uint32_t words) {
+    for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) zero[i] = 0u;
     for (int i = threadIdx.x; i < CTRL_WORDS; i += blockDim.x) ctrl[i] = 0u;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1139,8 +1141,9 @@ cudaError_t launch_words_to_host(uint32_t* host_dst_dev_ptr, const uint32_t* src
     return cudaGetLastError();
 }
 
-cudaError_t launch_reset_ctrl(uint32_t* ctrl, uint32_t spin, uint32_t withhold, uint32_t ntiles0, cudaStream_t st) {
-    k_reset_ctrl<<<1, 128, 0, st>>>(ctrl, spin, withhold, ntiles0);
+cudaError_t launch_reset_ctrl(uint32_t* ctrl, uint32_t spin, uint32_t withhold, uint32_t ntiles0, cudaStream_t st,
+                              uint32_t* zero, uint32_t words) {
+    k_reset_ctrl<<<1, words > 128 ? 512 : 128, 0, st>>>(ctrl, spin, withhold, ntiles0, zero, words);
     return cudaGetLastError();
 }
 

@@ -160,7 +160,8 @@ cudaError_t launch_rename_large(const uint32_t* SA, const uint32_t* key2, uint32
 
 // Control words: reset before a batch; advance after a round (and set the
 // graph loop condition); set the condition before the loop.
-cudaError_t launch_reset_ctrl(uint32_t* ctrl, uint32_t spin, uint32_t withhold, uint32_t ntiles0, cudaStream_t st);
+cudaError_t launch_reset_ctrl(uint32_t* ctrl, uint32_t spin, uint32_t withhold, uint32_t ntiles0, cudaStream_t st,
+                              uint32_t* zero = nullptr, uint32_t words = 0);
 
 // Copies `words` u32 from device memory to pinned host memory, written by a
 // kernel (host_dst_dev_ptr: the device view of the host buffer), so that no

@@ -519,9 +519,11 @@ static cudaError_t timed_onesweep(bwt_plan* p, int key_bytes, bool from_s, const
     return e;
 }
 
-bwt_status bwt::reset_ctrl(bwt_plan* p, cudaStream_t st) {
+// Sets the control words for a call and clears `words` further words (a few
+// hundred look-back words: no launch of their own).
+bwt_status bwt::reset_ctrl(bwt_plan* p, cudaStream_t st, uint32_t* zero, uint32_t words) {
     p->lazy_ranks = LazyRanks{};  // every rank stored, unless a learned first stage says otherwise
-    CK(launch_reset_ctrl(p->ctrl, p->spin_limit, (uint32_t)p->withhold, p->ntiles_il, st));
+    CK(launch_reset_ctrl(p->ctrl, p->spin_limit, (uint32_t)p->withhold, p->ntiles_il, st, zero, words));
     p->stats.kernel_launches++;
     return BWT_OK;
 }

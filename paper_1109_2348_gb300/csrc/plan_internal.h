@@ -218,7 +218,7 @@ bwt_status prepare_batch(bwt_plan* p, const uint64_t* offsets, uint32_t nb, cuda
 bwt_status upload_tables(bwt_plan* p, const uint64_t* off, uint32_t nb, cudaStream_t st);
 Bins bins_of(bwt_plan* p, int par);
 int round_radix_bits(const bwt_plan* p);
-bwt_status reset_ctrl(bwt_plan* p, cudaStream_t st);
+bwt_status reset_ctrl(bwt_plan* p, cudaStream_t st, uint32_t* zero = nullptr, uint32_t words = 0);
 bwt_status enqueue_initial_sort(bwt_plan* p, const uint8_t* d_in, cudaStream_t st);
 // One doubling round on bins[par]; records the kernels and radix passes of
 // its large-group section (cap_large_kernels, cap_large_radix).

@@ -20,12 +20,12 @@
 // them (one pass over the bytes, one over the chunks), and a warp encodes 32
 // bytes of a chunk at once (below).
 //
-// GB300 layout: the prefix sums are single passes over 4,096-element tiles
-// (256 threads x 16) with decoupled look-back between tiles, so each of the
-// steps reads and writes every element once; tiles start in order from a
-// tile counter. A tile's codewords are packed into 32-bit words in shared
-// memory and stored whole; only the two words a tile shares with its
-// neighbours are merged with atomic ORs.
+// GB300 layout: tiles are 4,096 elements (256 threads x 16). The run-length
+// prefix sums take two passes (sums by spans, then the tiles); the codeword
+// offsets a single pass with decoupled look-back between a block's tiles. A
+// tile's codewords are packed into 32-bit words in shared memory and stored
+// whole; only the two words a tile shares with its neighbours are merged with
+// atomic ORs.
 #include <algorithm>
 #include <cstring>
 
@@ -65,16 +65,40 @@ __device__ __forceinline__ uint32_t next_tile(uint32_t* s_tile, uint32_t* counte
     return t;
 }
 
-// The 16 bytes at S[t0 + 16 tid ..] of a tile of `len` bytes, as four words:
-// one 16-byte load where the tile is whole and aligned, else through sb
-// (RTILE bytes, 16-byte aligned; bytes past the tile are undefined). All
-// threads call; sb is free again after the next barrier.
-__device__ __forceinline__ uint4 tile_words(const uint8_t* __restrict__ S, uint32_t t0, uint32_t len, uint8_t* sb) {
-    if (len == RTILE && (reinterpret_cast<uintptr_t>(S + t0) & 15u) == 0u)
-        return __ldg(reinterpret_cast<const uint4*>(S + t0) + threadIdx.x);
-    for (uint32_t q = threadIdx.x; q < len; q += RT) sb[q] = S[t0 + q];
+// ---- tile prefixes of the run-length stages -----------------------------------
+//
+// The prefix sums run in two passes: every tile's sum, with the tiles' prefixes
+// by spans -- a span of consecutive tiles a CTA, at most four CTAs an SM, with
+// decoupled look-back between spans -- and then the tiles, which wait for
+// nothing. With the look-back between the tiles themselves (one pass, 1,200
+// tiles in flight polling each other's words) 64 mixed blocks took 147 us for
+// encoding and 147 for the lengths of decoding; with spans 42 + 75 and 43 + 50.
+// (Tried for one pass: 128 words a look-back step, a CTA-wide look-back,
+// 16,384-byte tiles: no faster. Two or eight spans an SM: 204 and 176 us a call
+// where four took 179.) The second passes launch several tiles' worth of CTAs
+// an SM: their tiles differ in work (encoding 161 us a call with 8, 152 with 48).
+
+// Turns sums[t] of the span's tiles [t0, t1) into their exclusive prefixes over
+// all tiles (mod 2^32). All RT threads call.
+__device__ __forceinline__ void span_prefixes(uint32_t* sums, uint32_t t0, uint32_t t1, uint64_t* status, uint32_t span,
+                                              uint32_t spin, uint32_t withhold, uint32_t* ctrl, uint32_t* scan_tmp,
+                                              uint64_t* s_excl) {
+    __syncthreads();  // the sums are written
+    uint64_t run = 0;
+    for (uint32_t base = t0; base < t1; base += RT) {
+        const uint32_t t = base + threadIdx.x;
+        uint32_t total;
+        const uint32_t ex = block_exclusive_scan<RT>(t < t1 ? sums[t] : 0u, scan_tmp, &total);
+        if (t < t1) sums[t] = (uint32_t)run + ex;
+        run += total;
+    }
+    if (threadIdx.x < 32) {
+        const uint64_t e = lookback_u64(status, span, 0, run & LB_VAL, spin, &ctrl[CTRL_ERR], withhold);
+        if (threadIdx.x == 0) *s_excl = e;
+    }
     __syncthreads();
-    return reinterpret_cast<const uint4*>(sb)[threadIdx.x];
+    const uint32_t e = (uint32_t)*s_excl;
+    for (uint32_t t = t0 + threadIdx.x; t < t1; t += RT) sums[t] += e;
 }
 
 // Bit j: byte j of a and of b differ.
@@ -82,102 +106,180 @@ __device__ __forceinline__ uint32_t bytes_differ(uint32_t a, uint32_t b) {
     return (__vsetne4(a, b) * 0x01020408u) >> 24;
 }
 
-// The last run end before tile t, from the tiles' published ones (`tail`:
-// LB_INC | end index, 0 for a tile without one, per tile; zero = not yet
-// published): the nearest tile with one, 32 tiles a step. 0 before the first.
-// All 32 lanes of a warp call; bounded like the look-back.
-__device__ __forceinline__ uint32_t last_end_before(const uint64_t* tail, uint32_t t, uint32_t spin_limit, uint32_t* err) {
+// Run ends among the 16 bytes v at global position i0 (bit j: byte j ends a
+// run), given the byte after them: the byte differs from the next one or is its
+// block's last. `len` bytes of the tile at t0 are real; b0 is the block of t0,
+// bend0 its end. With another block inside the tile, `starts` gets the bytes
+// that start one (bit j), and b the block of i0.
+__device__ __forceinline__ uint32_t run_ends(uint4 v, uint32_t after, uint32_t i0, uint32_t t0, uint32_t len, uint32_t N,
+                                             const BlockInfo* __restrict__ blocks, uint32_t nb, uint32_t b0,
+                                             uint32_t bend0, uint32_t& starts, uint32_t& b) {
+    uint32_t flags = bytes_differ(v.x, __funnelshift_r(v.x, v.y, 8)) |
+                     bytes_differ(v.y, __funnelshift_r(v.y, v.z, 8)) << 4 |
+                     bytes_differ(v.z, __funnelshift_r(v.z, v.w, 8)) << 8 |
+                     bytes_differ(v.w, __funnelshift_r(v.w, after, 8)) << 12;
+    const uint32_t q0 = i0 - t0;
+    starts = 0u;
+    b = b0;
+    if (bend0 < t0 + len) {  // uniform over the tile: another block starts in it
+        b = i0 < N ? block_at(blocks, nb, i0) : 0u;
+        uint32_t bb = b, bend = i0 < N ? blocks[b].off + blocks[b].n : 0u;
+        if (i0 < N && blocks[b].off == i0) starts |= 1u;
+#pragma unroll
+        for (int j = 0; j < RI; ++j) {
+            if (i0 + j >= N) break;
+            if (i0 + j == bend) {
+                ++bb;
+                bend = blocks[bb].off + blocks[bb].n;
+                starts |= 1u << j;
+            }
+            if (i0 + j + 1 == bend) flags |= 1u << j;
+        }
+    } else {
+        if (i0 == t0 && blocks[b0].off == t0) starts = 1u;
+        if (bend0 == t0 + len && bend0 - 1 - i0 < (uint32_t)RI) flags |= 1u << (bend0 - 1 - i0);
+    }
+    if (q0 + RI > len) flags &= q0 < len ? (1u << (len - q0)) - 1u : 0u;
+    return flags;
+}
+
+// The 16 bytes at S[i], i + 16 <= N or bytes past N undefined (zero): one load
+// where aligned.
+__device__ __forceinline__ uint4 load16(const uint8_t* __restrict__ S, uint32_t i, uint32_t N) {
+    if ((uint64_t)i + 16 <= N && (reinterpret_cast<uintptr_t>(S + i) & 15u) == 0u)
+        return __ldg(reinterpret_cast<const uint4*>(S + i));
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+        if ((uint64_t)i + j < N) w[j / 4] |= (uint32_t)S[i + j] << (8 * (j % 4));
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Tiles of a batch so small that the second pass finds its own prefixes, a warp
+// an earlier tile, and the first is left out: a launch and a look-back less (one
+// 30,000-byte batch: 50.0 -> 39.9 us a call).
+constexpr uint32_t FEW_TILES = RT / 32;
+
+// A tile's number of run ends and its last one (end index, 0: none), by a warp.
+__device__ __forceinline__ void tile_run_ends(const uint8_t* __restrict__ S, uint32_t N,
+                                              const BlockInfo* __restrict__ blocks, uint32_t nb, uint32_t t,
+                                              uint32_t& cnt, uint32_t& end) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t p0 = t * RTILE, len = min(RTILE, N - p0);
+    const uint32_t b0 = block_at(blocks, nb, p0), bend0 = blocks[b0].off + blocks[b0].n;
+    cnt = end = 0;
+#pragma unroll 4
+    for (uint32_t q = lane * 16; q < RTILE; q += 512) {
+        const uint32_t i0 = p0 + q;
+        const uint4 v = load16(S, i0, N);
+        uint32_t after = __shfl_down_sync(0xffffffffu, v.x, 1);
+        if (lane == 31) after = (uint64_t)i0 + 16 < N ? S[i0 + 16] : 0u;
+        uint32_t starts, b;
+        const uint32_t f = run_ends(v, after, i0, p0, len, N, blocks, nb, b0, bend0, starts, b);
+        cnt += __popc(f);
+        if (f) end = i0 + 32u - __clz(f);
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    end = __reduce_max_sync(0xffffffffu, end);
+}
+
+// Encode, sums: every tile's run ends, a warp a tile; then the tiles' prefixes.
+__global__ void __launch_bounds__(RT) k_rle_sums(const uint8_t* __restrict__ S, uint32_t N,
+                                                 const BlockInfo* __restrict__ blocks, uint32_t nb,
+                                                 uint32_t* __restrict__ sums, uint32_t* __restrict__ last,
+                                                 uint64_t* __restrict__ status, uint32_t* __restrict__ counter,
+                                                 uint32_t* ctrl) {
+    __shared__ uint32_t s_span, scan_tmp[32];
+    __shared__ uint64_t s_excl;
+    const uint32_t ntiles = (N + RTILE - 1) / RTILE, per = (ntiles + gridDim.x - 1) / gridDim.x;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t span = next_tile(&s_span, counter);  // in start order, so that earlier spans are in flight
+    const uint32_t t0 = min(ntiles, span * per), t1 = min(ntiles, t0 + per);
+    for (uint32_t t = t0 + warp; t < t1; t += RT / 32) {
+        uint32_t cnt, end;
+        tile_run_ends(S, N, blocks, nb, t, cnt, end);
+        if (lane == 0) {
+            sums[t] = cnt;
+            last[t] = end;
+        }
+    }
+    span_prefixes(sums, t0, t1, status, span, ctrl[CTRL_SPIN], ctrl[CTRL_WITHHOLD], ctrl, scan_tmp, &s_excl);
+}
+
+// The last run end before tile t: the nearest earlier tile with one, 32 tiles a
+// step (a warp calls); 0 before the first.
+__device__ __forceinline__ uint32_t last_end_before(const uint32_t* __restrict__ last, uint32_t t) {
     const uint32_t lane = threadIdx.x & 31;
     for (uint32_t end = t; end > 0; end = end > 32 ? end - 32 : 0) {
-        uint64_t v = 0;
-        if (lane < end) {
-            uint32_t it = 0;
-            while (((v = ld_volatile64(tail + (end - 1 - lane))) & LB_INC) == 0ull) {
-                if (++it > spin_limit) {
-                    atomicOr(err, ERR_TIMEOUT);
-                    break;
-                }
-                if (it > 32) __nanosleep(64);
-            }
-        }
-        const uint32_t m = __ballot_sync(0xffffffffu, (uint32_t)v != 0u);
-        if (m) return __shfl_sync(0xffffffffu, (uint32_t)v, __ffs(m) - 1);
+        const uint32_t v = lane < end ? last[end - 1 - lane] : 0u;
+        const uint32_t m = __ballot_sync(0xffffffffu, v != 0u);
+        if (m) return __shfl_sync(0xffffffffu, v, __ffs(m) - 1);
     }
     return 0u;
 }
 
-// Encode, one pass: run-end flags, their prefix sum (block scan and look-back
-// over the tiles), and every run's byte and length -- the difference of
-// consecutive end indices -- compacted through shared memory so that they are
-// written in rows. run_off[b] = the first run of block b (run_off[nb] = the
-// number of runs). 64 mixed blocks (57.6 MB, 38.5 M runs): 388 us with byte
-// loads and every thread writing its own runs, and 72 us for a second pass
-// over the end indices -> 147 us. Bound by the look-back: 1,200 tiles in
-// flight poll each other's words. Measured for the whole call (177 us): the
-// look-back by 128 words a warp 211, by the whole CTA 204, tiles of 16,384
-// bytes 181, five CTAs an SM 244.
+// Encode: run-end flags and their block scan give every run its slot; the runs'
+// bytes and lengths -- the differences of consecutive end indices -- are
+// compacted through shared memory so that they are written in rows.
+// run_off[b] = the first run of block b (run_off[nb] = the number of runs). 64
+// mixed blocks (57.6 MB, 38.5 M runs): 388 us at first, with byte loads and
+// every thread writing its own runs, and 72 us for a pass over the end indices;
+// 104 us with entries written one a thread, 75 four a thread.
 __global__ void __launch_bounds__(RT) k_rle_encode(const uint8_t* __restrict__ S, uint32_t N,
                                                    const BlockInfo* __restrict__ blocks, uint32_t nb,
+                                                   const uint32_t* __restrict__ first, const uint32_t* __restrict__ last,
                                                    uint8_t* __restrict__ chars, uint32_t* __restrict__ lens,
-                                                   uint64_t* __restrict__ run_off, uint64_t* __restrict__ status,
-                                                   uint64_t* __restrict__ tail, uint32_t* __restrict__ counter,
-                                                   uint32_t* ctrl) {
-    __shared__ __align__(16) uint8_t sb[RTILE];  // staged bytes, then the tile's run bytes
-    __shared__ uint16_t se[RTILE];               // the runs' end positions in the tile
-    __shared__ uint8_t s_first[RT / 32 + 1];     // each warp's first byte (and the next tile's)
-    __shared__ uint32_t s_tile, s_last, s_prev, scan_tmp[32];
-    __shared__ uint64_t s_excl;
+                                                   uint64_t* __restrict__ run_off, uint32_t* ctrl) {
+    // the tile's run bytes and end positions, from index k0 mod 4 on: a group
+    // of four entries has the alignment of its place in the outputs
+    __shared__ __align__(4) uint8_t sb[RTILE + 4];
+    __shared__ __align__(8) uint16_t se[RTILE + 4];
+    __shared__ uint8_t s_first[RT / 32 + 1];  // each warp's first byte (and the next tile's)
+    __shared__ uint32_t s_prev, s_few[2 * RT / 32], scan_tmp[32];
+    if (ld_volatile(&ctrl[CTRL_ERR])) return;  // a wait of the sums ran out: the prefixes are not to be used
     const uint32_t ntiles = (N + RTILE - 1) / RTILE;
-    const uint32_t spin = ctrl[CTRL_SPIN], withhold = ctrl[CTRL_WITHHOLD];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (;;) {
-        const uint32_t t = next_tile(&s_tile, counter);
-        if (t >= ntiles) break;
+    const bool vec = (reinterpret_cast<uintptr_t>(chars) & 3u) == 0u && (reinterpret_cast<uintptr_t>(lens) & 15u) == 0u;
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const uint32_t t0 = t * RTILE, len = min(RTILE, N - t0);
-        const uint4 v = tile_words(S, t0, len, sb);
+        const uint32_t q0 = threadIdx.x * RI, i0 = t0 + q0;
+        const uint4 v = load16(S, i0, N);
+        uint32_t k0 = 0;
         const uint32_t b0 = block_at(blocks, nb, t0), bend0 = blocks[b0].off + blocks[b0].n;
-        if (lane == 0) s_first[warp] = (uint8_t)v.x;
-        if (threadIdx.x == 0) {
-            s_first[RT / 32] = t0 + len < N ? S[t0 + len] : (uint8_t)0;
-            s_last = 0u;
+        if (first) {
+            k0 = first[t];
+            if (warp == 1) {
+                const uint32_t e = last_end_before(last, t);
+                if (lane == 0) s_prev = e;
+            }
+        } else {  // few tiles: warp w counts tile w
+            uint32_t cnt = 0, end = 0;
+            if (warp < t) tile_run_ends(S, N, blocks, nb, warp, cnt, end);
+            if (lane == 0) {
+                s_few[warp] = cnt;
+                s_few[RT / 32 + warp] = end;
+            }
+            __syncthreads();
+            uint32_t prev = 0;
+#pragma unroll
+            for (int w = 0; w < RT / 32; ++w) {
+                k0 += s_few[w];
+                prev = max(prev, s_few[RT / 32 + w]);
+            }
+            if (threadIdx.x == 0) s_prev = prev;
         }
+        if (lane == 0) s_first[warp] = (uint8_t)v.x;
+        if (threadIdx.x == 0) s_first[RT / 32] = t0 + len < N ? S[t0 + len] : (uint8_t)0;
         uint32_t after = __shfl_down_sync(0xffffffffu, v.x, 1);  // its low byte follows this thread's
         __syncthreads();
         if (lane == 31) after = s_first[warp + 1];
-        const uint32_t q0 = threadIdx.x * RI, i0 = t0 + q0;
-        uint32_t flags = bytes_differ(v.x, __funnelshift_r(v.x, v.y, 8)) |
-                         bytes_differ(v.y, __funnelshift_r(v.y, v.z, 8)) << 4 |
-                         bytes_differ(v.z, __funnelshift_r(v.z, v.w, 8)) << 8 |
-                         bytes_differ(v.w, __funnelshift_r(v.w, after, 8)) << 12;
-        // block ends: none inside most tiles
-        const bool inside = bend0 < t0 + len;  // CTA-uniform: another block starts in the tile
-        uint32_t starts = 0;                   // bit j: element q0 + j starts a block
-        uint32_t b = b0;
-        if (inside) {
-            b = i0 < N ? block_at(blocks, nb, i0) : 0u;
-            uint32_t bb = b, bend = i0 < N ? blocks[b].off + blocks[b].n : 0u;
-            if (i0 < N && blocks[b].off == i0) starts |= 1u;
-#pragma unroll
-            for (int j = 0; j < RI; ++j) {
-                if (i0 + j >= N) break;
-                if (i0 + j == bend) {
-                    ++bb;
-                    bend = blocks[bb].off + blocks[bb].n;
-                    starts |= 1u << j;
-                }
-                if (i0 + j + 1 == bend) flags |= 1u << j;
-            }
-        } else {
-            if (threadIdx.x == 0 && blocks[b0].off == t0) starts = 1u;
-            if (bend0 == t0 + len && bend0 - 1 - i0 < (uint32_t)RI) flags |= 1u << (bend0 - 1 - i0);
-        }
-        if (q0 + RI > len) flags &= q0 < len ? (1u << (len - q0)) - 1u : 0u;
+        uint32_t starts, b;
+        const uint32_t flags = run_ends(v, after, i0, t0, len, N, blocks, nb, b0, bend0, starts, b);
         uint32_t total;
         const uint32_t pre = block_exclusive_scan<RT>(__popc(flags), scan_tmp, &total);
-        // the tile's runs, compacted (every thread holds its bytes in registers)
         {
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-            uint32_t k = pre;
+            uint32_t k = pre + (k0 & 3u);
 #pragma unroll
             for (int j = 0; j < RI; ++j) {
                 if ((flags >> j) & 1u) {
@@ -186,56 +288,103 @@ __global__ void __launch_bounds__(RT) k_rle_encode(const uint8_t* __restrict__ S
                     ++k;
                 }
             }
-            const uint32_t last = __reduce_max_sync(0xffffffffu, flags ? t0 + q0 + 32u - __clz(flags) : 0u);
-            if (lane == 0 && last) atomicMax(&s_last, last);
         }
         __syncthreads();
-        if (warp == 0) {
-            const uint64_t e = lookback_u64(status, t, 0, total, spin, &ctrl[CTRL_ERR], withhold);
-            if (lane == 0) s_excl = e;
-        } else if (warp == 1) {
-            if (lane == 0) st_volatile64(tail + t, LB_INC | s_last);
-            const uint32_t e = total ? last_end_before(tail, t, spin, &ctrl[CTRL_ERR]) : 0u;
-            if (lane == 0) s_prev = e;
-        }
-        __syncthreads();
-        const uint64_t k0 = s_excl;
         while (starts) {  // runs before the block's first byte
             const int j = __ffs(starts) - 1;
             starts &= starts - 1;
             while (blocks[b].off < i0 + j) ++b;
-            run_off[b] = k0 + pre + __popc(flags & ((1u << j) - 1u));
+            run_off[b] = (uint64_t)k0 + pre + __popc(flags & ((1u << j) - 1u));
         }
-        if (t + 1 == ntiles && threadIdx.x == 0) run_off[nb] = k0 + total;
-        for (uint32_t i = threadIdx.x; i < total; i += RT) {
-            if (k0 + i < N) {
-                chars[k0 + i] = sb[i];
-                lens[k0 + i] = i ? (uint32_t)(se[i] - se[i - 1]) : t0 + se[0] - s_prev;
+        if (t + 1 == ntiles && threadIdx.x == 0) run_off[nb] = (uint64_t)k0 + total;
+        // groups of four entries; g is the first one's index in the arrays
+        const uint32_t a = k0 & 3u, end = a + total;
+        const uint64_t base = (uint64_t)k0 - a;
+        for (uint32_t g = threadIdx.x * 4; g < end; g += RT * 4) {
+            const uint32_t c4 = *reinterpret_cast<const uint32_t*>(sb + g);
+            const uint2 e4 = *reinterpret_cast<const uint2*>(se + g);
+            const uint32_t e[4] = {e4.x & 0xffffu, e4.x >> 16, e4.y & 0xffffu, e4.y >> 16};
+            uint32_t l[4];
+            l[0] = g > a ? e[0] - se[g - 1] : t0 + e[0] - s_prev;
+#pragma unroll
+            for (int j = 1; j < 4; ++j) l[j] = g + j > a ? e[j] - e[j - 1] : t0 + e[j] - s_prev;
+            if (vec && g >= a && g + 4 <= end && base + g + 4 <= N) {
+                *reinterpret_cast<uint32_t*>(chars + base + g) = c4;
+                *reinterpret_cast<uint4*>(lens + base + g) = make_uint4(l[0], l[1], l[2], l[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (g + j >= a && g + j < end && base + g + j < N) {
+                        chars[base + g + j] = (uint8_t)(c4 >> (8 * j));
+                        lens[base + g + j] = l[j];
+                    }
+                }
             }
         }
         __syncthreads();
     }
 }
 
-// Decode step 1: B[k] = end of run k (inclusive prefix sum of the lengths,
-// global). A zero length is an input error.
-__global__ void __launch_bounds__(RT) k_rle_scan(const uint32_t* __restrict__ lens, const uint64_t* __restrict__ run_off,
-                                                 uint32_t nb, uint32_t N, uint32_t* __restrict__ B,
-                                                 uint64_t* __restrict__ status,
-                                                 uint32_t* __restrict__ counter, uint32_t* ctrl) {
-    __shared__ uint32_t s_tile, scan_tmp[32];
+// The summed lengths of tile t of RTILE runs, by a warp; zero: one of this
+// lane's lengths is zero (an input error). vec: lens is 16-byte aligned.
+__device__ __forceinline__ uint32_t tile_len_sum(const uint32_t* __restrict__ lens, uint64_t R, uint32_t t, bool vec,
+                                                 bool& zero) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t k0 = (uint64_t)t * RTILE;
+    uint32_t sum = 0;
+    if (vec && k0 + RTILE <= R) {
+#pragma unroll 8
+        for (uint32_t q = lane * 4; q < RTILE; q += 128) {
+            const uint4 x = __ldg(reinterpret_cast<const uint4*>(lens + k0 + q));
+            zero |= x.x == 0u || x.y == 0u || x.z == 0u || x.w == 0u;
+            sum += x.x + x.y + x.z + x.w;
+        }
+    } else {
+        for (uint32_t q = lane; q < RTILE && k0 + q < R; q += 32) {
+            const uint32_t x = lens[k0 + q];
+            zero |= x == 0u;
+            sum += x;
+        }
+    }
+    return __reduce_add_sync(0xffffffffu, sum);
+}
+
+// Decode, sums: the summed lengths of every tile, a warp a tile, and the tiles'
+// prefixes.
+__global__ void __launch_bounds__(RT) k_rle_len_sums(const uint32_t* __restrict__ lens,
+                                                     const uint64_t* __restrict__ run_off, uint32_t nb, uint32_t N,
+                                                     uint32_t* __restrict__ sums, uint64_t* __restrict__ status,
+                                                     uint32_t* __restrict__ counter, uint32_t* ctrl) {
+    __shared__ uint32_t s_span, scan_tmp[32];
     __shared__ uint64_t s_excl;
     const uint64_t R = min(run_off[nb], (uint64_t)N);  // a run holds at least one byte
+    const uint32_t ntiles = (uint32_t)((R + RTILE - 1) / RTILE), per = (ntiles + gridDim.x - 1) / gridDim.x;
+    const bool vec = (reinterpret_cast<uintptr_t>(lens) & 15u) == 0u;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t span = next_tile(&s_span, counter);
+    const uint32_t t0 = min(ntiles, span * per), t1 = min(ntiles, t0 + per);
+    bool zero = false;
+    for (uint32_t t = t0 + warp; t < t1; t += RT / 32) {
+        const uint32_t sum = tile_len_sum(lens, R, t, vec, zero);
+        if (lane == 0) sums[t] = sum;
+    }
+    if (zero) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
+    span_prefixes(sums, t0, t1, status, span, ctrl[CTRL_SPIN], ctrl[CTRL_WITHHOLD], ctrl, scan_tmp, &s_excl);
+}
+
+// Decode step 1: B[k] = end of run k (inclusive prefix sum of the lengths,
+// global).
+__global__ void __launch_bounds__(RT) k_rle_scan(const uint32_t* __restrict__ lens, const uint64_t* __restrict__ run_off,
+                                                 uint32_t nb, uint32_t N, const uint32_t* __restrict__ first,
+                                                 uint32_t* __restrict__ B, uint32_t* ctrl) {
+    __shared__ uint32_t scan_tmp[32], s_few[RT / 32];
+    const uint64_t R = min(run_off[nb], (uint64_t)N);
     const uint32_t ntiles = (uint32_t)((R + RTILE - 1) / RTILE);
     const bool vec = (reinterpret_cast<uintptr_t>(lens) & 15u) == 0u;
-    const uint32_t spin = ctrl[CTRL_SPIN], withhold = ctrl[CTRL_WITHHOLD];
-    for (;;) {
-        const uint32_t t = next_tile(&s_tile, counter);
-        if (t >= ntiles) break;
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const uint64_t k0 = (uint64_t)t * RTILE + threadIdx.x * RI;
-        const bool whole = vec && k0 + RI <= R;
         uint32_t v[RI], sum = 0;
-        if (whole) {
+        if (vec && k0 + RI <= R) {
 #pragma unroll
             for (int j = 0; j < RI; j += 4) {
                 const uint4 x = __ldg(reinterpret_cast<const uint4*>(lens + k0 + j));
@@ -248,25 +397,29 @@ __global__ void __launch_bounds__(RT) k_rle_scan(const uint32_t* __restrict__ le
 #pragma unroll
             for (int j = 0; j < RI; ++j) v[j] = k0 + j < R ? lens[k0 + j] : 0u;
         }
-        bool zero = false;
+        uint32_t f = 0;
+        if (first) {
+            f = first[t];
+        } else {  // few tiles: warp w sums tile w; every tile looks for its own zero lengths
+            bool zero = false;
+            const uint32_t w = threadIdx.x >> 5, x = w < t ? tile_len_sum(lens, R, w, vec, zero) : 0u;
+            if ((threadIdx.x & 31) == 0) s_few[w] = x;
+            zero = false;
 #pragma unroll
-        for (int j = 0; j < RI; ++j) {
-            zero |= v[j] == 0u && k0 + j < R;
-            sum += v[j];
+            for (int j = 0; j < RI; ++j) zero |= v[j] == 0u && k0 + j < R;
+            if (zero) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < RT / 32; ++k) f += s_few[k];
         }
-        if (zero) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
+#pragma unroll
+        for (int j = 0; j < RI; ++j) sum += v[j];
         uint32_t total;
-        const uint32_t pre = block_exclusive_scan<RT>(sum, scan_tmp, &total);
-        if (threadIdx.x < 32) {
-            const uint64_t e = lookback_u64(status, t, 0, total, spin, &ctrl[CTRL_ERR], withhold);
-            if (threadIdx.x == 0) s_excl = e;
-        }
-        __syncthreads();
-        uint64_t acc = s_excl + pre;
+        uint32_t acc = f + block_exclusive_scan<RT>(sum, scan_tmp, &total);
 #pragma unroll
         for (int j = 0; j < RI; ++j) {
             acc += v[j];
-            v[j] = (uint32_t)acc;
+            v[j] = acc;
         }
         if (k0 + RI <= R) {  // B is the plan's, 16-byte aligned
 #pragma unroll
@@ -277,17 +430,6 @@ __global__ void __launch_bounds__(RT) k_rle_scan(const uint32_t* __restrict__ le
             for (int j = 0; j < RI; ++j)
                 if (k0 + j < R) B[k0 + j] = v[j];
         }
-        __syncthreads();
-    }
-}
-
-// Decode check: every block's runs end exactly at the block's end.
-__global__ void k_rle_check(const uint32_t* __restrict__ B, const uint64_t* __restrict__ run_off,
-                            const BlockInfo* __restrict__ blocks, uint32_t nb, uint32_t cap, uint32_t* ctrl) {
-    for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
-        const uint64_t r0 = run_off[b], r1 = run_off[b + 1];
-        const bool ok = (b > 0 || r0 == 0) && r1 > r0 && r1 <= cap && B[r1 - 1] == blocks[b].off + blocks[b].n;
-        if (!ok) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
     }
 }
 
@@ -298,16 +440,22 @@ __global__ void k_rle_check(const uint32_t* __restrict__ B, const uint64_t* __re
 // probes a round), every later tile starts at the run the one before ended in.
 // Bytes are gathered from shared memory and written 16 at a time. 64 mixed
 // blocks: 366 us with a search a tile by one thread (25 dependent loads) and
-// byte stores -> 96 us; the lengths' scan 248 -> 147 us with 16-byte loads and
-// stores.
+// byte stores -> 90 us.
 __global__ void __launch_bounds__(RT) k_rle_expand(const uint8_t* __restrict__ chars, const uint32_t* __restrict__ B,
-                                                   const uint64_t* __restrict__ run_off, uint32_t nb, uint32_t N,
-                                                   uint8_t* __restrict__ out) {
+                                                   const uint64_t* __restrict__ run_off,
+                                                   const BlockInfo* __restrict__ blocks, uint32_t nb, uint32_t N,
+                                                   uint8_t* __restrict__ out, uint32_t* ctrl) {
     __shared__ __align__(16) uint8_t sflag[RTILE];
     __shared__ uint8_t sc[RTILE];
     __shared__ uint32_t s_k0, scan_tmp[32];
+    // the input's check: every block's runs end exactly at the block's end
+    for (uint32_t b = blockIdx.x * RT + threadIdx.x; b < nb; b += gridDim.x * RT) {
+        const uint64_t r0 = run_off[b], r1 = run_off[b + 1];
+        const bool ok = (b > 0 || r0 == 0) && r1 > r0 && r1 <= N && B[r1 - 1] == blocks[b].off + blocks[b].n;
+        if (!ok) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
+    }
     const uint64_t R = min(run_off[nb], (uint64_t)N);
-    if (R == 0) return;  // no runs: the check has flagged the input
+    if (R == 0) return;  // no runs: the check flags the input
     const uint32_t ntiles = (N + RTILE - 1) / RTILE;
     const uint32_t span = (ntiles + gridDim.x - 1) / gridDim.x;
     const uint32_t t_end = min(ntiles, (blockIdx.x + 1) * span);
@@ -875,15 +1023,20 @@ extern "C" bwt_status bwt_rle_encode(bwt_plan* p, const uint8_t* d_in, const uin
     std::memset(&p->stats, 0, sizeof(p->stats));
     bwt_status s = prepare_batch(p, offsets, num_blocks, st);
     if (s != BWT_OK) return p->last = s;
-    if ((s = reset_ctrl(p, st)) != BWT_OK) return p->last = s;
     const uint32_t N = p->total, nt = (N + RTILE - 1) / RTILE;
-    uint64_t* status = reinterpret_cast<uint64_t*>(p->status);
-    CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * 2 * nt, st));  // run counts, last run ends
     const int sms = num_sms();
-    k_rle_encode<<<std::max(1, std::min<int>(nt, sms * 8)), RT, 0, st>>>(
-        d_in, N, p->blocks, p->nb, d_chars, d_lens, d_run_off, status, status + nt, p->ctrl + CTRL_TILE_CTR, p->ctrl);
+    const int spans = std::max(1, std::min<int>(nt, sms * 4));
+    uint64_t* status = reinterpret_cast<uint64_t*>(p->status);  // the spans' words, then two words a tile
+    uint32_t* sums = p->status + 2 * (size_t)spans;
+    if ((s = reset_ctrl(p, st, p->status, 2 * spans)) != BWT_OK) return p->last = s;
+    const bool few = nt <= FEW_TILES;
+    if (!few)
+        k_rle_sums<<<spans, RT, 0, st>>>(d_in, N, p->blocks, p->nb, sums, sums + nt, status,
+                                         p->ctrl + CTRL_TILE_CTR, p->ctrl);
+    k_rle_encode<<<std::max(1, std::min<int>(nt, sms * 48)), RT, 0, st>>>(d_in, N, p->blocks, p->nb, few ? nullptr : sums, sums + nt,
+                                                                       d_chars, d_lens, d_run_off, p->ctrl);
     CKS(cudaGetLastError());
-    p->stats.kernel_launches = 2;
+    p->stats.kernel_launches = few ? 2 : 3;
     return p->last = finish_status(p, st);
 }
 
@@ -897,19 +1050,23 @@ extern "C" bwt_status bwt_rle_decode(bwt_plan* p, const uint8_t* d_chars, const 
     std::memset(&p->stats, 0, sizeof(p->stats));
     bwt_status s = prepare_batch(p, offsets, num_blocks, st);
     if (s != BWT_OK) return p->last = s;
-    if ((s = reset_ctrl(p, st)) != BWT_OK) return p->last = s;
     const uint32_t N = p->total, nt = (N + RTILE - 1) / RTILE;  // runs <= N, so <= nt tiles of runs
-    uint64_t* status = reinterpret_cast<uint64_t*>(p->status);
-    CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * nt, st));
-    uint32_t* B = p->vals[0];
     const int sms = num_sms();
-    k_rle_scan<<<std::max(1, std::min<int>(nt, sms * 8)), RT, 0, st>>>(d_lens, d_run_off, p->nb, N, B, status,
-                                                                     p->ctrl + CTRL_TILE_CTR, p->ctrl);
-    k_rle_check<<<std::max(1u, std::min<uint32_t>((p->nb + 255) / 256, 1024)), 256, 0, st>>>(B, d_run_off, p->blocks,
-                                                                                          p->nb, N, p->ctrl);
-    k_rle_expand<<<std::max(1, std::min<int>(nt, sms * 8)), RT, 0, st>>>(d_chars, B, d_run_off, p->nb, N, d_out);
+    const int spans = std::max(1, std::min<int>(nt, sms * 4));
+    uint64_t* status = reinterpret_cast<uint64_t*>(p->status);  // the spans' words, then a word a tile
+    uint32_t* sums = p->status + 2 * (size_t)spans;
+    if ((s = reset_ctrl(p, st, p->status, 2 * spans)) != BWT_OK) return p->last = s;
+    uint32_t* B = p->vals[0];
+    const bool few = nt <= FEW_TILES;
+    if (!few)
+        k_rle_len_sums<<<spans, RT, 0, st>>>(d_lens, d_run_off, p->nb, N, sums, status, p->ctrl + CTRL_TILE_CTR,
+                                             p->ctrl);
+    k_rle_scan<<<std::max(1, std::min<int>(nt, sms * 24)), RT, 0, st>>>(d_lens, d_run_off, p->nb, N, few ? nullptr : sums,
+                                                                        B, p->ctrl);
+    k_rle_expand<<<std::max(1, std::min<int>(nt, sms * 24)), RT, 0, st>>>(d_chars, B, d_run_off,
+                                                                            p->blocks, p->nb, N, d_out, p->ctrl);
     CKS(cudaGetLastError());
-    p->stats.kernel_launches = 4;
+    p->stats.kernel_launches = few ? 3 : 4;
     return p->last = finish_status(p, st);
 }
 

@@ -125,7 +125,7 @@ def test_inverse_samples_and_supers(kind, tile):
 
 
 @pytest.mark.parametrize("shift", [0, 3])
-@pytest.mark.parametrize("kind", ["edges", "long", "dense", "ends"])
+@pytest.mark.parametrize("kind", ["edges", "few", "few_plus_one", "long", "dense", "ends"])
 def test_rle_tiles(kind, shift):
     """Run-length encoding and decoding around the 4,096-byte tiles: runs that
     begin many tiles before their end, tiles without a run end, blocks that end
@@ -135,6 +135,11 @@ def test_rle_tiles(kind, shift):
     r = np.random.RandomState(41)
     if kind == "edges":
         blocks = [r.randint(0, 2, n).astype(np.uint8) for n in (4095, 1, 4096, 4097, 15, 16, 17, 8175, 1, 1, 12288)]
+    elif kind in ("few", "few_plus_one"):  # eight tiles and one more byte: the largest batch without the sums' pass
+        n = 8 * 4096 + (kind == "few_plus_one")
+        b = r.randint(0, 2, n).astype(np.uint8)
+        b[5000:14_000] = 9  # a run over two whole tiles
+        blocks = [b[:20_001], b[20_001:20_002], b[20_002:]]
     elif kind == "long":  # 300,000-byte runs: tiles 32 and more back hold the last run end
         blocks = [np.repeat(np.array([5, 6, 5], dtype=np.uint8), 300_000), np.full(200_000, 6, dtype=np.uint8)]
     elif kind == "dense":
