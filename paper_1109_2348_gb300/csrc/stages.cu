@@ -46,6 +46,7 @@ namespace {
 constexpr int RT = 256;                 // threads per tile
 constexpr int RI = 16;                  // elements per thread
 constexpr uint32_t RTILE = RT * RI;     // 4096
+constexpr uint32_t PART = RTILE / (RT / 32);  // a warp's share of a tile
 
 // Block holding global position i (blocks are contiguous and cover the batch).
 __device__ __forceinline__ uint32_t block_at(const BlockInfo* blocks, uint32_t nb, uint32_t i) {
@@ -156,20 +157,22 @@ __device__ __forceinline__ uint4 load16(const uint8_t* __restrict__ S, uint32_t 
 }
 
 // Tiles of a batch so small that the second pass finds its own prefixes, a warp
-// an earlier tile, and the first is left out: a launch and a look-back less (one
-// 30,000-byte batch: 50.0 -> 39.9 us a call).
+// an earlier tile, and the first is left out: a launch and a look-back less (a
+// 30,000-byte batch: 38.0 -> 35.5 us a call; two tiles a warp, up to 65,000
+// bytes: the same to encode, 40 -> 50 to decode).
 constexpr uint32_t FEW_TILES = RT / 32;
 
-// A tile's number of run ends and its last one (end index, 0: none), by a warp.
+// A tile's number of run ends and its last one (end index, 0: none), or those of
+// its bytes [from, to), by a warp.
 __device__ __forceinline__ void tile_run_ends(const uint8_t* __restrict__ S, uint32_t N,
                                               const BlockInfo* __restrict__ blocks, uint32_t nb, uint32_t t,
-                                              uint32_t& cnt, uint32_t& end) {
+                                              uint32_t& cnt, uint32_t& end, uint32_t from = 0, uint32_t to = RTILE) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t p0 = t * RTILE, len = min(RTILE, N - p0);
     const uint32_t b0 = block_at(blocks, nb, p0), bend0 = blocks[b0].off + blocks[b0].n;
     cnt = end = 0;
 #pragma unroll 4
-    for (uint32_t q = lane * 16; q < RTILE; q += 512) {
+    for (uint32_t q = from + lane * 16; q < to; q += 512) {
         const uint32_t i0 = p0 + q;
         const uint4 v = load16(S, i0, N);
         uint32_t after = __shfl_down_sync(0xffffffffu, v.x, 1);
@@ -183,24 +186,44 @@ __device__ __forceinline__ void tile_run_ends(const uint8_t* __restrict__ S, uin
     end = __reduce_max_sync(0xffffffffu, end);
 }
 
-// Encode, sums: every tile's run ends, a warp a tile; then the tiles' prefixes.
+// Encode, sums: every tile's run ends, a warp a tile (a batch of no more tiles
+// than spans: a CTA a tile, as a lone warp's loads wait for each other: 400,000
+// bytes 48 -> 37 us a call, decoded 53 -> 42); then the tiles' prefixes.
 __global__ void __launch_bounds__(RT) k_rle_sums(const uint8_t* __restrict__ S, uint32_t N,
                                                  const BlockInfo* __restrict__ blocks, uint32_t nb,
                                                  uint32_t* __restrict__ sums, uint32_t* __restrict__ last,
                                                  uint64_t* __restrict__ status, uint32_t* __restrict__ counter,
                                                  uint32_t* ctrl) {
-    __shared__ uint32_t s_span, scan_tmp[32];
+    __shared__ uint32_t s_span, s_part[2], scan_tmp[32];
     __shared__ uint64_t s_excl;
     const uint32_t ntiles = (N + RTILE - 1) / RTILE, per = (ntiles + gridDim.x - 1) / gridDim.x;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t span = next_tile(&s_span, counter);  // in start order, so that earlier spans are in flight
     const uint32_t t0 = min(ntiles, span * per), t1 = min(ntiles, t0 + per);
-    for (uint32_t t = t0 + warp; t < t1; t += RT / 32) {
-        uint32_t cnt, end;
-        tile_run_ends(S, N, blocks, nb, t, cnt, end);
-        if (lane == 0) {
-            sums[t] = cnt;
-            last[t] = end;
+    if (per == 1) {
+        if (threadIdx.x < 2) s_part[threadIdx.x] = 0u;
+        __syncthreads();
+        if (t0 < t1) {
+            uint32_t cnt, end;
+            tile_run_ends(S, N, blocks, nb, t0, cnt, end, warp * PART, warp * PART + PART);
+            if (lane == 0) {
+                atomicAdd(&s_part[0], cnt);
+                atomicMax(&s_part[1], end);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && t0 < t1) {
+            sums[t0] = s_part[0];
+            last[t0] = s_part[1];
+        }
+    } else {
+        for (uint32_t t = t0 + warp; t < t1; t += RT / 32) {
+            uint32_t cnt, end;
+            tile_run_ends(S, N, blocks, nb, t, cnt, end);
+            if (lane == 0) {
+                sums[t] = cnt;
+                last[t] = end;
+            }
         }
     }
     span_prefixes(sums, t0, t1, status, span, ctrl[CTRL_SPIN], ctrl[CTRL_WITHHOLD], ctrl, scan_tmp, &s_excl);
@@ -325,37 +348,41 @@ __global__ void __launch_bounds__(RT) k_rle_encode(const uint8_t* __restrict__ S
     }
 }
 
-// The summed lengths of tile t of RTILE runs, by a warp; zero: one of this
-// lane's lengths is zero (an input error). vec: lens is 16-byte aligned.
-__device__ __forceinline__ uint32_t tile_len_sum(const uint32_t* __restrict__ lens, uint64_t R, uint32_t t, bool vec,
-                                                 bool& zero) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint64_t k0 = (uint64_t)t * RTILE;
-    uint32_t sum = 0;
-    if (vec && k0 + RTILE <= R) {
-#pragma unroll 8
-        for (uint32_t q = lane * 4; q < RTILE; q += 128) {
-            const uint4 x = __ldg(reinterpret_cast<const uint4*>(lens + k0 + q));
-            zero |= x.x == 0u || x.y == 0u || x.z == 0u || x.w == 0u;
-            sum += x.x + x.y + x.z + x.w;
-        }
-    } else {
-        for (uint32_t q = lane; q < RTILE && k0 + q < R; q += 32) {
-            const uint32_t x = lens[k0 + q];
-            zero |= x == 0u;
-            sum += x;
-        }
-    }
-    return __reduce_add_sync(0xffffffffu, sum);
+// Four lengths from k on, those past the last run (R) read as one, which is no
+// input error. vec: lens is 16-byte aligned.
+__device__ __forceinline__ uint4 lens4(const uint32_t* __restrict__ lens, uint64_t R, uint64_t k, bool vec) {
+    if (vec && k + 4 <= R) return __ldg(reinterpret_cast<const uint4*>(lens + k));
+    return make_uint4(k < R ? lens[k] : 1u, k + 1 < R ? lens[k + 1] : 1u, k + 2 < R ? lens[k + 2] : 1u,
+                      k + 3 < R ? lens[k + 3] : 1u);
 }
 
-// Decode, sums: the summed lengths of every tile, a warp a tile, and the tiles'
-// prefixes.
+// The summed lengths of tile t of RTILE runs, or of its runs [from, to), by a
+// warp; zero: one of this lane's lengths is zero (an input error). The last tile's missing entries
+// count one and are subtracted, so that it takes the same eight loads in flight
+// as a full one: 4 blocks of up to 415 KB waited 41 us for its lengths read one
+// after the other.
+__device__ __forceinline__ uint32_t tile_len_sum(const uint32_t* __restrict__ lens, uint64_t R, uint32_t t, bool vec,
+                                                 bool& zero, uint32_t from = 0, uint32_t to = RTILE) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t k0 = (uint64_t)t * RTILE, k1 = k0 + to;
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (uint32_t q = from + lane * 4; q < to; q += 128) {
+        const uint4 x = lens4(lens, R, k0 + q, vec);
+        zero |= x.x == 0u || x.y == 0u || x.z == 0u || x.w == 0u;
+        sum += x.x + x.y + x.z + x.w;
+    }
+    const uint32_t pad = k1 <= R ? 0u : (uint32_t)(k1 - max(R, k0 + from));
+    return __reduce_add_sync(0xffffffffu, sum) - pad;
+}
+
+// Decode, sums: the summed lengths of every tile, a warp a tile (no more tiles
+// than spans: a CTA a tile), and the tiles' prefixes.
 __global__ void __launch_bounds__(RT) k_rle_len_sums(const uint32_t* __restrict__ lens,
                                                      const uint64_t* __restrict__ run_off, uint32_t nb, uint32_t N,
                                                      uint32_t* __restrict__ sums, uint64_t* __restrict__ status,
                                                      uint32_t* __restrict__ counter, uint32_t* ctrl) {
-    __shared__ uint32_t s_span, scan_tmp[32];
+    __shared__ uint32_t s_span, s_part, scan_tmp[32];
     __shared__ uint64_t s_excl;
     const uint64_t R = min(run_off[nb], (uint64_t)N);  // a run holds at least one byte
     const uint32_t ntiles = (uint32_t)((R + RTILE - 1) / RTILE), per = (ntiles + gridDim.x - 1) / gridDim.x;
@@ -364,9 +391,20 @@ __global__ void __launch_bounds__(RT) k_rle_len_sums(const uint32_t* __restrict_
     const uint32_t span = next_tile(&s_span, counter);
     const uint32_t t0 = min(ntiles, span * per), t1 = min(ntiles, t0 + per);
     bool zero = false;
-    for (uint32_t t = t0 + warp; t < t1; t += RT / 32) {
-        const uint32_t sum = tile_len_sum(lens, R, t, vec, zero);
-        if (lane == 0) sums[t] = sum;
+    if (per == 1) {
+        if (threadIdx.x == 0) s_part = 0u;
+        __syncthreads();
+        if (t0 < t1) {
+            const uint32_t sum = tile_len_sum(lens, R, t0, vec, zero, warp * PART, warp * PART + PART);
+            if (lane == 0) atomicAdd(&s_part, sum);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && t0 < t1) sums[t0] = s_part;
+    } else {
+        for (uint32_t t = t0 + warp; t < t1; t += RT / 32) {
+            const uint32_t sum = tile_len_sum(lens, R, t, vec, zero);
+            if (lane == 0) sums[t] = sum;
+        }
     }
     if (zero) atomicOr(&ctrl[CTRL_ERR], ERR_INPUT);
     span_prefixes(sums, t0, t1, status, span, ctrl[CTRL_SPIN], ctrl[CTRL_WITHHOLD], ctrl, scan_tmp, &s_excl);
@@ -626,8 +664,10 @@ __global__ void __launch_bounds__(1024) k_vle_offsets(const unsigned long long* 
 
 // Zeroes the output words [0, ceil(byte_off[nb] / 4)) that lie inside the
 // buffer (partial words at the end are merged by atomic OR, so they need it).
+// Also clears the packing's look-back words.
 __global__ void k_vle_zero(uint32_t* __restrict__ out32, const uint64_t* __restrict__ byte_off, uint32_t nb,
-                           uint64_t cap_words) {
+                           uint64_t cap_words, uint64_t* __restrict__ status, uint32_t ntiles) {
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) status[t] = 0ull;
     const uint64_t words = min((byte_off[nb] + 3) / 4, cap_words);
     for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x)
         out32[w] = 0u;
@@ -1096,9 +1136,8 @@ extern "C" bwt_status bwt_vle_encode(bwt_plan* p, const uint8_t* d_in, const uin
     k_vle_bits<<<std::max(1, std::min<int>(nt, sms * 8)), RT, 0, st>>>(d_in, p->tiles0, nt, d_len, bits, p->ctrl);
     k_vle_offsets<<<1, 1024, 0, st>>>(bits, nb, out_cap, d_byte_off, p->ctrl);
     const uint64_t cap_words = out_cap / 4;  // whole words inside the buffer
-    k_vle_zero<<<sms * 8, 256, 0, st>>>(reinterpret_cast<uint32_t*>(d_out), d_byte_off, nb, cap_words);
     uint64_t* status = reinterpret_cast<uint64_t*>(p->status);
-    CKS(cudaMemsetAsync(status, 0, sizeof(uint64_t) * nt, st));
+    k_vle_zero<<<sms * 8, 256, 0, st>>>(reinterpret_cast<uint32_t*>(d_out), d_byte_off, nb, cap_words, status, nt);
     k_vle_pack<<<std::max(1, std::min<int>(nt, sms * 6)), RT, VLE_SMEM, st>>>(
         d_in, p->blocks, p->rtile == p->tile ? p->tiles_il : p->tiles0, nt, d_code, d_len, d_byte_off, cap_words, reinterpret_cast<uint32_t*>(d_out), status,
         p->ctrl + CTRL_TILE_CTR, p->ctrl);

@@ -125,7 +125,7 @@ def test_inverse_samples_and_supers(kind, tile):
 
 
 @pytest.mark.parametrize("shift", [0, 3])
-@pytest.mark.parametrize("kind", ["edges", "few", "few_plus_one", "long", "dense", "ends"])
+@pytest.mark.parametrize("kind", ["edges", "few", "few_plus_one", "long", "dense", "ends", "spans"])
 def test_rle_tiles(kind, shift):
     """Run-length encoding and decoding around the 4,096-byte tiles: runs that
     begin many tiles before their end, tiles without a run end, blocks that end
@@ -142,6 +142,8 @@ def test_rle_tiles(kind, shift):
         blocks = [b[:20_001], b[20_001:20_002], b[20_002:]]
     elif kind == "long":  # 300,000-byte runs: tiles 32 and more back hold the last run end
         blocks = [np.repeat(np.array([5, 6, 5], dtype=np.uint8), 300_000), np.full(200_000, 6, dtype=np.uint8)]
+    elif kind == "spans":  # more tiles, of bytes and of runs, than spans: a warp sums a tile
+        blocks = [r.randint(0, 256, n).astype(np.uint8) for n in (4_000_001, 999_999)]
     elif kind == "dense":
         blocks = [np.arange(70_001, dtype=np.uint32).astype(np.uint8), r.randint(0, 256, 9).astype(np.uint8)]
     else:  # a run of one byte at every edge, long runs between
