@@ -330,3 +330,19 @@ def test_scatter_units_of_several_tiles(tile):
         L, prim, st = gpu_bwt(buf, off, plan)
     assert st["blocks_routed_plain"] == 0
     assert_matches_oracle(buf, off, L, prim, f"tile {tile}")
+
+
+@pytest.mark.parametrize("more", [-1, 0, 1, 700])
+def test_radix_tiles_around_the_grid(more):
+    """The radix passes claim one tile a CTA where the grid has a CTA for each,
+    and go on claiming beyond: tile counts about the largest grid of 1,024-key
+    tiles (six CTAs an SM), with a partial last tile."""
+    import torch
+    r = np.random.RandomState(53)
+    tiles = 6 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    n = tiles * 1024 - 5
+    buf = r.randint(0, 4, n).astype(np.uint8)
+    off = np.array([0, 300_001, n], dtype=np.uint64)
+    with Plan(max_blocks=2, max_total_bytes=n, max_block_bytes=n - 300_001, tile_keys=1024) as plan:
+        L, prim = plan.forward(torch.from_numpy(buf).cuda(), off)
+    assert_matches_oracle(buf, off, L.cpu().numpy(), prim.cpu().numpy(), more)
