@@ -212,14 +212,44 @@ __global__ void k_build_index(const uint64_t* __restrict__ spl, uint16_t* __rest
     }
 }
 
-// Loads the splitters and their index into shared memory.
+// The splitters and their index in shared memory, whose bank conflicts bound the
+// counting kernel: an index entry holds a cell's first splitter and the number
+// of them (FEW: as many or more, the next cell says where they end), so that a
+// search reads one entry at random instead of two.
+constexpr uint32_t FEW = 15;
+static_assert(NSP <= 4095, "a cell's first splitter takes 12 bits, the count four");
+
 __device__ __forceinline__ void load_splitters(const uint64_t* __restrict__ splitters,
-                                               const uint16_t* __restrict__ index, uint64_t* spl, uint16_t* first) {
+                                               const uint16_t* __restrict__ index, uint64_t* spl, uint16_t* cell) {
     for (int i = threadIdx.x; i < NSP; i += blockDim.x) spl[i] = splitters[i];
-    const uint4* src = reinterpret_cast<const uint4*>(index);
-    uint4* dst = reinterpret_cast<uint4*>(first);
-    for (int i = threadIdx.x; i < IDX_WORDS / 8; i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < IDX_CELLS / 8; i += blockDim.x) {
+        const uint4 v = reinterpret_cast<const uint4*>(index)[i];
+        const uint32_t w[5] = {v.x, v.y, v.z, v.w, index[i * 8 + 8]};
+        uint32_t out[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t a = w[k] & 0xffffu, b = w[k] >> 16, c = w[k + 1] & 0xffffu;
+            out[k] = a | min(b - a, FEW) << 12 | b << 16 | min(c - b, FEW) << 28;
+        }
+        reinterpret_cast<uint4*>(cell)[i] = make_uint4(out[0], out[1], out[2], out[3]);
+    }
+    if (threadIdx.x == 0) cell[IDX_CELLS] = (uint16_t)NSP;
     __syncthreads();
+}
+
+// bucket_of on those tables. Measured and not kept: the splitters' next 32 bits
+// apart from the last 17, so that most steps read 4 bytes (a quarter fewer
+// wavefronts, a fifth more instructions: 4,923 us a call against 4,884), and two
+// or four keys searched at once (4,904, 4,953).
+__device__ __forceinline__ uint32_t bucket_of_shared(const uint64_t* spl, const uint16_t* cell, uint64_t key) {
+    const uint32_t c = (uint32_t)(key >> (64 - IDX_BITS)), e = cell[c];
+    uint32_t lo = e & 0xfffu, hi = lo + (e >> 12);
+    if (hi - lo == FEW) hi = cell[c + 1] & 0xfffu;
+    while (lo < hi) {
+        const uint32_t at = (lo + hi) >> 1;
+        if (spl[at] <= key) lo = at + 1; else hi = at;
+    }
+    return lo;
 }
 
 constexpr size_t SPL_BYTES = 4096 * 8 + IDX_WORDS * 2;  // splitters + prefix index
@@ -266,10 +296,10 @@ __global__ void __launch_bounds__(COUNT_THREADS, 2) k_bucket_count(const uint8_t
                                                                     const uint32_t* __restrict__ need) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t* spl = reinterpret_cast<uint64_t*>(smem);
-    uint16_t* first = reinterpret_cast<uint16_t*>(smem + 4096 * 8);
+    uint16_t* cell = reinterpret_cast<uint16_t*>(smem + 4096 * 8);
     uint32_t* h = reinterpret_cast<uint32_t*>(smem + SPL_BYTES);
     uint8_t* sb = smem + SPL_BYTES + CNT_BYTES;
-    if (!FLAT) load_splitters(splitters, index, spl, first);
+    if (!FLAT) load_splitters(splitters, index, spl, cell);
     for (int i = threadIdx.x; i < NBK / 2; i += blockDim.x) h[i] = 0;
     __syncthreads();
     const uint32_t nspan = (ntiles + span - 1) / span;
@@ -334,7 +364,7 @@ __global__ void __launch_bounds__(COUNT_THREADS, 2) k_bucket_count(const uint8_t
                     const uint32_t b = (uint32_t)(key >> 52);
                     atomicAdd(&h[b & (NBK / 2 - 1)], b < NBK / 2 ? 1u : 1u << 16);
                 } else {
-                    const uint32_t b = bucket_of(spl, first, key);
+                    const uint32_t b = bucket_of_shared(spl, cell, key);
                     fb[td.start + q] = (uint16_t)b;
                     atomicAdd(&h[b & (NBK / 2 - 1)], b < NBK / 2 ? 1u : 1u << 16);
                 }
@@ -585,6 +615,16 @@ __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__
     }
 }
 
+// The key of the 8 bytes from sb[idx + 1] on, and the byte sb[idx] before them:
+// nine bytes lie in three aligned words.
+__device__ __forceinline__ uint64_t pack8_after_smem(const uint8_t* sb, uint32_t idx, uint32_t& before) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(sb) + (idx >> 2);
+    const uint32_t w0 = w[0], w1 = w[1], w2 = w[2], sh = 8u * (idx & 3u);
+    before = w0 >> sh & 0xffu;
+    const uint32_t hi = __funnelshift_rc(w0, w1, sh + 8u), lo = __funnelshift_rc(w1, w2, sh + 8u);
+    return (uint64_t)__byte_perm(hi, 0, 0x0123) << 32 | __byte_perm(lo, 0, 0x0123);
+}
+
 // Scatters the tiles of bucketed blocks to their chunks. A CTA takes runs of
 // consecutive tiles (up to 16, fewer when there are few tiles per CTA) (reloading the block's chunk map and chunk starts into
 // shared memory when the block changes). A rotation's bucket is its stored
@@ -599,10 +639,14 @@ __global__ void __launch_bounds__(256) k_chunk_plan(const uint32_t* __restrict__
 // both and a chunk's runs are twice as long (30 rotations on 900,000-byte
 // blocks). Per 240 blocks the call took 5,118 us with 256 threads and 4,096
 // rotations, 4,990 with this; 512 x 12 rotations a thread 5,174, x 20 5,025, x 24
-// 5,001, three CTAs 5,118 (spills), 1,024 x 8 5,256, 1,024 x 16 5,106.
+// 5,001, three CTAs 5,118 (spills), 1,024 x 8 5,256, 1,024 x 16 5,106. The
+// shared-memory pipe bounds it (80%), so the way out reads, beside the three words
+// of its nine bytes, one packed word and one word a chunk: 37 -> 30 wavefronts a
+// row of 32 rotations, 270 -> 245 us per 48 blocks (before, the bucket's map
+// entry, two words a chunk and the byte before the key apart).
 constexpr int SC_NT = 512, SC_ITEMS = 16, SC_CTAS = 2;
 template <int NT, int ITEMS>
-constexpr size_t CHUNK_SCATTER_SMEM = NBK * 2 + 4 * MAXCH * 4 + (NT * ITEMS + 48) + NT * ITEMS * 4;
+constexpr size_t CHUNK_SCATTER_SMEM = NBK * 2 + 4 * MAXCH * 4 + (NT * ITEMS + 64) + NT * ITEMS * 4;
 
 template <int NT, int ITEMS, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __restrict__ S,
@@ -614,15 +658,15 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __res
                                                        uint64_t* __restrict__ K, uint32_t* __restrict__ I,
                                                        uint32_t* err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    uint8_t* sb = smem;                                                  // [TILE_BYTES], 16-aligned
-    uint16_t* cm = reinterpret_cast<uint16_t*>(smem + NT * ITEMS + 48);  // [NBK] chunk of each bucket
+    uint8_t* sb = smem + 16;                                             // the unit's bytes, and the one before them
+    uint16_t* cm = reinterpret_cast<uint16_t*>(smem + NT * ITEMS + 64);  // [NBK] chunk of each bucket
     uint32_t* cb = reinterpret_cast<uint32_t*>(cm + NBK);                // [MAXCH] chunk starts (block-relative)
     uint32_t* lcount = cb + MAXCH;                                       // [MAXCH] tile's rotations per chunk
     uint32_t* pre = lcount + MAXCH;                                      // [MAXCH] tile-local chunk offsets
-    uint32_t* dbase = pre + MAXCH;                                       // [MAXCH] destination of pre[c]
-    uint32_t* stQC = dbase + MAXCH;  // [NT * ITEMS] by rank: position (low 16 bits) | fine bucket (high 16)
+    uint32_t* dbase = pre + MAXCH;                                       // [MAXCH] chunk's destination less pre[c]
+    uint32_t* stQC = dbase + MAXCH;  // [NT * ITEMS] by rank: position | chunk << 13 | tag << 23 | wide << 31
+    static_assert(NT * ITEMS <= 1 << 13 && MAXCH <= 1 << 10, "the fields above");
     __shared__ uint32_t scan_tmp[32];
-    __shared__ uint8_t s_before;  // the byte before the tile's first rotation
     const uint32_t ntiles = *ntiles_dev;
     const uint32_t span = max(1u, min(16u, ntiles / (gridDim.x * 4u)));
     const uint32_t nspan = (ntiles + span - 1) / span;
@@ -650,6 +694,7 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __res
             const uint32_t i0 = td.start - bi.off;
             for (int i = threadIdx.x; i < (int)MAXCH; i += blockDim.x) lcount[i] = 0;
             uint32_t bk[ITEMS];  // fine bucket of each item
+            uint8_t before = 0;
             if (!flat) {
 #pragma unroll
                 for (int j = 0; j < ITEMS; ++j) {
@@ -658,11 +703,12 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __res
                 }
             }
             const uint32_t shift = stage_tile_bytes(S, bi, i0, td.len, sb, threadIdx.x, NT);
-            if (threadIdx.x == 0) s_before = S[bi.off + (i0 ? i0 : bi.n) - 1];
+            if (threadIdx.x == 0) before = S[bi.off + (i0 ? i0 : bi.n) - 1];
             __syncthreads();
-            // chunk (low 10 bits) | slot within the tile's share of the chunk << 10;
-            // every item's chunk is looked up before the first count, so the
-            // lookups overlap
+            if (threadIdx.x == 0) sb[(int)shift - 1] = before;  // read on the way out
+            // chunk (low 10 bits) | slot within the tile's share of the chunk << 10
+            // | the bucket's tag << 23; every item's chunk is looked up before the
+            // first count, so the lookups overlap
             uint32_t cs[ITEMS];
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j) {
@@ -670,12 +716,13 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __res
                 cs[j] = 0xffffffffu;
                 if (q < td.len) {
                     if (flat) bk[j] = (uint32_t)(pack8_smem(sb, shift + q) >> 52);
-                    cs[j] = cm[bk[j]] & (MAXCH - 1);
+                    const uint32_t e = cm[bk[j]];
+                    cs[j] = (e & (MAXCH - 1)) | ((e & CM_OWN) ? 0u : (bk[j] & 0xffu) << 23);
                 }
             }
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
-                if (cs[j] != 0xffffffffu) cs[j] |= atomicAdd(&lcount[cs[j]], 1u) << 10;
+                if (cs[j] != 0xffffffffu) cs[j] |= atomicAdd(&lcount[cs[j] & (MAXCH - 1)], 1u) << 10;
             __syncthreads();
             // the global reservation (issued first: its round trip overlaps
             // the scan) and the tile-local exclusive prefix over chunks
@@ -694,7 +741,7 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __res
                 for (int i = 0; i < PER; ++i) {
                     const uint32_t c = threadIdx.x * PER + i;
                     pre[c] = ex | (cb[c] & CB_WIDE);
-                    if (v[i]) dbase[c] = bi.off + (cb[c] & ~CB_WIDE) + g[i];
+                    if (v[i]) dbase[c] = bi.off + (cb[c] & ~CB_WIDE) + g[i] - ex;
                     ex += v[i];
                 }
             }
@@ -703,19 +750,19 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_scatter(const uint8_t* __res
             for (int j = 0; j < ITEMS; ++j) {
                 if (cs[j] != 0xffffffffu) {
                     const uint32_t c = cs[j] & (MAXCH - 1);
-                    const uint32_t pos = (pre[c] & ~CB_WIDE) + (cs[j] >> 10);
-                    stQC[pos] = (j * NT + threadIdx.x) | (bk[j] << 16);
+                    const uint32_t pc = pre[c], pos = (pc & ~CB_WIDE) + (cs[j] >> 10 & 0x1fffu);
+                    stQC[pos] = (j * NT + threadIdx.x) | c << 13 | (cs[j] & 0x7f800000u) | (pc & CB_WIDE);
                 }
             }
             __syncthreads();
             for (uint32_t r = threadIdx.x; r < td.len; r += blockDim.x) {
-                const uint32_t qc = stQC[r], q = qc & 0xffffu, b = qc >> 16, e = cm[b], c = e & (MAXCH - 1);
-                const uint32_t pc = pre[c];
-                const uint32_t dst = dbase[c] + (r - (pc & ~CB_WIDE));
+                const uint32_t qc = stQC[r], q = qc & 0x1fffu;
+                const uint32_t dst = dbase[qc >> 13 & (MAXCH - 1)] + r;
                 BWT_DCHECK(dst - bi.off < bi.n, err);  // inside the tile's block
-                const uint64_t key = pack8_smem(sb, shift + q);
-                K[dst] = pc & CB_WIDE ? key : (key << 8) | (q ? sb[shift + q - 1] : s_before);
-                I[dst] = (i0 + q) | ((e & CM_OWN) ? 0u : (b & 0xffu) << TAG_SHIFT);
+                uint32_t l;
+                const uint64_t key = pack8_after_smem(smem, 15 + shift + q, l);
+                K[dst] = (qc & CB_WIDE) ? key : (key << 8) | l;
+                I[dst] = (i0 + q) | (qc >> 23 & 0xffu) << TAG_SHIFT;
             }
             __syncthreads();
         }

@@ -346,3 +346,30 @@ def test_radix_tiles_around_the_grid(more):
     with Plan(max_blocks=2, max_total_bytes=n, max_block_bytes=n - 300_001, tile_keys=1024) as plan:
         L, prim = plan.forward(torch.from_numpy(buf).cuda(), off)
     assert_matches_oracle(buf, off, L.cpu().numpy(), prim.cpu().numpy(), more)
+
+
+@pytest.mark.parametrize("cells", [(14, 15, 16), (15, 1, 0), (3000, 1000)])
+def test_crowded_index_cells(cells):
+    """The counting kernel's index stores up to 14 splitters of a cell (the keys'
+    first 15 bits) and looks at the next cell above that: cells around the limit,
+    first and last cells, keys that equal splitters, and the byte before the
+    first rotation of the block at a staged tile's edge."""
+    import torch
+    r = np.random.RandomState(59)
+    spl = []
+    for i, k in enumerate(cells):  # crowded cells at the key space's start, middle and end
+        base = np.uint64([0, 0x4142 << 48, 0xFFFE << 48][i])
+        spl.append(base + np.arange(k, dtype=np.uint64) * np.uint64((1 << 36) + 12_345))
+    have = np.concatenate(spl)
+    rest = np.linspace(1 << 52, (1 << 64) - (1 << 52), 4095 - have.size).astype(np.uint64)
+    spl = np.sort(np.concatenate([have, rest]))
+    some = spl[r.randint(0, 4095, 400)]
+    text = np.concatenate([np.frombuffer(int(x).to_bytes(8, "big"), dtype=np.uint8) for x in some])
+    blocks = [np.concatenate([text, r.randint(0x41, 0x43, 20_000).astype(np.uint8)]),
+              r.randint(0, 256, 30_011).astype(np.uint8), np.tile(text, 3)[:9_001]]
+    buf, off = batch_from_blocks(blocks)
+    with Plan(max_blocks=3, max_total_bytes=buf.size, max_block_bytes=int(np.diff(off.astype(np.int64)).max()),
+              flags=F_LEARNED) as plan:
+        model.install(plan, spl)
+        L, prim = plan.forward(torch.from_numpy(buf).cuda(), off)
+    assert_matches_oracle(buf, off, L.cpu().numpy(), prim.cpu().numpy(), cells)
