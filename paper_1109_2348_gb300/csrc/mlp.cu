@@ -71,10 +71,20 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ p
 // sample. The gradient's 1,377 sums over the samples then spread over all 256
 // threads. A step is latency (64 CTAs for a batch of 4,096): 98 steps of 4,096
 // samples and the compilation took 5.75 ms with 64 threads a CTA and one thread
-// a sample, 2.13 ms now (13 us a gradient, 7 us a reduction, 0.15 ms the
-// compilation). Sums unrolled by 64 instead of 16: 2.33 ms.
+// a sample, 2.13 ms with four (13 us a gradient, 7 us a reduction, 0.15 ms the
+// compilation), 1.54 ms as dependent launches (step_wait). Sums unrolled by 64
+// instead of 16: 2.33 ms against 2.13.
 constexpr int GT = 4 * GS;   // threads
 constexpr int UQ = H / 4;    // units a thread
+
+// The launches of a training step follow each other as dependent launches: a
+// kernel starts while the one before it ends, reads what that one does not
+// write, and waits for its end and its results here. (Without the attribute at
+// the launch both are empty.) A gradient lets the reduction start only after its
+// own wait, so the weights and moments, which the last reduction wrote, are in
+// place when the next one reads them ahead.
+__device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void step_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ x,
                                                  const float* __restrict__ t, const uint32_t* __restrict__ idx,
@@ -91,6 +101,9 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
     const uint32_t src = valid ? (idx ? idx[first + b] : first + b) : 0u;
     // two of the sample's eight inputs a thread
     for (int i = u0 / 4; i < u0 / 4 + 2; ++i) sx[s][i] = valid ? x[(size_t)src * IN + i] : 0.f;
+    const float want = valid && u0 == 0 ? t[src] : 0.f;
+    step_wait();
+    step_next();
     for (int i = threadIdx.x; i < NP; i += GT) P[i] = params[i];
     __syncthreads();
     if (valid) {
@@ -125,7 +138,7 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
             float y = P[OFF_B3];
 #pragma unroll
             for (int i = 0; i < H; ++i) y = fmaf(P[OFF_W3 + i], sh2[s][i], y);
-            const float e = y - t[src];
+            const float e = y - want;
             serr[s] = e * e;
             sdy[s] = 2.f * e / (float)B;
         } else {
@@ -202,6 +215,17 @@ __global__ void k_mlp_reduce(const float* __restrict__ partial, const float* __r
                              float* __restrict__ params, float* __restrict__ m, float* __restrict__ v, int step,
                              float lr, float beta1, float beta2, float eps) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool adam = params && step > 0 && i < NP;
+    float c1 = 1.f, c2 = 1.f, m0 = 0.f, v0 = 0.f, p0 = 0.f;
+    if (adam) {
+        c1 = 1.f - powf(beta1, (float)step);
+        c2 = 1.f - powf(beta2, (float)step);
+        m0 = m[i];
+        v0 = v[i];
+        p0 = params[i];
+    }
+    step_wait();
+    step_next();
     if (i == (int)(gridDim.x * blockDim.x) - 1 && loss_out) {  // past the parameters
         float l = 0.f;
 #pragma unroll 16
@@ -213,13 +237,13 @@ __global__ void k_mlp_reduce(const float* __restrict__ partial, const float* __r
 #pragma unroll 16
     for (int b = 0; b < nblk; ++b) g += partial[(size_t)b * NP + i];
     if (grad_out) grad_out[i] = g;
-    if (params && step > 0) {
-        const float c1 = 1.f - powf(beta1, (float)step), c2 = 1.f - powf(beta2, (float)step);
-        const float mi = beta1 * m[i] + (1.f - beta1) * g;
-        const float vi = beta2 * v[i] + (1.f - beta2) * g * g;
+    if (adam) {
+        // the roundings spelled out: they do not hang on where the loads stand
+        const float mi = fmaf(1.f - beta1, g, __fmul_rn(beta1, m0));
+        const float vi = fmaf(__fmul_rn(1.f - beta2, g), g, __fmul_rn(beta2, v0));
         m[i] = mi;
         v[i] = vi;
-        params[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        params[i] = p0 - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     }
 }
 
@@ -422,6 +446,25 @@ extern "C" bwt_status bwt_mlp_adam_step(float* d_params, const float* d_grad, fl
     return BWT_OK;
 }
 
+namespace {
+
+// dependent: the kernel before it in the stream is one of a training step (step_wait).
+template <typename... P>
+cudaError_t launch_step(void (*kernel)(P...), unsigned grid, unsigned threads, bool dependent, cudaStream_t st, P... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+}  // namespace
+
 extern "C" bwt_status bwt_model_train(float* d_params, const float* d_x, const float* d_t, uint32_t count,
                                       const uint32_t* d_order, uint32_t epochs, uint32_t batch, float lr,
                                       float* d_epoch_loss, void* stream) {
@@ -452,12 +495,15 @@ extern "C" bwt_status bwt_model_train(float* d_params, const float* d_x, const f
             const uint32_t B = std::min(batch, count - b0);
             const uint32_t nb = (B + GS - 1) / GS;
             ++step;
-            k_mlp_grad<<<nb, GT, 0, st>>>(d_params, d_x, d_t, order, b0, B, s.partial, s.loss_partial);
-            k_mlp_reduce<<<NP / 32 + 1, 32, 0, st>>>(s.partial, s.loss_partial, (int)nb, B, nullptr,
-                                                           batch_loss + b0 / batch, d_params, s.m, s.v, step, lr,
-                                                           0.9f, 0.999f, 1e-8f);
+            // an epoch's first gradient follows work that is not a reduction: an ordinary launch
+            e = launch_step(k_mlp_grad, nb, GT, b0 != 0, st, (const float*)d_params, d_x, d_t, order, b0, B, s.partial,
+                            s.loss_partial);
+            if (e != cudaSuccess) break;
+            e = launch_step(k_mlp_reduce, NP / 32 + 1, 32, true, st, (const float*)s.partial, (const float*)s.loss_partial,
+                            (int)nb, B, (float*)nullptr, batch_loss + b0 / batch, d_params, s.m, s.v, step, lr, 0.9f,
+                            0.999f, 1e-8f);
+            if (e != cudaSuccess) break;
         }
-        e = cudaGetLastError();
         if (d_epoch_loss && e == cudaSuccess) {
             // mean of the epoch's batch losses, computed on the host from a copy
             e = cudaMemcpyAsync(h_loss.data(), batch_loss, sizeof(float) * steps_per_epoch, cudaMemcpyDeviceToHost,
