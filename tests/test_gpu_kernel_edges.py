@@ -373,3 +373,38 @@ def test_crowded_index_cells(cells):
         model.install(plan, spl)
         L, prim = plan.forward(torch.from_numpy(buf).cuda(), off)
     assert_matches_oracle(buf, off, L.cpu().numpy(), prim.cpu().numpy(), cells)
+
+
+@pytest.mark.parametrize("count,batch", [(1000, 256), (64, 64), (130, 1000)])
+def test_training_steps_in_order(count, batch):
+    """Training's dependent launches against the gradient and the Adam step
+    called one after the other, with a partial last batch, one batch an epoch
+    and a batch larger than the samples. Both round differently by some 2^-24 a
+    step; a step that read old weights or sums would be off by the learning rate,
+    1e-3, in most of the parameters."""
+    import ctypes
+
+    import torch
+    from paper_1109_2348_gb300 import _lib
+    lib, r, epochs = _lib.load(), np.random.RandomState(count), 3
+    x, t = r.rand(count, 8).astype(np.float32), r.rand(count).astype(np.float32)
+    order = np.concatenate([r.permutation(count) for _ in range(epochs)]).astype(np.int32)
+    vp = lambda a: ctypes.c_void_p(a.data_ptr())
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        st = ctypes.c_void_p(stream.cuda_stream)
+        d_x, d_t, d_o = (torch.from_numpy(a).cuda() for a in (x, t, order))
+        got = torch.from_numpy(model.init_params(7)).cuda()
+        want = got.clone()
+        _lib.check(lib.bwt_model_train(vp(got), vp(d_x), vp(d_t), count, vp(d_o), epochs, batch,
+                                       ctypes.c_float(1e-3), ctypes.c_void_p(0), st), "train")
+        g, m, v, loss = (torch.zeros(n, device="cuda") for n in (want.numel(),) * 3 + (1,))
+        step = 0
+        for e in range(epochs):
+            for b in range(0, count, batch):
+                i = d_o[e * count + b:e * count + min(b + batch, count)].long()
+                xs, ts, step = d_x[i].contiguous(), d_t[i].contiguous(), step + 1
+                _lib.check(lib.bwt_mlp_loss_grad(vp(want), vp(xs), vp(ts), i.numel(), vp(g), vp(loss), st), "grad")
+                _lib.check(lib.bwt_mlp_adam_step(vp(want), vp(g), vp(m), vp(v), step, ctypes.c_float(1e-3), st), "adam")
+        diff = (got - want).abs().cpu().numpy()
+    assert np.median(diff) <= 1e-6 and diff.max() <= 1e-4, (np.median(diff), diff.max())
