@@ -247,8 +247,9 @@ def timed_cpu_baseline(w, cores: int, target_s: float = 12.0):
 ONESWEEP_DRAM_BYTES_PER_KEY = 23.37
 # DRAM bytes (read + write) per rotation of the learned chunk sort
 # (k_chunk_sort_name<256, 4, 0>) as ncu counted them for the current kernel on
-# 24 blocks of the learned-eval workload; None when the kernel has changed since.
-CHUNK_SORT_DRAM_BYTES_PER_KEY = 15.1
+# 24 blocks of 900,000 bytes (nine text-like to one uniform); None when the
+# kernel has changed since.
+CHUNK_SORT_DRAM_BYTES_PER_KEY = 16.9
 
 
 def reference_arm(args):
@@ -531,7 +532,7 @@ def ours(args):
             return None
         achieved = by / (ms / 1e3) / 1e9
         per_launch_keys = keys / la
-        return {"bound": "hbm", "kernel": "k_chunk_sort_name<256, 4, 0> (learned chunk sort: sort, SA, naming)",
+        return {"bound": "hbm", "kernel": "k_chunk_sort_name<256, 4, 0> (learned chunk sort: sort, SA, L, naming)",
                 "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
                 "peak_source": peak_kind + " hbm_gbs",
                 "traffic": None if CHUNK_SORT_DRAM_BYTES_PER_KEY is None else

@@ -226,9 +226,10 @@ bwt_status bwt_vle_encode(bwt_plan* plan, const uint8_t* d_in, const uint64_t* o
  * the 256 byte values starts in ascending order; every byte is replaced by
  * its position in the list and then moved to the front.
  *   d_in   device, uint8[offsets[num_blocks]]; d_out: the same size (the
- *          positions). Allocates scratch on the first call: 1 KB a chunk, i.e.
- *          2 bytes per byte of max_total_bytes up to 16 MB, then the larger of
- *          16 MB and 0.25 bytes per byte, plus 1 KB a block. */
+ *          positions). Uses the plan's scratch; only a batch of so many short
+ *          blocks that 1 KB a block does not fit it (blocks of under some 150
+ *          bytes) allocates its own, once: up to 2 bytes per byte of
+ *          max_total_bytes and 1 KB a block. */
 bwt_status bwt_mtf_encode(bwt_plan* plan, const uint8_t* d_in, const uint64_t* offsets, uint32_t num_blocks,
                           uint8_t* d_out, void* stream);
 

@@ -182,7 +182,8 @@ extern "C" bwt_status bwt_model_samples(bwt_plan* p, const uint8_t* d_in, const 
 //            rotation index (digits taken from the value), then by K, which
 //            leaves equal prefixes in index order as the doubling rounds
 //            require, and named inside their own bounds.
-// Then prefix doubling and the L gather run as on the plain path.
+// The chunk sorts write their rows' bytes of L; prefix doubling runs as on the
+// plain path, and the L gather fills in the rows marked in lgather.
 
 namespace {
 
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(COUNT_THREADS, 2) k_bucket_count(const uint8_t
     for (int i = threadIdx.x; i < NBK / 2; i += blockDim.x) h[i] = 0;
     __syncthreads();
     const uint32_t nspan = (ntiles + span - 1) / span;
-    // One CTA an SM, so nothing else hides a tile's load: the next tile's
+    // Two CTAs an SM hide little of a tile's load: the next tile's
     // bytes (one 16-byte word a thread, from the aligned addresses covering
     // them) are loaded into registers while the current tile is counted.
     auto fetch = [&](uint32_t t, uint4& w, uint32_t& shift, bool& fast) {
@@ -626,8 +627,8 @@ __device__ __forceinline__ uint64_t pack8_after_smem(const uint8_t* sb, uint32_t
 }
 
 // Scatters the tiles of bucketed blocks to their chunks. A CTA takes runs of
-// consecutive tiles (up to 16, fewer when there are few tiles per CTA) (reloading the block's chunk map and chunk starts into
-// shared memory when the block changes). A rotation's bucket is its stored
+// consecutive tiles (up to 16, fewer when there are few tiles per CTA), reloading
+// the block's chunk map and chunk starts into shared memory when the block changes. A rotation's bucket is its stored
 // learned bucket (fb) or, in blocks routed to equal-width buckets, its top 12
 // key bits. Each tile is ranked by chunk in shared memory (tile-local
 // positions and chunks only, 4 bytes a rotation; keys are re-packed from the
@@ -842,13 +843,16 @@ __device__ __forceinline__ void sort13(uint64_t (&w)[MS_IT]) {
 // Measured per 240 blocks of 900,000 bytes (nine text-like, one uniform):
 // 3,412 us with (key, index) pairs of 12 bytes moved through every round,
 // 2,657 us with words, 2,611 us with one key offset a chunk instead of one a
-// bucket. On 24 blocks (ncu): 11.8 -> 9.0 warp instructions a rotation, 81% of
-// the shared-memory pipe, issue 58%, 15.1 DRAM bytes a rotation. Measured
+// bucket, 2,738 us since it writes L too (the L gather's 600 us are gone). On 24
+// blocks (ncu): 11.8 -> 9.7 warp instructions a rotation, 80% of the
+// shared-memory pipe, issue 60%, 16.9 DRAM bytes a rotation. Measured
 // and not kept: five CTAs an SM at 48 registers (2,734), the second run of a
 // merge stored backwards so that no bounds are tested (2,839), one load a
 // merge step from a selected address (2,691), the first merge round by
 // shuffles between neighbouring threads (2,673: fewer wavefronts, more
-// instructions).
+// instructions), all against 2,611; an end mark behind every run, so that a step
+// tests no bounds and reads one word (2,858 against 2,739: two-way conflicts in
+// the stores and a barrier more).
 //
 // A chunk is a run of whole fine buckets, and a fine bucket is a key range,
 // so the chunk is sorted bucket by bucket: no merge crosses a bucket edge.

@@ -4,8 +4,8 @@
 // Encode: a byte ends a run if the next byte differs or starts another block
 // (runs never cross blocks); an exclusive prefix sum of these flags gives
 // every run its output slot; a run's length is the difference of consecutive
-// end indices (the end before a tile's first run comes from the tiles before). Decode: the inclusive prefix sum of the lengths
-// gives every run's end; flags at the last byte of every run, prefix-summed
+// end indices (the end before a tile's first run comes from the tiles before).
+// Decode: the inclusive prefix sum of the lengths gives every run's end; flags at the last byte of every run, prefix-summed
 // over the output, give every output byte its run; the byte is copied.
 //
 // Variable-length encoding (Section 3.4, Fig. 3; the substitution method of
@@ -807,7 +807,6 @@ constexpr int MTF_WARPS = 8;
 constexpr uint32_t MTF_MIN = 512, MTF_MAX = 4096;  // chunk sizes
 constexpr uint32_t MTF_CHUNKS = 16384;             // chunks shorter than MTF_MAX: at most this many
 
-
 struct MtfChunk {
     uint32_t start, len, rel, n;  // global start, bytes, block-relative start, bytes of the block
 };
@@ -1160,12 +1159,6 @@ extern "C" bwt_status bwt_mtf_encode(bwt_plan* p, const uint8_t* d_in, const uin
     // small batch is latency: more and shorter chunks), 4,096 for large batches
     uint32_t mc = MTF_MIN;
     while (mc < MTF_MAX && N / mc > MTF_CHUNKS) mc <<= 1;
-    // scratch (first use): 256 words a chunk, per block its first chunk
-    const size_t cap_chunks = std::min<size_t>(p->cap_n / MTF_MIN, std::max<size_t>(MTF_CHUNKS, p->cap_n / MTF_MAX)) +
-                              (size_t)p->cap_b + 1;
-    if (!p->mtf_lists) CKS(cudaMalloc(&p->mtf_lists, cap_chunks * 1024 + 4 * ((size_t)p->cap_b + 1)));
-    uint32_t* tab = reinterpret_cast<uint32_t*>(p->mtf_lists);
-    uint32_t* cfirst = tab + cap_chunks * 256;
     uint32_t* h_first = p->h_inv_items;  // pinned staging, free outside the inverse
     uint32_t nc = 0;
     for (uint32_t b = 0; b < nb; ++b) {
@@ -1173,6 +1166,18 @@ extern "C" bwt_status bwt_mtf_encode(bwt_plan* p, const uint8_t* d_in, const uin
         nc += (uint32_t)((p->h_off[b + 1] - p->h_off[b] + mc - 1) / mc);
     }
     h_first[nb] = nc;
+    // scratch: 256 words a chunk, per block its first chunk: in the sort's key
+    // buffers, or, for blocks of a few bytes, on its own from first use on (a
+    // plan's first call on 3 blocks of 233,843 bytes: 214 us with it allocated)
+    uint32_t *tab = reinterpret_cast<uint32_t*>(p->keys[0]), *cfirst = reinterpret_cast<uint32_t*>(p->keys[1]);
+    const size_t room = sizeof(uint64_t) * (size_t)p->cap_n;
+    if ((size_t)nc * 1024 > room || ((size_t)nb + 1) * 4 > room) {
+        const size_t cap_chunks = std::min<size_t>(p->cap_n / MTF_MIN, std::max<size_t>(MTF_CHUNKS, p->cap_n / MTF_MAX)) +
+                                  (size_t)p->cap_b + 1;
+        if (!p->mtf_lists) CKS(cudaMalloc(&p->mtf_lists, cap_chunks * 1024 + 4 * ((size_t)p->cap_b + 1)));
+        tab = reinterpret_cast<uint32_t*>(p->mtf_lists);
+        cfirst = tab + cap_chunks * 256;
+    }
     CKS(cudaMemcpyAsync(cfirst, h_first, sizeof(uint32_t) * (nb + 1), cudaMemcpyHostToDevice, st));
     const int sms = num_sms();
     const size_t smem = (size_t)MTF_WARPS * (mc + 32);

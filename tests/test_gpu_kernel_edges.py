@@ -62,6 +62,8 @@ def _mtf_blocks(kind):
         b[1_000_000:1_200_000] = 7
         b[5_000_000:5_002_560] = np.tile(np.arange(255, -1, -1), 10)
         return [b, b[:70_001]]
+    if kind == "tiny":  # blocks too short for the chunks' lists to fit the key buffers
+        return [r.randint(0, 256, 1 + k % 5).astype(np.uint8) for k in range(300)]
     # over 2^24 bytes: recencies that need more than 24 bits; a byte value last seen at the very start
     b = (datagen.block(datagen.RUNS16, 5, 17_000_000) + 1).astype(np.uint8)
     b[:300] = np.arange(300) % 256
@@ -70,7 +72,7 @@ def _mtf_blocks(kind):
 
 
 @pytest.mark.parametrize("shift_in, shift_out", [(0, 0), (5, 5), (3, 8)])
-@pytest.mark.parametrize("kind", ["edges", "large_chunks", "over_24_bits"])
+@pytest.mark.parametrize("kind", ["edges", "tiny", "large_chunks", "over_24_bits"])
 def test_mtf_steps_and_chunks(kind, shift_in, shift_out):
     """Move-to-front by 32-byte steps: sizes around steps and chunks, every
     chunk size, and buffers of equal and of different alignment."""
