@@ -18,7 +18,7 @@
  * plan owns all scratch; it is sized at plan creation from the descriptor
  * (including the learned bucketing's tables when BWT_F_LEARNED is set), so
  * bwt_forward_batch allocates nothing. bwt_inverse_batch and bwt_mtf_encode
- * allocate their extra scratch once, on their first call on the plan; the
+ * allocate what extra scratch they need once, on their first call on the plan; the
  * MLP training calls allocate temporaries (each says so). All entry points
  * return a bwt_status and never abort the process; kernels never trap.
  * Device-side failures (a bounded wait that ran out, a capacity overflow) are
@@ -166,10 +166,10 @@ bwt_status bwt_inverse_check(const uint8_t* L, uint64_t n, int32_t primary, cons
  *   d_primary   device, int32[num_blocks]: the primary index of every block.
  *   d_out       device, uint8[offsets[num_blocks]]: receives the blocks.
  *   stream      cudaStream_t to run on (NULL = the legacy default stream).
- * Uses the plan's scratch plus about 0.75 bytes per byte of max_total_bytes
- * (and 44 a block; 4 bytes per byte and 64 a block more in a plan whose
- * blocks average under 16 bytes) allocated on the first call. Returns BWT_EINVAL for bad arguments and for a primary
- * outside [0, n) (found on the device; that block's output is undefined).
+ * Uses the plan's scratch plus 8 bytes a block (in a plan whose blocks average
+ * under 20 bytes, up to 5 bytes per byte of max_total_bytes and 110 a block)
+ * allocated on the first call. Returns BWT_EINVAL for bad arguments and for a
+ * primary outside [0, n) (found on the device; that block's output is undefined).
  * The call synchronises `stream` before it returns. d_out must not alias
  * d_L. For any L that is a permutation of some block's bytes the result is
  * the block whose BWT (with this primary) is L. */

@@ -559,12 +559,16 @@ extern "C" bwt_status bwt_inverse_batch(bwt_plan* p, const uint8_t* d_L, const u
     }
     h_qbase[nb] = Q;
     h_sbase[nb] = nodes;
-    // scratch (allocated on first use): a row a sample and 16 bytes a super; the
-    // samples themselves go to keys[0], which the inverse does not use otherwise
-    // (a plan for blocks of a few bytes allocates them too)
+    // scratch: a row a sample and 16 bytes a super in vals[0], the samples in
+    // keys[0], which the inverse does not use otherwise (a plan for blocks of a
+    // few bytes allocates its own on first use)
     const size_t slots = (size_t)(p->cap_n / SMP) + 2 * (size_t)p->cap_b + 1;
     const size_t sups = slots / SUP + 2 * (size_t)p->cap_b + 1;
-    if (!p->inv_slots) CKI(cudaMalloc(&p->inv_slots, 4 * slots + 16 * sups));
+    uint32_t* row = p->vals[0];
+    if (4 * slots + 16 * sups > sizeof(uint32_t) * (size_t)p->cap_n) {
+        if (!p->inv_slots) CKI(cudaMalloc(&p->inv_slots, 4 * slots + 16 * sups));
+        row = p->inv_slots;
+    }
     if (!p->inv_items) CKI(cudaMalloc(&p->inv_items, sizeof(uint32_t) * 2 * ((size_t)p->cap_b + 1)));
     Sample* sample = reinterpret_cast<Sample*>(p->keys[0]);
     if (slots * sizeof(Sample) > sizeof(uint64_t) * p->cap_n) {
@@ -596,7 +600,7 @@ extern "C" bwt_status bwt_inverse_batch(bwt_plan* p, const uint8_t* d_L, const u
     c.sbase = p->inv_items + p->cap_b + 1;
     c.nb = nb;
     c.P = p->keys[1];
-    c.row = p->inv_slots;
+    c.row = row;
     c.sample = sample;
     c.out = d_out;
     c.ctrl = p->ctrl;

@@ -140,7 +140,7 @@ struct bwt_plan {
     uint32_t cap_parts = 0, nparts = 0;
 
     // GPU inverse (allocated on first use)
-    uint32_t* inv_slots = nullptr;     // inverse: the samples' records and the supers' lists
+    uint32_t* inv_slots = nullptr;     // inverse: rows of the samples and the supers' lists, where vals[0] is too small for them
     uint8_t* inv_buf = nullptr;        // inverse: the samples' bytes, where keys[0] is too small for them
     uint32_t* inv_items = nullptr;     // [2][cap_b + 1] prefixes of samples and of supers per block
     uint32_t* h_inv_items = nullptr;   // pinned staging (also the move-to-front chunk table)
