@@ -244,7 +244,7 @@ def timed_cpu_baseline(w, cores: int, target_s: float = 12.0):
 # DRAM bytes (read + write) per key of one u64 onesweep pass as ncu counted
 # them (1-pass metrics) for the current kernel on one full-size pass of the
 # mixed3-64x900000 workload; None when the kernel has changed since.
-ONESWEEP_DRAM_BYTES_PER_KEY = 23.37
+ONESWEEP_DRAM_BYTES_PER_KEY = 23.74
 # DRAM bytes (read + write) per rotation of the learned chunk sort
 # (k_chunk_sort_name<256, 4, 0>) as ncu counted them for the current kernel on
 # 24 blocks of 900,000 bytes (nine text-like to one uniform); None when the
