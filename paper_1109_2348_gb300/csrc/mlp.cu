@@ -72,10 +72,16 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ p
 // threads. A step is latency (64 CTAs for a batch of 4,096): 98 steps of 4,096
 // samples and the compilation took 5.75 ms with 64 threads a CTA and one thread
 // a sample, 2.13 ms with four (13 us a gradient, 7 us a reduction, 0.15 ms the
-// compilation), 1.54 ms as dependent launches (step_wait). Sums unrolled by 64
-// instead of 16: 2.33 ms against 2.13.
-constexpr int GT = 4 * GS;   // threads
-constexpr int UQ = H / 4;    // units a thread
+// compilation), 1.54 ms as dependent launches (step_wait), 1.27-1.32 ms with the
+// values of a unit in a row (four samples' values a 16-byte read) and
+// four sums of W2 a thread sharing its reads: 8 shared-memory wavefronts for 16
+// products instead of 32.
+constexpr int TPS = 4;         // threads a sample
+constexpr int GT = TPS * GS;   // threads
+constexpr int UQ = H / TPS;    // units a thread
+constexpr int GP = GS + 4;     // row length: 16-byte reads of eight lanes' rows fall in different banks
+constexpr int GR = H / (GT / 32);  // rows of W2 a warp sums
+static_assert(GT >= IN * H && IN % TPS == 0 && GR >= 1 && GT >= 128, "the sums' split over the threads");
 
 // The launches of a training step follow each other as dependent launches: a
 // kernel starts while the one before it ends, reads what that one does not
@@ -90,17 +96,16 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
                                                  const float* __restrict__ t, const uint32_t* __restrict__ idx,
                                                  uint32_t first, uint32_t B, float* __restrict__ partial,
                                                  float* __restrict__ loss_partial) {
-    __shared__ float P[NP];
-    __shared__ float sx[GS][IN + 1];
-    __shared__ float sh1[GS][H + 1], sh2[GS][H + 1], sd1[GS][H + 1], sd2[GS][H + 1];
+    __shared__ __align__(16) float P[NP];
+    // a row a unit (or input), a column a sample
+    __shared__ __align__(16) float sx[IN][GP], sh1[H][GP], sh2[H][GP], sd1[H][GP], sd2[H][GP];
     __shared__ float sdy[GS], serr[GS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = (warp & 1) * 32 + lane, u0 = (warp >> 1) * UQ;  // the thread's sample and first unit
     const uint32_t b = blockIdx.x * GS + s;
     const bool valid = b < B;
     const uint32_t src = valid ? (idx ? idx[first + b] : first + b) : 0u;
-    // two of the sample's eight inputs a thread
-    for (int i = u0 / 4; i < u0 / 4 + 2; ++i) sx[s][i] = valid ? x[(size_t)src * IN + i] : 0.f;
+    for (int i = u0 / UQ * (IN / TPS), n = 0; n < IN / TPS; ++i, ++n) sx[i][s] = valid ? x[(size_t)src * IN + i] : 0.f;
     const float want = valid && u0 == 0 ? t[src] : 0.f;
     step_wait();
     step_next();
@@ -112,8 +117,8 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
             const int j = u0 + k;
             float a = P[OFF_B1 + j];
 #pragma unroll
-            for (int i = 0; i < IN; ++i) a = fmaf(P[OFF_W1 + j * IN + i], sx[s][i], a);
-            sh1[s][j] = a > 0.f ? a : 0.f;
+            for (int i = 0; i < IN; ++i) a = fmaf(P[OFF_W1 + j * IN + i], sx[i][s], a);
+            sh1[j][s] = a > 0.f ? a : 0.f;
         }
     }
     __syncthreads();
@@ -121,7 +126,7 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
     if (valid) {
         float h1[H];
 #pragma unroll
-        for (int i = 0; i < H; ++i) h1[i] = sh1[s][i];
+        for (int i = 0; i < H; ++i) h1[i] = sh1[i][s];
 #pragma unroll
         for (int k = 0; k < UQ; ++k) {
             const int j = u0 + k;
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
 #pragma unroll
             for (int i = 0; i < H; ++i) a = fmaf(P[OFF_W2 + j * H + i], h1[i], a);
             h2[k] = a > 0.f ? a : 0.f;
-            sh2[s][j] = h2[k];
+            sh2[j][s] = h2[k];
         }
     }
     __syncthreads();
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
         if (valid) {
             float y = P[OFF_B3];
 #pragma unroll
-            for (int i = 0; i < H; ++i) y = fmaf(P[OFF_W3 + i], sh2[s][i], y);
+            for (int i = 0; i < H; ++i) y = fmaf(P[OFF_W3 + i], sh2[i][s], y);
             const float e = y - want;
             serr[s] = e * e;
             sdy[s] = 2.f * e / (float)B;
@@ -150,59 +155,82 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
     if (valid) {
         const float dy = sdy[s];
 #pragma unroll
-        for (int k = 0; k < UQ; ++k) sd2[s][u0 + k] = h2[k] > 0.f ? dy * P[OFF_W3 + u0 + k] : 0.f;
+        for (int k = 0; k < UQ; ++k) sd2[u0 + k][s] = h2[k] > 0.f ? dy * P[OFF_W3 + u0 + k] : 0.f;
     }
     __syncthreads();
     if (valid) {
         float d2[H];
 #pragma unroll
-        for (int j = 0; j < H; ++j) d2[j] = sd2[s][j];
+        for (int j = 0; j < H; ++j) d2[j] = sd2[j][s];
 #pragma unroll
         for (int k = 0; k < UQ; ++k) {
             const int i = u0 + k;
             float a = 0.f;
 #pragma unroll
             for (int j = 0; j < H; ++j) a = fmaf(P[OFF_W2 + j * H + i], d2[j], a);
-            sd1[s][i] = sh1[s][i] > 0.f ? a : 0.f;
+            sd1[i][s] = sh1[i][s] > 0.f ? a : 0.f;
         }
     } else {
-        for (int k = 0; k < UQ; ++k) sd1[s][u0 + k] = sd2[s][u0 + k] = sh1[s][u0 + k] = sh2[s][u0 + k] = 0.f;
+        for (int k = 0; k < UQ; ++k) sd1[u0 + k][s] = sd2[u0 + k][s] = sh1[u0 + k][s] = sh2[u0 + k][s] = 0.f;
     }
     __syncthreads();
     float* out = partial + (size_t)blockIdx.x * NP;
-    for (int e = threadIdx.x; e < NP; e += GT) {
-        float g = 0.f;
-        if (e < OFF_B1) {
-            const int j = e / IN, i = e % IN;
-#pragma unroll 16
-            for (int q = 0; q < GS; ++q) g = fmaf(sd1[q][j], sx[q][i], g);
-        } else if (e < OFF_W2) {
-            const int j = e - OFF_B1;
-#pragma unroll 16
-            for (int q = 0; q < GS; ++q) g += sd1[q][j];
-        } else if (e < OFF_B2) {
-            const int j = (e - OFF_W2) / H, i = (e - OFF_W2) % H;
-#pragma unroll 16
-            for (int q = 0; q < GS; ++q) g = fmaf(sd2[q][j], sh1[q][i], g);
-        } else if (e < OFF_W3) {
-            const int j = e - OFF_B2;
-#pragma unroll 16
-            for (int q = 0; q < GS; ++q) g += sd2[q][j];
-        } else if (e < OFF_B3) {
-            const int i = e - OFF_W3;
-#pragma unroll 16
-            for (int q = 0; q < GS; ++q) g = fmaf(sdy[q], sh2[q][i], g);
-        } else {
-#pragma unroll 16
-            for (int q = 0; q < GS; ++q) g += sdy[q];
+    {  // W2: GR rows a warp, a column a lane
+        float g[GR] = {};
+#pragma unroll 4
+        for (int q = 0; q < GS; q += 4) {
+            const float4 h = *reinterpret_cast<const float4*>(&sh1[lane][q]);
+#pragma unroll
+            for (int k = 0; k < GR; ++k) {
+                const float4 d = *reinterpret_cast<const float4*>(&sd2[warp * GR + k][q]);
+                g[k] = fmaf(d.x, h.x, g[k]);
+                g[k] = fmaf(d.y, h.y, g[k]);
+                g[k] = fmaf(d.z, h.z, g[k]);
+                g[k] = fmaf(d.w, h.w, g[k]);
+            }
         }
-        out[e] = g;
+#pragma unroll
+        for (int k = 0; k < GR; ++k) out[OFF_W2 + (warp * GR + k) * H + lane] = g[k];
     }
-    if (threadIdx.x == GT - 1) {  // a thread with fewer sums than the first ones
-        float l = 0.f;
+    if (threadIdx.x < IN * H) {  // W1: an entry a thread
+        const int j = threadIdx.x / IN, i = threadIdx.x % IN;
+        float g = 0.f;
+#pragma unroll 4
+        for (int q = 0; q < GS; q += 4) {
+            const float4 d = *reinterpret_cast<const float4*>(&sd1[j][q]);
+            const float4 v = *reinterpret_cast<const float4*>(&sx[i][q]);
+            g = fmaf(d.x, v.x, g);
+            g = fmaf(d.y, v.y, g);
+            g = fmaf(d.z, v.z, g);
+            g = fmaf(d.w, v.w, g);
+        }
+        out[OFF_W1 + threadIdx.x] = g;
+    }
+    // the biases, W3 and the loss: a warp each
+    if (warp < 2) {
+        const float* d = warp == 0 ? sd1[lane] : sd2[lane];
+        float g = 0.f;
+#pragma unroll 4
+        for (int q = 0; q < GS; q += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(&d[q]);
+            g += v.x;
+            g += v.y;
+            g += v.z;
+            g += v.w;
+        }
+        out[(warp == 0 ? OFF_B1 : OFF_B2) + lane] = g;
+    } else if (warp == 2) {
+        float g = 0.f;
 #pragma unroll 16
-        for (int q = 0; q < GS; ++q) l += serr[q];
-        loss_partial[blockIdx.x] = l;
+        for (int q = 0; q < GS; ++q) g = fmaf(sdy[q], sh2[lane][q], g);
+        out[OFF_W3 + lane] = g;
+    } else if (warp == 3 && lane < 2) {
+        const float* d = lane == 0 ? sdy : serr;
+        float g = 0.f;
+#pragma unroll 16
+        for (int q = 0; q < GS; ++q) g += d[q];
+        if (lane == 0) out[OFF_B3] = g;
+        else loss_partial[blockIdx.x] = g;
     }
 }
 
