@@ -101,7 +101,12 @@ __global__ void __launch_bounds__(OsThreads<TILE>::value, OsMinBlocks<TILE>::val
     // 900,000 keys 6,428 -> 6,709 us a call.
     const bool claimer = tid == OS_THREADS - 1;
     if (claimer) {
-        const uint32_t at = atomicAdd(p.tile_counter, 1u);
+        // After a failure no tile is taken: the rows that a pass with a wait run
+        // out has left are not a permutation and no longer match the histograms,
+        // so that a destination could lie outside its segment. (A claim is given
+        // up for it rather than made later: the two reads overlap.)
+        uint32_t at = atomicAdd(p.tile_counter, 1u);
+        if (ld_volatile(&p.ctrl[CTRL_ERR]) != 0u) at = 0xffffffffu;
         *s_tile = at;
         if (at < num_tiles) *s_td = p.tiles[at];
     }
