@@ -213,6 +213,15 @@ __device__ __forceinline__ void st_volatile(uint32_t* p, uint32_t v) {
     *reinterpret_cast<volatile uint32_t*>(p) = v;
 }
 
+// Whether an earlier stage has failed (its output is then not to be used): one
+// answer for the CTA, all of whose threads call. Kernels on other branches of a
+// graph may set the error word while this CTA starts, so threads that each left
+// on their own reading would leave the others without their share of the CTA's
+// work, or, if the one that hands out its tiles had left, without an end.
+__device__ __forceinline__ bool failed_before(const uint32_t* ctrl) {
+    return __syncthreads_or(ld_volatile(&ctrl[CTRL_ERR]) != 0u) != 0;
+}
+
 // The 8 bytes sb[idx .. idx + 7] as a big-endian u64 (the rotation's sort
 // key). sb must be 4-byte aligned and readable up to idx + 11: three aligned
 // 32-bit words are funnel-shifted to the byte offset and byte-swapped.

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256) k_name_initial(const uint64_t* __restrict
     __shared__ uint32_t s_carry[2];
     __shared__ uint32_t s_t;
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;  // an earlier stage failed: SA is not a permutation
+    if (failed_before(ctrl)) return;  // an earlier stage failed: SA is not a permutation
     WarpEmitter em;
     em.init(ebuf[threadIdx.x >> 5]);
     if (num_tiles_dev) num_tiles = *num_tiles_dev;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(256) k_sort_micro(uint32_t* __restrict__ SA, c
                                                     Bins cur, Bins next, const uint32_t* __restrict__ depth,
                                                     uint32_t* ctrl) {
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;
+    if (failed_before(ctrl)) return;
     const uint32_t new_depth = 2u * *depth;
     const uint32_t count = bin_count(cur, 0);
     const uint32_t lane = threadIdx.x & 31;
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(256) k_sort_tiny(uint32_t* __restrict__ SA, co
                                                    Bins cur, Bins next, const uint32_t* __restrict__ depth,
                                                    uint32_t* ctrl) {
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;
+    if (failed_before(ctrl)) return;
     const uint32_t new_depth = 2u * *depth;
     const uint32_t count = bin_count(cur, 1);
     const uint32_t lane = threadIdx.x & 31;
@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(256) k_sort_small(uint32_t* __restrict__ SA, c
                                                     uint32_t* ctrl) {
     __shared__ uint64_t comp[8][CS_IT * 32 + 1];
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;
+    if (failed_before(ctrl)) return;
     const uint32_t new_depth = 2u * *depth;
     const uint32_t count = bin_count(cur, 2);
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(256) k_sort_med(uint32_t* __restrict__ SA, con
                                                   uint32_t* ctrl) {
     __shared__ uint64_t comp[CS_IT * 256 + 1];
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;
+    if (failed_before(ctrl)) return;
     const uint32_t new_depth = 2u * *depth;
     const uint32_t count = bin_count(cur, 3);
     WarpEmitter em;
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(256) k_rename_large(const uint32_t* __restrict
     __shared__ uint32_t ssa[4096];
     __shared__ uint32_t s_carry[2];
     __shared__ GroupDesc ebuf[8][NCLS * EMIT_BUF];
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;
+    if (failed_before(ctrl)) return;
     const uint32_t new_depth = 2u * *depth;
     const uint32_t nt = *num_tiles;
     WarpEmitter em;

@@ -972,7 +972,7 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
     __shared__ uint64_t s_wfirst[NT / 32];
     __shared__ uint32_t s_c, s_rounds;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (ld_volatile(&ctrl[CTRL_ERR])) return;  // an earlier stage failed: the chunks are not permutations
+    if (failed_before(ctrl)) return;  // an earlier stage failed: the chunks are not permutations
     const uint32_t count = bin_count(chunks, LIST);
     // chunks in list order from an atomic counter (zeroed before the launch):
     // the chunks in flight stay within a few blocks, whose rank ranges stay
@@ -1108,7 +1108,7 @@ __global__ void __launch_bounds__(NT, MINB) k_chunk_sort_name(const uint64_t* __
                 if ((uint32_t)j < nreal) sO[first + j] = sI[(uint32_t)w[j] & SLOT_MASK];
             __syncthreads();
             for (uint32_t i = tid; i < len; i += NT) {
-                const uint32_t x = sO[i], sa = x & IDX_MASK;
+                const uint32_t x = sO[i], sa = min(x & IDX_MASK, bi.n - 1u);
                 SA[gd.start + i] = sa | SA_FINAL;
                 L[gd.start + i] = wide ? S[bi.off + (sa ? sa : bi.n) - 1u] : (uint8_t)(x >> TAG_SHIFT);
                 if (sa == 0u) primary[gd.blk] = (int32_t)(cstart + i);

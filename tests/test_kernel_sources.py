@@ -49,3 +49,19 @@ def test_radix_pass_takes_no_tile_after_a_failure():
     _, body = _kernel("k_onesweep", "radix.cu")
     claim = body[body.index("atomicAdd(p.tile_counter"):body.index("for (;;)")]
     assert "ld_volatile(&p.ctrl[CTRL_ERR])" in claim and "at = 0xffffffffu" in claim
+
+
+def test_cta_leaves_as_one():
+    """The branches of a captured graph run side by side, so one branch's kernel
+    may set the error word while a CTA of another's starts: a kernel that a
+    branch launches asks for it once for the whole CTA, before any other use of
+    its barriers, and no thread leaves on a reading of its own."""
+    kernels = [("k_name_initial", "doubling.cu"), ("k_sort_micro", "doubling.cu"), ("k_sort_tiny", "doubling.cu"),
+               ("k_sort_small", "doubling.cu"), ("k_sort_med", "doubling.cu"), ("k_rename_large", "doubling.cu"),
+               ("k_chunk_sort_name", "learned.cu")]
+    for name, file in kernels:
+        _, body = _kernel(name, file)
+        assert "ld_volatile(&ctrl[CTRL_ERR])" not in body, f"{name}: a thread's own reading of the error word"
+        at = body.find("if (failed_before(ctrl)) return;")
+        assert at >= 0, f"{name} does not ask for the error word"
+        assert not re.search(r"__sync|coop_sync|\breturn\b|for \(", body[:at]), f"{name}: asked too late"
