@@ -84,18 +84,18 @@ constexpr int GR = H / (GT / 32);  // rows of W2 a warp sums
 static_assert(GT >= IN * H && IN % TPS == 0 && GR >= 1 && GT >= 128, "the sums' split over the threads");
 
 // The launches of a training step follow each other as dependent launches: a
-// kernel starts while the one before it ends, reads what that one does not
-// write, and waits for its end and its results here. (Without the attribute at
-// the launch both are empty.) A gradient lets the reduction start only after its
-// own wait, so the weights and moments, which the last reduction wrote, are in
-// place when the next one reads them ahead.
+// kernel starts while the one before it ends, reads what no kernel of the
+// training writes (samples, targets, order), and waits for its end and its
+// results here. (Without the attribute at the launch both are empty.) What the
+// kernels before it write is read after the wait and through plain pointers:
+// const and __restrict__ together say that a value stands for the whole kernel,
+// and the loads might then be moved ahead of the wait.
 __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void step_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-__global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ x,
+__global__ void __launch_bounds__(GT) k_mlp_grad(const float* params, const float* __restrict__ x,
                                                  const float* __restrict__ t, const uint32_t* __restrict__ idx,
-                                                 uint32_t first, uint32_t B, float* __restrict__ partial,
-                                                 float* __restrict__ loss_partial) {
+                                                 uint32_t first, uint32_t B, float* partial, float* loss_partial) {
     __shared__ __align__(16) float P[NP];
     // a row a unit (or input), a column a sample
     __shared__ __align__(16) float sx[IN][GP], sh1[H][GP], sh2[H][GP], sd1[H][GP], sd2[H][GP];
@@ -238,22 +238,23 @@ __global__ void __launch_bounds__(GT) k_mlp_grad(const float* __restrict__ param
 // the mean loss, and optionally applies one Adam step (Kingma and Ba 2015). A
 // thread a parameter, 32 to a CTA so that the sums spread over the SMs, and 16
 // partials loaded at a time: a sum is a chain of additions, not of loads.
-__global__ void k_mlp_reduce(const float* __restrict__ partial, const float* __restrict__ loss_partial, int nblk,
-                             uint32_t B, float* __restrict__ grad_out, float* __restrict__ loss_out,
-                             float* __restrict__ params, float* __restrict__ m, float* __restrict__ v, int step,
-                             float lr, float beta1, float beta2, float eps) {
+__global__ void k_mlp_reduce(const float* partial, const float* loss_partial, int nblk, uint32_t B, float* grad_out,
+                             float* loss_out, float* params, float* m, float* v, int step, float lr, float beta1,
+                             float beta2, float eps) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool adam = params && step > 0 && i < NP;
     float c1 = 1.f, c2 = 1.f, m0 = 0.f, v0 = 0.f, p0 = 0.f;
     if (adam) {
         c1 = 1.f - powf(beta1, (float)step);
         c2 = 1.f - powf(beta2, (float)step);
+    }
+    step_wait();
+    step_next();
+    if (adam) {
         m0 = m[i];
         v0 = v[i];
         p0 = params[i];
     }
-    step_wait();
-    step_next();
     if (i == (int)(gridDim.x * blockDim.x) - 1 && loss_out) {  // past the parameters
         float l = 0.f;
 #pragma unroll 16

@@ -65,3 +65,18 @@ def test_cta_leaves_as_one():
         at = body.find("if (failed_before(ctrl)) return;")
         assert at >= 0, f"{name} does not ask for the error word"
         assert not re.search(r"__sync|coop_sync|\breturn\b|for \(", body[:at]), f"{name}: asked too late"
+
+
+def test_training_reads_results_after_the_wait():
+    """Training's kernels start while the one before them runs. What that one
+    writes (weights, moments, partial sums) is read after the wait and through
+    pointers that promise nothing about the values' standing still: such a
+    promise lets a compiler move the loads ahead of the wait."""
+    for name, shared in (("k_mlp_grad", ("params",)),
+                         ("k_mlp_reduce", ("partial", "loss_partial", "params", "m", "v"))):
+        params, body = _kernel(name, "mlp.cu")
+        before = body[:body.index("step_wait();")]
+        for p in shared:
+            decl = re.search(r"[^,]*\b" + p + r"\s*(?:,|$)", params.strip()).group(0)
+            assert "__restrict__" not in decl, f"{name}: {decl}"
+            assert not re.search(r"\b" + p + r"\s*\[", before), f"{name} reads {p} before its wait"
