@@ -79,6 +79,36 @@ __device__ __forceinline__ uint32_t next_tile(uint32_t* s_tile, uint32_t* counte
 // where four took 179.) The second passes launch several tiles' worth of CTAs
 // an SM: their tiles differ in work (encoding 161 us a call with 8, 152 with 48).
 
+// Turns last[t] of the span's tiles [t0, t1) -- a tile's last run end, 0: none --
+// into the last one before t in the span, and returns the span's last one. Ends
+// increase with the tile, so both are maxima. All RT threads call.
+__device__ __forceinline__ uint32_t span_last_ends(uint32_t* last, uint32_t t0, uint32_t t1, uint32_t* warp_max) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t run = 0;
+    for (uint32_t base = t0; base < t1; base += RT) {
+        const uint32_t t = base + threadIdx.x;
+        uint32_t x = t < t1 ? last[t] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x = max(x, y);
+        }
+        if (lane == 31) warp_max[warp] = x;
+        __syncthreads();
+        uint32_t ex = __shfl_up_sync(0xffffffffu, x, 1);
+        ex = max(run, lane ? ex : 0u);
+#pragma unroll
+        for (uint32_t w = 0; w < RT / 32; ++w) {
+            const uint32_t y = warp_max[w];
+            if (w < warp) ex = max(ex, y);
+            run = max(run, y);
+        }
+        if (t < t1) last[t] = ex;
+        __syncthreads();
+    }
+    return run;
+}
+
 // Turns sums[t] of the span's tiles [t0, t1) into their exclusive prefixes over
 // all tiles (mod 2^32). All RT threads call.
 __device__ __forceinline__ void span_prefixes(uint32_t* sums, uint32_t t0, uint32_t t1, uint64_t* status, uint32_t span,
@@ -188,12 +218,13 @@ __device__ __forceinline__ void tile_run_ends(const uint8_t* __restrict__ S, uin
 
 // Encode, sums: every tile's run ends, a warp a tile (a batch of no more tiles
 // than spans: a CTA a tile, as a lone warp's loads wait for each other: 400,000
-// bytes 48 -> 37 us a call, decoded 53 -> 42); then the tiles' prefixes.
+// bytes 48 -> 37 us a call, decoded 53 -> 42); then the tiles' prefixes, and the
+// last run ends before the tiles in their span.
 __global__ void __launch_bounds__(RT) k_rle_sums(const uint8_t* __restrict__ S, uint32_t N,
                                                  const BlockInfo* __restrict__ blocks, uint32_t nb,
                                                  uint32_t* __restrict__ sums, uint32_t* __restrict__ last,
-                                                 uint64_t* __restrict__ status, uint32_t* __restrict__ counter,
-                                                 uint32_t* ctrl) {
+                                                 uint32_t* __restrict__ span_last, uint64_t* __restrict__ status,
+                                                 uint32_t* __restrict__ counter, uint32_t* ctrl) {
     __shared__ uint32_t s_span, s_part[2], scan_tmp[32];
     __shared__ uint64_t s_excl;
     const uint32_t ntiles = (N + RTILE - 1) / RTILE, per = (ntiles + gridDim.x - 1) / gridDim.x;
@@ -227,16 +258,25 @@ __global__ void __launch_bounds__(RT) k_rle_sums(const uint8_t* __restrict__ S, 
         }
     }
     span_prefixes(sums, t0, t1, status, span, ctrl[CTRL_SPIN], ctrl[CTRL_WITHHOLD], ctrl, scan_tmp, &s_excl);
+    const uint32_t end = span_last_ends(last, t0, t1, scan_tmp);  // after it: later spans wait for the prefixes
+    if (threadIdx.x == 0) span_last[span] = end;
 }
 
-// The last run end before tile t: the nearest earlier tile with one, 32 tiles a
-// step (a warp calls); 0 before the first.
-__device__ __forceinline__ uint32_t last_end_before(const uint32_t* __restrict__ last, uint32_t t) {
-    const uint32_t lane = threadIdx.x & 31;
-    for (uint32_t end = t; end > 0; end = end > 32 ? end - 32 : 0) {
-        const uint32_t v = lane < end ? last[end - 1 - lane] : 0u;
-        const uint32_t m = __ballot_sync(0xffffffffu, v != 0u);
-        if (m) return __shfl_sync(0xffffffffu, v, __ffs(m) - 1);
+// The last run end before tile t (a warp calls; 0 before the first): the one in
+// its span, else the nearest earlier span's, 128 spans a step. There are at most
+// four spans an SM, so a run over any number of tiles is a few steps: one run of
+// 2^26 bytes 122 us a call, of 2^28 340. (Walking back over the tiles themselves,
+// 32 a step: 615 us and 11.1 ms.)
+__device__ __forceinline__ uint32_t last_end_before(const uint32_t* __restrict__ last,
+                                                    const uint32_t* __restrict__ span_last, uint32_t t, uint32_t per) {
+    const uint32_t lane = threadIdx.x & 31, v = last[t];
+    if (v) return v;
+    for (uint32_t end = t / per; end > 0; end = end > 128 ? end - 128 : 0) {
+        uint32_t m = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) m = max(m, k * 32 + lane < end ? span_last[end - 1 - k * 32 - lane] : 0u);
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (m) return m;
     }
     return 0u;
 }
@@ -251,6 +291,7 @@ __device__ __forceinline__ uint32_t last_end_before(const uint32_t* __restrict__
 __global__ void __launch_bounds__(RT) k_rle_encode(const uint8_t* __restrict__ S, uint32_t N,
                                                    const BlockInfo* __restrict__ blocks, uint32_t nb,
                                                    const uint32_t* __restrict__ first, const uint32_t* __restrict__ last,
+                                                   const uint32_t* __restrict__ span_last, uint32_t per,
                                                    uint8_t* __restrict__ chars, uint32_t* __restrict__ lens,
                                                    uint64_t* __restrict__ run_off, uint32_t* ctrl) {
     // the tile's run bytes and end positions, from index k0 mod 4 on: a group
@@ -272,7 +313,7 @@ __global__ void __launch_bounds__(RT) k_rle_encode(const uint8_t* __restrict__ S
         if (first) {
             k0 = first[t];
             if (warp == 1) {
-                const uint32_t e = last_end_before(last, t);
+                const uint32_t e = last_end_before(last, span_last, t, per);
                 if (lane == 0) s_prev = e;
             }
         } else {  // few tiles: warp w counts tile w
@@ -1065,15 +1106,17 @@ extern "C" bwt_status bwt_rle_encode(bwt_plan* p, const uint8_t* d_in, const uin
     const uint32_t N = p->total, nt = (N + RTILE - 1) / RTILE;
     const int sms = num_sms();
     const int spans = std::max(1, std::min<int>(nt, sms * 4));
-    uint64_t* status = reinterpret_cast<uint64_t*>(p->status);  // the spans' words, then two words a tile
+    uint64_t* status = reinterpret_cast<uint64_t*>(p->status);  // the spans' words, two words a tile, a word a span
     uint32_t* sums = p->status + 2 * (size_t)spans;
     if ((s = reset_ctrl(p, st, p->status, 2 * spans)) != BWT_OK) return p->last = s;
     const bool few = nt <= FEW_TILES;
     if (!few)
-        k_rle_sums<<<spans, RT, 0, st>>>(d_in, N, p->blocks, p->nb, sums, sums + nt, status,
+        k_rle_sums<<<spans, RT, 0, st>>>(d_in, N, p->blocks, p->nb, sums, sums + nt, sums + 2 * (size_t)nt, status,
                                          p->ctrl + CTRL_TILE_CTR, p->ctrl);
-    k_rle_encode<<<std::max(1, std::min<int>(nt, sms * 48)), RT, 0, st>>>(d_in, N, p->blocks, p->nb, few ? nullptr : sums, sums + nt,
-                                                                       d_chars, d_lens, d_run_off, p->ctrl);
+    const uint32_t per = (nt + (uint32_t)spans - 1) / (uint32_t)spans;  // tiles a span, as the sums' kernel takes them
+    k_rle_encode<<<std::max(1, std::min<int>(nt, sms * 48)), RT, 0, st>>>(
+        d_in, N, p->blocks, p->nb, few ? nullptr : sums, sums + nt, sums + 2 * (size_t)nt, per, d_chars, d_lens, d_run_off,
+        p->ctrl);
     CKS(cudaGetLastError());
     p->stats.kernel_launches = few ? 2 : 3;
     return p->last = finish_status(p, st);
