@@ -38,3 +38,22 @@ def test_learned_batch_with_plain_and_bucketed_blocks(flags):
         st = plan.stats()
         assert st["blocks_routed_plain"] == 1 and st["buckets_overflowed"] >= 1, st
         assert_matches_oracle(buf, off, L.cpu().numpy(), p.cpu().numpy(), "after the timeout")
+
+
+@pytest.mark.parametrize("tile", [0, 1024, 4096])
+def test_inverse(tile):
+    """The inverse's byte sort has a look-back of its own; the walks after it
+    end only on a permutation, so they leave when it has failed. Tiles of 1,024
+    rows (a small batch, or asked for) and of 4,096."""
+    import torch
+    blocks = [datagen.block(datagen.MARKOV3_Z96, 8, 40_001), datagen.block(datagen.UNIFORM, 9, 20_000)]
+    buf, off = batch_from_blocks(blocks)
+    d_in = torch.from_numpy(buf).cuda()
+    out = torch.zeros_like(d_in)
+    with Plan(max_blocks=2, max_total_bytes=buf.size, max_block_bytes=40_001, tile_keys=tile) as plan:
+        L, p = plan.forward(d_in, off)
+        plan.debug_waits(2000, True)
+        assert plan.inverse_into(L, off, p, out, raise_on_error=False) == _lib.BWT_ETIMEOUT
+        plan.debug_waits(0, False)
+        assert plan.inverse_into(L, off, p, out, raise_on_error=False) == _lib.BWT_OK
+    assert torch.equal(out, d_in)
