@@ -271,6 +271,8 @@ bwt_status bwt_plan_set_round_radix(bwt_plan* plan, int radix_bits);
  * the result is appended to that JSON-lines file under (GPU name, workload
  * signature = block count, total bytes, largest block, plan flags) and a
  * later call with the same signature reads it back instead of sweeping.
+ * In a plan created with tile_keys 0, 8 bits and 4,096 keys stand for that
+ * default (1,024-key passes on small batches).
  * Arguments as for bwt_forward_batch; d_L and d_primary receive the output
  * of a final run with the chosen configuration (bwt_plan_stats describes it). */
 bwt_status bwt_plan_autotune(bwt_plan* plan, const uint8_t* d_in, const uint64_t* offsets, uint32_t num_blocks,

@@ -14,6 +14,10 @@
 // The workload signature is the block count, total bytes, largest block and
 // plan flags, so uneven batches of the same shape reuse one entry. A later
 // entry for the same (gpu, key) overrides an earlier one.
+// In a plan whose tile size was left to the library, 8 bits with 4,096-key tiles
+// stand for that default, timed and installed as such: it takes 1,024-key passes
+// on small batches and 4,096-key rounds, which no fixed tile size does (a plan
+// tuned to a fixed 4,096 would also lose the small passes for its other batches).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -93,6 +97,13 @@ extern "C" bwt_status bwt_plan_autotune(bwt_plan* plan, const uint8_t* d_in, con
     const std::string key = ks.str();
     const std::string gpu = gpu_name(plan->device);
 
+    const bool open = plan->desc.tile_keys == 0;
+    auto choose = [&](int b, int t) {
+        const bwt_status r = bwt_plan_set_radix(plan, b, t);
+        if (r == BWT_OK) plan->tile_auto = open && b == 8 && t == 4096;
+        return r;
+    };
+
     if (cache_path && *cache_path) {
         std::ifstream in(cache_path);
         std::string line, best_line;
@@ -104,7 +115,7 @@ extern "C" bwt_status bwt_plan_autotune(bwt_plan* plan, const uint8_t* d_in, con
         if (!best_line.empty() && json_field(best_line, "radix_bits", &rb) && json_field(best_line, "tile_keys", &tk)) {
             const int r = std::atoi(rb.c_str()), t = std::atoi(tk.c_str());
             const int rrb = json_field(best_line, "round_radix_bits", &rr) ? std::atoi(rr.c_str()) : 0;
-            if (bwt_plan_set_radix(plan, r, t) == BWT_OK && bwt_plan_set_round_radix(plan, rrb) == BWT_OK) {
+            if (choose(r, t) == BWT_OK && bwt_plan_set_round_radix(plan, rrb) == BWT_OK) {
                 if (out_radix_bits) *out_radix_bits = r;
                 if (out_tile_keys) *out_tile_keys = t;
                 if (out_ms) *out_ms = json_field(best_line, "ms", &ms) ? (float)std::atof(ms.c_str()) : 0.f;
@@ -129,7 +140,7 @@ extern "C" bwt_status bwt_plan_autotune(bwt_plan* plan, const uint8_t* d_in, con
     };
     for (int b : bits) {
         for (int t : tiles) {
-            if ((status = bwt_plan_set_radix(plan, b, t)) != BWT_OK) {
+            if ((status = choose(b, t)) != BWT_OK) {
                 if (b == 16 && (status == BWT_ENOMEM || status == BWT_EINVAL)) {  // no room for its scratch
                     cudaGetLastError();
                     status = BWT_OK;
@@ -163,7 +174,7 @@ extern "C" bwt_status bwt_plan_autotune(bwt_plan* plan, const uint8_t* d_in, con
     // the doubling rounds' digit width, with the best first-sort choice
     int best_r = 0;
     if (status == BWT_OK) {
-        bwt_plan_set_radix(plan, best_b, best_t);
+        choose(best_b, best_t);
         float best_round = 1e30f;
         for (int rbits : {8, 10, 11}) {
             if ((status = bwt_plan_set_round_radix(plan, rbits)) != BWT_OK) break;
@@ -190,7 +201,7 @@ extern "C" bwt_status bwt_plan_autotune(bwt_plan* plan, const uint8_t* d_in, con
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (status != BWT_OK) return status;
-    bwt_plan_set_radix(plan, best_b, best_t);
+    choose(best_b, best_t);
     bwt_plan_set_round_radix(plan, best_r);
     // one run with the chosen configuration: outputs and statistics are its
     if ((status = bwt_forward_batch(plan, d_in, offsets, num_blocks, d_L, d_primary, stream)) != BWT_OK) return status;
