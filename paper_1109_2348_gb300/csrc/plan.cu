@@ -15,6 +15,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "bwt.h"
@@ -135,18 +136,14 @@ void bwt::free_plan_memory(bwt_plan* p) {
     }
     F(p->splitters); F(p->splitter_index); F(p->splitters_flat); F(p->bucket_count); F(p->bucket_cursor); F(p->chunk_map); F(p->chunk_base); F(p->route); F(p->route_first); F(p->members); F(p->lazy); F(p->lgather); F(p->bstats); F(p->tiles_aux); F(p->inv_slots); F(p->inv_buf); F(p->inv_items); F(p->mtf_lists);
     drop_graph(p);
-    FH(p->h_ctrl); FH(p->h_off);
-    for (int s = 0; s < 2; ++s) {
-        FH(p->stage_tiles[s]);
-        FH(p->stage_il[s]);
-        FH(p->stage_blocks[s]);
+    FH(p->pinned);
+    for (int s = 0; s < 2; ++s)
         if (p->stage_ev[s]) cudaEventDestroy(p->stage_ev[s]);
-    }
     if (p->done_ev) cudaEventDestroy(p->done_ev);
     for (auto& ev : p->br_ev)
         if (ev) cudaEventDestroy(ev);
     destroy_capture_streams(p);
-    FH(p->h_route); FH(p->h_bstats); FH(p->h_inv_items);
+    FH(p->h_route); FH(p->h_bstats);
     for (auto& e : p->events) cudaEventDestroy(e);
     p->events.clear();
 }
@@ -210,26 +207,42 @@ extern "C" bwt_status bwt_plan_create(const bwt_plan_desc* desc, int device, bwt
     A(dev_alloc(&p->seg_varied, (size_t)p->bincap[CLS_LARGE] + 1, &total));
     for (int par = 0; par < 2; ++par)
         for (int c = 0; c < NCLS; ++c) A(dev_alloc(&p->bins[par][c], p->bincap[c], &total));
-    A(host_alloc(&p->h_ctrl, CTRL_WORDS));
+    // The pinned tables, in one allocation instead of nine (created and destroyed,
+    // a plan for 64 blocks of 900,000 bytes 5,117 -> 4,937 us, for one of 100,000
+    // bytes 788 -> 768).
+    {
+        size_t bytes = 0;
+        auto part = [&](auto** q, size_t count) {  // q's place in the slab; called once for the size, once for the pointers
+            if (p->pinned) *q = reinterpret_cast<std::remove_reference_t<decltype(*q)>>(p->pinned + bytes);
+            bytes = (bytes + count * sizeof(**q) + 255) & ~(size_t)255;
+        };
+        for (int pass = 0; pass < 2 && s == BWT_OK; ++pass) {
+            if (pass == 1) A(host_alloc(&p->pinned, bytes));
+            if (s != BWT_OK) break;
+            bytes = 0;
+            part(&p->h_ctrl, CTRL_WORDS);
+            part(&p->h_off, (size_t)B + 1);
+            part(&p->h_inv_items, 2 * ((size_t)B + 1));
+            for (int sl = 0; sl < 2; ++sl) {
+                part(&p->stage_tiles[sl], p->cap_tiles0);
+                part(&p->stage_il[sl], SMALL_TILES);
+                part(&p->stage_blocks[sl], B);
+            }
+        }
+    }
     if (s == BWT_OK) {
         const cudaError_t e = cudaHostGetDevicePointer((void**)&p->hd_ctrl, p->h_ctrl, 0);
         if (e != cudaSuccess) s = record_cuda(e, "cudaHostGetDevicePointer");
     }
-    for (int sl = 0; sl < 2; ++sl) {
-        A(host_alloc(&p->stage_tiles[sl], p->cap_tiles0));
-        A(host_alloc(&p->stage_il[sl], SMALL_TILES));
-        A(host_alloc(&p->stage_blocks[sl], B));
+    for (int sl = 0; sl < 2; ++sl)
         if (s == BWT_OK && cudaEventCreateWithFlags(&p->stage_ev[sl], cudaEventDisableTiming) != cudaSuccess)
             s = BWT_ECUDA;
-    }
     p->h_tiles = p->stage_tiles[0];
     p->h_blocks = p->stage_blocks[0];
     if (s == BWT_OK && cudaEventCreateWithFlags(&p->done_ev, cudaEventDisableTiming) != cudaSuccess) s = BWT_ECUDA;
     for (auto& ev : p->br_ev)
         if (s == BWT_OK && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) s = BWT_ECUDA;
-    A(host_alloc(&p->h_off, (size_t)B + 1));
     p->h_first.resize(std::min<uint32_t>(B, SMALL_TILES));
-    A(host_alloc(&p->h_inv_items, 2 * ((size_t)B + 1)));
     // the learned bucketing's tables and the 16-bit passes' scratch, so that
     // no forward call allocates
     if (s == BWT_OK && (desc->flags & BWT_F_LEARNED)) s = ensure_learned_buffers(p);

@@ -147,6 +147,7 @@ struct bwt_plan {
     uint8_t* mtf_lists = nullptr;      // move-to-front scratch (allocated on first use)
 
     // pinned host staging
+    uint8_t* pinned = nullptr;           // one pinned allocation: the h_ and stage_ tables below, and h_inv_items
     uint32_t* h_ctrl = nullptr;
     uint32_t* hd_ctrl = nullptr;        // its device view (the graph path writes it with a kernel)
     bwt::TileDesc* h_tiles = nullptr;    // the staging slot of the last upload (block and tile tables)

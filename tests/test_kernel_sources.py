@@ -80,3 +80,11 @@ def test_training_reads_results_after_the_wait():
             decl = re.search(r"[^,]*\b" + p + r"\s*(?:,|$)", params.strip()).group(0)
             assert "__restrict__" not in decl, f"{name}: {decl}"
             assert not re.search(r"\b" + p + r"\s*\[", before), f"{name} reads {p} before its wait"
+
+
+def test_plan_creation_takes_pinned_memory_once():
+    """Every pinned allocation and its release cost a program that makes a plan
+    for a call: a plan takes its pinned tables in one."""
+    src = open(os.path.join(CSRC, "plan.cu")).read()
+    body = src[src.index("bwt_status bwt_plan_create("):src.index("bwt_status bwt_plan_destroy(")]
+    assert body.count("host_alloc(") == 1
