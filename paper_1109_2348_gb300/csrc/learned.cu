@@ -843,7 +843,7 @@ __device__ __forceinline__ void sort13(uint64_t (&w)[MS_IT]) {
 // Measured per 240 blocks of 900,000 bytes (nine text-like, one uniform):
 // 3,412 us with (key, index) pairs of 12 bytes moved through every round,
 // 2,657 us with words, 2,611 us with one key offset a chunk instead of one a
-// bucket, 2,738 us since it writes L too (the L gather's 600 us are gone). On 24
+// bucket, 2,738 us since it writes L too (the L gather's 740 us are gone). On 24
 // blocks (ncu): 11.8 -> 9.7 warp instructions a rotation, 80% of the
 // shared-memory pipe, issue 60%, 16.9 DRAM bytes a rotation. Measured
 // and not kept: five CTAs an SM at 48 registers (2,734), the second run of a
@@ -1393,12 +1393,6 @@ bwt_status bwt::ensure_learned_buffers(bwt_plan* p) {
     if (!p->lgather) CKL(cudaMalloc(&p->lgather, sizeof(uint32_t) * ((size_t)(p->cap_n >> LG_WORD_SHIFT) + 2)));
     if (!p->bstats) CKL(cudaMalloc(&p->bstats, sizeof(unsigned long long) * 10 * p->cap_b));
     if (!p->tiles_aux) CKL(cudaMalloc(&p->tiles_aux, sizeof(TileDesc) * 2 * (size_t)p->cap_tiles0));
-    if (!p->splitters_flat) {
-        std::vector<uint64_t> flat(NSP);
-        for (int j = 0; j < NSP; ++j) flat[j] = (uint64_t)(j + 1) << 52;  // bucket = top 12 key bits
-        CKL(cudaMalloc(&p->splitters_flat, sizeof(uint64_t) * NSP));
-        CKL(cudaMemcpy(p->splitters_flat, flat.data(), sizeof(uint64_t) * NSP, cudaMemcpyHostToDevice));
-    }
     if (!p->h_route) {
         CKL(cudaMallocHost(&p->h_route, sizeof(uint32_t) * p->cap_b));
         CKL(cudaHostGetDevicePointer((void**)&p->hd_route, p->h_route, 0));

@@ -134,7 +134,7 @@ void bwt::free_plan_memory(bwt_plan* p) {
         FH(p->stage_parts[sl]);
         FH(p->stage_pfirst[sl]);
     }
-    F(p->splitters); F(p->splitter_index); F(p->splitters_flat); F(p->bucket_count); F(p->bucket_cursor); F(p->chunk_map); F(p->chunk_base); F(p->route); F(p->route_first); F(p->members); F(p->lazy); F(p->lgather); F(p->bstats); F(p->tiles_aux); F(p->inv_slots); F(p->inv_buf); F(p->inv_items); F(p->mtf_lists);
+    F(p->splitters); F(p->splitter_index); F(p->bucket_count); F(p->bucket_cursor); F(p->chunk_map); F(p->chunk_base); F(p->route); F(p->route_first); F(p->members); F(p->lazy); F(p->lgather); F(p->bstats); F(p->tiles_aux); F(p->inv_slots); F(p->inv_buf); F(p->inv_items); F(p->mtf_lists);
     drop_graph(p);
     FH(p->pinned);
     for (int s = 0; s < 2; ++s)
@@ -450,7 +450,7 @@ bwt_status bwt::upload_tables(bwt_plan* p, const uint64_t* off, uint32_t nb, cud
     if (small > 0 && small <= SMALL_TILES) {
         TileDesc* il = p->stage_il[sl];
         uint32_t k = 0, left = nb;
-        for (uint32_t b = 0, first = 0; b < nb; ++b) {  // first tiles, kept in the block's pinned entry below
+        for (uint32_t b = 0, first = 0; b < nb; ++b) {  // every block's first tile
             p->h_first[b] = first;
             first += (uint32_t)((off[b + 1] - off[b] + SMALL_RTILE - 1) / SMALL_RTILE);
         }

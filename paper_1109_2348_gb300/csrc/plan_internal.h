@@ -72,7 +72,9 @@ constexpr size_t kGraphCache = 4;
 }  // namespace bwt
 
 // Small batches (tile size left to the library): tiles of SMALL_RTILE keys while
-// there are at most SMALL_TILES of them, six an SM.
+// there are at most SMALL_TILES of them: just under six an SM of the 152, so that
+// all are in flight at once. (The choice is one of speed; tiles are claimed in
+// order, so a look-back ends however few run.)
 constexpr uint32_t SMALL_RTILE = 1024, SMALL_TILES = 900;
 
 struct bwt_plan {
@@ -107,8 +109,7 @@ struct bwt_plan {
 
     // learned bucketing (allocated when a model is installed)
     uint64_t* splitters = nullptr;      // [BWT_SPLITTERS] sorted
-    uint16_t* splitter_index = nullptr; // [65,544] first splitter of every two-byte key prefix
-    uint64_t* splitters_flat = nullptr; // [BWT_SPLITTERS] equal-width fallback (top 12 key bits)
+    uint16_t* splitter_index = nullptr; // [IDX_WORDS] first splitter of every 15-bit key prefix
     uint32_t* bucket_count = nullptr;   // [2][block][BWT_BUCKETS] counts (learned, equal-width), then starts
     uint32_t* bucket_cursor = nullptr;  // [block][BWT_BUCKETS] slots taken so far (per chunk)
     uint16_t* chunk_map = nullptr;      // [block][BWT_BUCKETS] chunk of each bucket
@@ -253,7 +254,7 @@ void learned_stats(bwt_plan* p);
 bwt_status load_model(bwt_plan* p, const char* path);
 void graph_stats(bwt_plan* p);
 bwt_status ensure_learned_buffers(bwt_plan* p);
-// The two-byte-prefix index of the installed splitter table (synchronous).
+// The 15-bit-prefix index of the installed splitter table (synchronous).
 bwt_status build_splitter_index(bwt_plan* p);
 // Scratch of the 16-bit digit passes (a no-op once allocated).
 bwt_status ensure_radix16(bwt_plan* p);
